@@ -19,7 +19,9 @@
 //   x-inverse, y-inverse.  A spatial pass is an FFT (k_fft.cu) when the axis
 //   length is a power of two from 8 to 512, otherwise a small dense matrix
 //   applied along the axis (a SIMT GEMM with the transform matrix on the
-//   left); the time pass keeps a strip of all N_t planes in shared memory.
+//   left); the time pass is a tridiagonal elimination per spatial mode, or the
+//   two dense products on the tensor cores (k_time_tc.cu).
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
@@ -102,6 +104,7 @@ int build_prec_tables(const mfg_problem& p, const Geom& g, PrecTables* t, std::s
   t->nx = g.nx;
   t->ny = g.ny;
   t->nt = g.nt;
+  t->l = p.l;
   std::vector<double> Hx, lx, Hy, ly, V, lt;
   axis_basis(g.nx, g.perx, Hx, lx);
   axis_basis(g.ny, g.pery, Hy, ly);
@@ -314,222 +317,127 @@ static void axis_pass(const TI* in, TO* out, const T* M, int N, long long inner,
     k_axis<TI, T, TO, false><<<grid, 256, 0, s>>>(in, out, M, N, inner, ncols, trans, sc);
 }
 
-// ------------------------------------------------------ fused time pass --
-// For a strip of TSW spatial modes: Y = V X (time forward), Y /= S(k, s),
-// out = V^T Y (time inverse).  One strip buffer (N_t x TSW) is reused for X
-// and then Y; V is streamed through shared memory in 16-column chunks.
-constexpr int TSW = 32, TCH = 16, TU = kMaxNt / 8;
+// ------------------------------------------------------------ time pass --
+// Time forward, division by S(k, s) and time inverse of Alg. 1 in one
+// elimination.  V diagonalises the second difference D of Sec. 4.1 (tridiagonal
+// -1, 2, -1, first diagonal entry l), so per spatial mode s
+//   V^T diag_k(1 / (Lambda_1 + lambda_k Lambda_2)) V = (Lambda_1 I + Lambda_2 D)^{-1},
+// a symmetric positive definite tridiagonal system: O(N_t) operations per mode
+// where the two dense products take O(N_t^2).  With rho = Lambda_1 / Lambda_2 >= 0
+// the pivots of the elimination are 1 + delta_k,
+//   delta_0 = l - 1 + rho,  delta_k = rho + delta_{k-1} / (1 + delta_{k-1}),
+// sums and quotients of non-negative numbers only, so neither a small rho (the
+// low modes) nor a large one loses digits; g_k = 1 / (1 + delta_k),
+//   e_k = b_k + g_{k-1} e_{k-1},   x_k = g_k (e_k / Lambda_2 + x_{k+1}).
+//
+// One thread per mode.  The pass is bound by memory (one read and one write of
+// the data) in FP32 and by ~9 FP64 instructions per element in FP64, if enough
+// bytes are in flight: a thread issues its whole column of N_t loads as
+// cp.async into its own column of shared memory, forms the g_k (which need no
+// data) while they land, and then runs the two recurrences in place.  No
+// thread reads another's column, so nothing synchronises.  512^2 x 128 FP32:
+// 169 us (dense products on the tensor cores) -> 64 us, with a tenth of the
+// apply's error (3e-6 -> 3e-7 against 64 bits); 256^2 x 64 FP64: 973 us (dense
+// products on the CUDA cores) -> ~105 us.
+template <typename T>
+__device__ __forceinline__ void cp_async_elem(T* smem, const T* gmem) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(sa), "l"(gmem), "n"((int)sizeof(T)) : "memory");
+}
+
+// 1/x to one unit in the last place
+__device__ __forceinline__ float recip(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+// 1/x for x >= 1: the hardware's approximation (relative error below 2^-20)
+// and one third-order (Halley) step, y (1 + e + e^2) with e = 1 - x y.  Past
+// 2^1000 the pivot's reciprocal is taken as 0 (nothing is coupled there).
+__device__ __forceinline__ double recip(double x) {
+  if (!(x < 1.0715086071862673e301)) return x != x ? x : 0.0;
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
 
 template <typename T>
-__global__ void __launch_bounds__(256) k_time(const T* __restrict__ in, T* __restrict__ out,
-                                              const T* __restrict__ V, const T* __restrict__ lamt,
-                                              const T* __restrict__ L1, const T* __restrict__ L2,
-                                              int nt, int S, const DevScalars* sc) {
+__global__ void __launch_bounds__(128) k_time_tri(const T* __restrict__ in, T* __restrict__ out,
+                                                  const T* __restrict__ L1, const T* __restrict__ L2, int l,
+                                                  int nt, int S, const DevScalars* sc) {
   if (sc != nullptr && sc->cg_done) return;
-  extern __shared__ unsigned char smem_raw[];
-  T* X = reinterpret_cast<T*>(smem_raw);   // [nt][TSW]
-  T* Vs = X + (size_t)nt * TSW;            // [nt][TCH]
-  const int tid = threadIdx.x, c = tid % TSW, r0 = tid / TSW;
-  const int s0 = blockIdx.x * TSW;
-  const int sc_ = s0 + c;
-  for (int q = tid; q < nt * TSW; q += 256) {
-    const int k = q / TSW, cc = q % TSW;
-    X[q] = (s0 + cc < S) ? in[(long long)k * S + s0 + cc] : T(0);
-  }
-  const int nu_ = (nt + 7) / 8;
-  T acc[TU];
-#pragma unroll
-  for (int u = 0; u < TU; ++u) acc[u] = T(0);
-  // Y = V X
-  for (int b0 = 0; b0 < nt; b0 += TCH) {
-    __syncthreads();
-    for (int q = tid; q < nt * TCH; q += 256) {
-      const int a = q / TCH, bb = q % TCH;
-      Vs[q] = (b0 + bb < nt) ? V[(long long)a * nt + b0 + bb] : T(0);
-    }
-    __syncthreads();
-    const int bmax = min(TCH, nt - b0);
-    for (int bb = 0; bb < bmax; ++bb) {
-      const T xb = X[(b0 + bb) * TSW + c];
-#pragma unroll
-      for (int u = 0; u < TU; ++u)
-        if (u < nu_) {
-          const int a = r0 + 8 * u;
-          if (a < nt) acc[u] = fma(Vs[a * TCH + bb], xb, acc[u]);
-        }
-    }
-  }
-  __syncthreads();
-  // divide by S(k, s) = Lambda_1(s) + lambda_k Lambda_2(s); overwrite X with Y
-  const T l1 = sc_ < S ? L1[sc_] : T(1), l2 = sc_ < S ? L2[sc_] : T(0);
-#pragma unroll
-  for (int u = 0; u < TU; ++u)
-    if (u < nu_) {
-      const int a = r0 + 8 * u;
-      if (a < nt) X[a * TSW + c] = acc[u] / (l1 + lamt[a] * l2);
-      acc[u] = T(0);
-    }
-  // out = V^T Y
-  for (int b0 = 0; b0 < nt; b0 += TCH) {
-    __syncthreads();
-    for (int q = tid; q < nt * TCH; q += 256) {
-      const int a = q / TCH, bb = q % TCH;
-      Vs[q] = (b0 + bb < nt) ? V[(long long)(b0 + bb) * nt + a] : T(0);
-    }
-    __syncthreads();
-    const int bmax = min(TCH, nt - b0);
-    for (int bb = 0; bb < bmax; ++bb) {
-      const T yb = X[(b0 + bb) * TSW + c];
-#pragma unroll
-      for (int u = 0; u < TU; ++u)
-        if (u < nu_) {
-          const int a = r0 + 8 * u;
-          if (a < nt) acc[u] = fma(Vs[a * TCH + bb], yb, acc[u]);
-        }
-    }
-  }
-  if (sc_ < S) {
-#pragma unroll
-    for (int u = 0; u < TU; ++u)
-      if (u < nu_) {
-        const int a = r0 + 8 * u;
-        if (a < nt) out[(long long)a * S + sc_] = acc[u];
-      }
-  }
-}
-
-// Fixed-N_t time pass: the whole (symmetric, orthonormal) time matrix V sits in
-// shared memory next to an N_t x TW strip; each thread owns an RM x RN register
-// tile, so one pass over b costs RM + RN shared loads for RM * RN FMAs.  Both
-// DCT-VIII and DST-I are symmetric (V = V^T, checked on the host), so rows of V
-// serve the forward and the inverse product.
-template <typename T, int NT>
-struct TimeShape {
-  static constexpr int TW = 32;                           // strip width (spatial modes)
-  static constexpr int RN = 2;                            // columns per thread
-  static constexpr int CG = TW / RN;                      // column groups
-  static constexpr int RG = 256 / CG;                     // row groups
-  static constexpr int RM = NT / RG;                      // rows per thread
-  static constexpr size_t smem = sizeof(T) * ((size_t)NT * NT + (size_t)NT * TW);
-};
-
-// K consecutive shared-memory values with the widest aligned vector loads.
-template <int K>
-__device__ __forceinline__ void lds_vec(const float* p, float (&o)[K]) {
-  if constexpr (K % 4 == 0) {
-#pragma unroll
-    for (int q = 0; q < K; q += 4) {
-      const float4 v = *reinterpret_cast<const float4*>(p + q);
-      o[q] = v.x; o[q + 1] = v.y; o[q + 2] = v.z; o[q + 3] = v.w;
-    }
-  } else {
-#pragma unroll
-    for (int q = 0; q < K; ++q) o[q] = p[q];
-  }
-}
-template <int K>
-__device__ __forceinline__ void lds_vec(const double* p, double (&o)[K]) {
-  if constexpr (K % 2 == 0) {
-#pragma unroll
-    for (int q = 0; q < K; q += 2) {
-      const double2 v = *reinterpret_cast<const double2*>(p + q);
-      o[q] = v.x; o[q + 1] = v.y;
-    }
-  } else {
-#pragma unroll
-    for (int q = 0; q < K; ++q) o[q] = p[q];
-  }
-}
-
-template <typename T, int NT>
-__global__ void __launch_bounds__(256) k_time_fast(const T* __restrict__ in, T* __restrict__ out,
-                                                   const T* __restrict__ V, const T* __restrict__ lamt,
-                                                   const T* __restrict__ L1, const T* __restrict__ L2,
-                                                   int S, const DevScalars* sc) {
-  if (sc != nullptr && sc->cg_done) return;
-  using Sh = TimeShape<T, NT>;
-  constexpr int TW = Sh::TW, RN = Sh::RN, CG = Sh::CG, RM = Sh::RM;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* Vs = reinterpret_cast<T*>(smem_raw);  // [NT][NT], loaded once per block
-  T* X = Vs + NT * NT;                      // [NT][TW]
-  const int tid = threadIdx.x;
-  const int cg = tid % CG, rg = tid / CG;
-  const int r0 = rg * RM;  // this thread's rows r0 .. r0 + RM - 1
-  for (int q = tid; q < NT * NT; q += 256) Vs[q] = V[q];
-  T lam[RM];
-#pragma unroll
-  for (int u = 0; u < RM; ++u) lam[u] = lamt[r0 + u];
-  const int nstrips = (S + TW - 1) / TW;
-  // the block walks strips of TW spatial modes, reusing V from shared memory
-  for (int strip = blockIdx.x; strip < nstrips; strip += gridDim.x) {
-    const int s0 = strip * TW;
-    __syncthreads();  // previous strip done with X (and V loaded on the first pass)
-    for (int q = tid; q < NT * TW; q += 256) {
-      const int k = q / TW, c = q % TW;
-      X[q] = (s0 + c < S) ? in[(long long)k * S + s0 + c] : T(0);
-    }
-    __syncthreads();
-    T acc[RM][RN];
-#pragma unroll
-    for (int u = 0; u < RM; ++u)
-#pragma unroll
-      for (int v = 0; v < RN; ++v) acc[u][v] = T(0);
-    // Y = V X: row r uses V[r][b] = V[b][r] (symmetric V), contiguous in r
+  const int bd = blockDim.x, s = blockIdx.x * bd + threadIdx.x;
+  T* E = reinterpret_cast<T*>(smem_raw) + threadIdx.x;  // [nt][bd], this thread's column
+  T* G = E + (size_t)nt * bd;
+  if (s >= S) return;
+  const T* src = in + s;
+#pragma unroll 8
+  for (int k = 0; k < nt; ++k) cp_async_elem(E + k * bd, src + (long long)k * S);
+  asm volatile("cp.async.commit_group;\n" ::: "memory");
+  const T l2 = L2[s], rho = L1[s] / l2, il2 = T(1) / l2;
+  T d = T(l - 1) + rho, g = recip(T(1) + d);
+  G[0] = g;
 #pragma unroll 4
-    for (int b = 0; b < NT; ++b) {
-      T xv[RN], vv[RM];
-      lds_vec<RN>(X + b * TW + cg * RN, xv);
-      lds_vec<RM>(Vs + b * NT + r0, vv);
+  for (int k = 1; k < nt; ++k) {
+    d = fma(d, g, rho);
+    g = recip(T(1) + d);
+    G[k * bd] = g;
+  }
+  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  // eight steps at a time: their shared loads are issued together, ahead of
+  // the chain and of the stores they cannot be moved across
+  T e = T(0);
+  g = T(0);
+  int k = 0;
+  for (; k + 8 <= nt; k += 8) {
+    T ev[8], gv[8];
 #pragma unroll
-      for (int u = 0; u < RM; ++u)
+    for (int u = 0; u < 8; ++u) { ev[u] = E[(k + u) * bd]; gv[u] = G[(k + u) * bd]; }
 #pragma unroll
-        for (int v = 0; v < RN; ++v) acc[u][v] = fma(vv[u], xv[v], acc[u][v]);
-    }
-    __syncthreads();
-    // divide by S(k, s) = Lambda_1(s) + lambda_k Lambda_2(s); Y overwrites X
+    for (int u = 0; u < 8; ++u) { e = fma(u ? gv[u - 1] : g, e, ev[u]); ev[u] = e; }
+    g = gv[7];
 #pragma unroll
-    for (int v = 0; v < RN; ++v) {
-      const int c = cg * RN + v;
-      const int s = s0 + c;
-      const T l1 = s < S ? L1[s] : T(1), l2 = s < S ? L2[s] : T(0);
+    for (int u = 0; u < 8; ++u) E[(k + u) * bd] = ev[u];
+  }
+  for (; k < nt; ++k) {
+    e = fma(g, e, E[k * bd]);
+    E[k * bd] = e;
+    g = G[k * bd];
+  }
+  T* dst = out + s;
+  T x = T(0);
+  for (k = nt; k % 8 != 0; --k) {
+    x = G[(k - 1) * bd] * fma(E[(k - 1) * bd], il2, x);
+    dst[(long long)(k - 1) * S] = x;
+  }
+  for (; k > 0; k -= 8) {
+    T ev[8], gv[8];
 #pragma unroll
-      for (int u = 0; u < RM; ++u) {
-        X[(r0 + u) * TW + c] = acc[u][v] / (l1 + lam[u] * l2);
-        acc[u][v] = T(0);
-      }
-    }
-    __syncthreads();
-    // out = V^T Y: out[a][c] = sum_b V[b][a] Y[b][c]
-#pragma unroll 4
-    for (int b = 0; b < NT; ++b) {
-      T yv[RN], vv[RM];
-      lds_vec<RN>(X + b * TW + cg * RN, yv);
-      lds_vec<RM>(Vs + b * NT + r0, vv);
+    for (int u = 0; u < 8; ++u) { ev[u] = E[(k - 1 - u) * bd]; gv[u] = G[(k - 1 - u) * bd]; }
 #pragma unroll
-      for (int u = 0; u < RM; ++u)
-#pragma unroll
-        for (int v = 0; v < RN; ++v) acc[u][v] = fma(vv[u], yv[v], acc[u][v]);
-    }
-#pragma unroll
-    for (int u = 0; u < RM; ++u) {
-      const int r = r0 + u;
-#pragma unroll
-      for (int v = 0; v < RN; ++v) {
-        const int s = s0 + cg * RN + v;
-        if (s < S) out[(long long)r * S + s] = acc[u][v];
-      }
+    for (int u = 0; u < 8; ++u) {
+      x = gv[u] * fma(ev[u], il2, x);
+      dst[(long long)(k - 1 - u) * S] = x;
     }
   }
 }
 
-template <typename T, int NT>
-static void launch_time_fast(const T* in, T* out, const T* V, const T* lamt, const T* L1, const T* L2,
-                             int S, const DevScalars* sc, cudaStream_t s) {
-  using Sh = TimeShape<T, NT>;
-  // enough blocks to fill the GPU (several resident per SM); each walks strips
-  const int nstrips = (S + Sh::TW - 1) / Sh::TW;
-  const int blocks = nstrips < 152 * 4 ? nstrips : 152 * 4;
-  k_time_fast<T, NT><<<blocks, 256, Sh::smem, s>>>(in, out, V, lamt, L1, L2, S, sc);
+// Threads per block: 128, 64 or 32, the largest whose two columns per thread
+// fit in 64 KB (three blocks per SM) and whose grid still has a block per SM.
+template <typename T>
+static int tri_threads(int nt, int S) {
+  int bd = 128;
+  while (bd > 32 && (2 * sizeof(T) * (size_t)nt * bd > 65536 || (S + bd - 1) / bd < 152)) bd >>= 1;
+  return bd;
+}
+
+template <typename T>
+static void time_pass(const T* in, T* out, const T* L1, const T* L2, int l, int nt, int S, const DevScalars* sc,
+                      cudaStream_t s) {
+  const int bd = tri_threads<T>(nt, S);
+  k_time_tri<T><<<(S + bd - 1) / bd, bd, 2 * sizeof(T) * (size_t)nt * bd, s>>>(in, out, L1, L2, l, nt, S, sc);
 }
 
 // Exact time solve of the l = 0 variant: per spatial mode s, the tridiagonal
@@ -562,22 +470,9 @@ __global__ void __launch_bounds__(256) k_thomas(const T* __restrict__ in, T* __r
 }
 
 template <typename T>
-static size_t time_smem(int nt) { return sizeof(T) * (size_t)nt * (TSW + TCH); }
-
-template <typename T>
-static void time_pass(const T* in, T* out, const T* V, const T* lamt, const T* L1, const T* L2,
-                      int nt, int S, const DevScalars* sc, cudaStream_t s) {
-  if (nt == 32) return launch_time_fast<T, 32>(in, out, V, lamt, L1, L2, S, sc, s);
-  if (nt == 64) return launch_time_fast<T, 64>(in, out, V, lamt, L1, L2, S, sc, s);
-  if (nt == 128) return launch_time_fast<T, 128>(in, out, V, lamt, L1, L2, S, sc, s);
-  const size_t sm = time_smem<T>(nt);
-  k_time<T><<<(S + TSW - 1) / TSW, 256, sm, s>>>(in, out, V, lamt, L1, L2, nt, S, sc);
-}
-
-template <typename T>
 static void precond_typed(const Geom& g, const T* Hx, const T* Hy, const T* V, const T* lamt,
                           const T* L1, const T* L2, const T* twx, const T* dctx, const T* twy,
-                          const T* dcty, const T* thc, const T* thd, const T* tho,
+                          const T* dcty, const T* thc, const T* thd, const T* tho, int l,
                           const double* r, double* z, T* w0, T* w1,
                           const DevScalars* sc, cudaStream_t s, const PcgDot* dot,
                           const PcgZr* zr, bool tc = false) {
@@ -606,9 +501,9 @@ static void precond_typed(const Geom& g, const T* Hx, const T* Hy, const T* V, c
     if (tc && !g.time_simt && time_tc_supported(g.nt))
       launch_time_tc(a, b, V, lamt, L1, L2, g.nt, (int)S, sc, s);
     else
-      time_pass<T>(a, b, V, lamt, L1, L2, g.nt, (int)S, sc, s);
+      time_pass<T>(a, b, L1, L2, l, g.nt, (int)S, sc, s);
   } else {
-    time_pass<T>(a, b, V, lamt, L1, L2, g.nt, (int)S, sc, s);
+    time_pass<T>(a, b, L1, L2, l, g.nt, (int)S, sc, s);
   }
   { T* t = a; a = b; b = t; }
   if (g.nx > 1) {
@@ -637,11 +532,11 @@ void launch_precond(const Geom& g, const PrecTables& t, int precision, const dou
   }
   if (precision == MFG_MIXED || precision == MFG_MIXED_DF || precision == MFG_MIXED_TC)
     precond_typed<float>(g, t.Hx32, t.Hy32, t.Vt32, t.lamt32, t.L1_32, t.L2_32, t.twx32, t.dctx32,
-                         t.twy32, t.dcty32, t.thc32, t.thd32, t.tho32, r, z, work32, work32 + g.n,
+                         t.twy32, t.dcty32, t.thc32, t.thd32, t.tho32, t.l, r, z, work32, work32 + g.n,
                          sc, s, dot, zr, precision == MFG_MIXED_TC);
   else
     precond_typed<double>(g, t.Hx64, t.Hy64, t.Vt64, t.lamt64, t.L1_64, t.L2_64, t.twx64, t.dctx64,
-                          t.twy64, t.dcty64, t.thc64, t.thd64, t.tho64, r, z, work64, work64 + g.n,
+                          t.twy64, t.dcty64, t.thc64, t.thd64, t.tho64, t.l, r, z, work64, work64 + g.n,
                           sc, s, dot, zr);
 }
 
@@ -657,17 +552,12 @@ int precond_step_kernel_count(const Geom& g, const PrecTables& t) {
 // Opt-in shared memory for the time pass; called once per device before any
 // launch or stream capture.
 int precond_configure() {
-  cudaError_t e1 = cudaFuncSetAttribute(k_time<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)time_smem<double>(kMaxNt));
-  cudaError_t e2 = cudaFuncSetAttribute(k_time<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)time_smem<float>(kMaxNt));
-  int bad = (e1 != cudaSuccess) || (e2 != cudaSuccess);
-#define MFG_TF_ATTR(T, NT)                                                                    \
-  bad |= cudaFuncSetAttribute(k_time_fast<T, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                              (int)TimeShape<T, NT>::smem) != cudaSuccess;
-  MFG_TF_ATTR(float, 32) MFG_TF_ATTR(float, 64) MFG_TF_ATTR(float, 128)
-  MFG_TF_ATTR(double, 32) MFG_TF_ATTR(double, 64) MFG_TF_ATTR(double, 128)
-#undef MFG_TF_ATTR
+  // one warp's columns of the longest time axis
+  const int tri = 2 * kMaxNt * 32;
+  int bad = cudaFuncSetAttribute(k_time_tri<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 std::max(65536, tri * (int)sizeof(double))) != cudaSuccess;
+  bad |= cudaFuncSetAttribute(k_time_tri<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              std::max(65536, tri * (int)sizeof(float))) != cudaSuccess;
   bad |= fft_configure() != MFG_OK;
   bad |= band_configure() != MFG_OK;
   bad |= prox_configure() != MFG_OK;

@@ -37,7 +37,7 @@ struct Geom {
   // operator a kernel applies.
   int vec_blocks;   // grid cap of the vector and reduction kernels
   int aat_want;     // target block count of the AAt stencil launch
-  int time_simt;    // 1: time pass on the CUDA cores even where the tensor-core pass applies
+  int time_simt;    // 1: time pass by elimination on the CUDA cores even where the tensor-core pass applies
   int fft_x, fft_y; // 1: FFT spatial pass where the axis length allows it; 0: dense pass
   // Viscosity field (mfg_problem::nu_field): per node, the coefficient of its
   // "plus" face on each axis, nu_face * ax (kfx) and nu_face * ay (kfy), face i
@@ -119,6 +119,7 @@ void launch_scalars_begin(DevScalars* sc, cudaGraphConditionalHandle h, int use_
 // Preconditioner (k_precond.cu).  Tables are per instance, FP64 and FP32.
 struct PrecTables {
   int nx, ny, nt;
+  int l = 1;  // time preconditioner (mfg_problem::l)
   double *Hx64, *Hy64, *Vt64, *lamt64, *L1_64, *L2_64;  // device, FP64
   float *Hx32, *Hy32, *Vt32, *lamt32, *L1_32, *L2_32;   // device, FP32
   // FFT twiddles for power-of-two axes (null otherwise): tw (N/2 complex),

@@ -131,7 +131,7 @@ __global__ void k_noalloc_tables(Geom g, int l, T* Hx, T* Hy, T* V, T* lamt, T* 
 }
 
 template <typename T>
-void carve(double* base, const Geom& g, PrecTables* t, T** w0) {
+void carve(double* base, const Geom& g, int l, PrecTables* t, T** w0) {
   T* p = reinterpret_cast<T*>(base);
   *w0 = p;
   p += kNaWork;
@@ -154,6 +154,7 @@ void carve(double* base, const Geom& g, PrecTables* t, T** w0) {
     t->twx32 = twx; t->dctx32 = dctx; t->twy32 = twy; t->dcty32 = dcty;
   }
   t->nx = g.nx; t->ny = g.ny; t->nt = g.nt;
+  t->l = l;
 }
 
 }  // namespace
@@ -204,13 +205,13 @@ extern "C" int mfg_apply_precond_noalloc(const mfg_problem* p, const double* r, 
     // plan, MFG_MIXED_DF (which differs from MFG_MIXED only in the AAt stencil)
     // runs as MFG_MIXED
     float* w0 = nullptr;
-    carve<float>(base, g, &t, &w0);
+    carve<float>(base, g, p->l, &t, &w0);
     k_noalloc_tables<float><<<nb, kThreads, 0, s>>>(g, p->l, t.Hx32, t.Hy32, t.Vt32, t.lamt32, t.L1_32, t.L2_32,
                                                      t.twx32, t.dctx32, t.twy32, t.dcty32);
     launch_precond(g, t, p->precision == MFG_MIXED_TC ? MFG_MIXED_TC : MFG_MIXED, r, z, nullptr, w0, nullptr, s);
   } else {
     double* w0 = nullptr;
-    carve<double>(base, g, &t, &w0);
+    carve<double>(base, g, p->l, &t, &w0);
     k_noalloc_tables<double><<<nb, kThreads, 0, s>>>(g, p->l, t.Hx64, t.Hy64, t.Vt64, t.lamt64, t.L1_64,
                                                       t.L2_64, t.twx64, t.dctx64, t.twy64, t.dcty64);
     launch_precond(g, t, MFG_FP64, r, z, w0, nullptr, nullptr, s);
