@@ -14,6 +14,7 @@
 #include <cstdint>
 
 #include "mfg_internal.cuh"
+#include "pcg_tail.cuh"
 #include "reduce.cuh"
 
 namespace mfg {
@@ -110,26 +111,7 @@ __global__ void __launch_bounds__(kThreads) k_update_zr(long long n, double* __r
     r[e] = rv;
     acc = fma(rv, rv, acc);
   }, vec)
-  double part[1] = {acc};
-  block_sum<1>(part);
-  if (!publish_and_check_last<1>(part, partials, &sc->counter)) return;
-  double tot[1];
-  gather_partials<1>(partials, tot);
-  if (flat_tid() == 0) {
-    sc->rr = tot[0];
-    sc->cg_it += 1;
-    const double tol = sc->cg_tol;
-    if (!isfinite(tot[0])) {
-      sc->cg_done = 1;
-      if (sc->status == MFG_OK) sc->status = MFG_ERR_NONFINITE;
-    } else if (tot[0] <= tol * tol * sc->bnorm2) {
-      sc->cg_done = 1;
-    } else if (sc->cg_it >= sc->max_cg) {
-      sc->cg_done = 1;
-      if (sc->status == MFG_OK) sc->status = MFG_ERR_NOT_CONVERGED;
-    }
-    sc->counter = 0;
-  }
+  zr_tail(acc, partials, sc);
 }
 
 // rz_new = r.zp (and qz = q.zp for the flexible variant); beta; rz = rz_new.
@@ -156,22 +138,7 @@ __global__ void __launch_bounds__(kThreads) k_dot_beta(long long n, const double
     a0 = fma(r[e], zv, a0);
     if (FLEX) a1 = fma(q[e], zv, a1);
   }, vec)
-  double part[2] = {a0, a1};
-  block_sum<2>(part);
-  if (!publish_and_check_last<2>(part, partials, &sc->counter)) return;
-  double tot[2];
-  gather_partials<2>(partials, tot);
-  if (flat_tid() == 0) {
-    const double rz_old = sc->rz;
-    sc->qz = tot[1];
-    sc->beta = FLEX ? (-sc->alpha * tot[1] / rz_old) : (tot[0] / rz_old);
-    sc->rz = tot[0];
-    if (!isfinite(sc->beta) || !(tot[0] > 0.0)) {
-      sc->cg_done = 1;
-      if (sc->status == MFG_OK) sc->status = MFG_ERR_NONFINITE;
-    }
-    sc->counter = 0;
-  }
+  dot_tail(a0, a1, FLEX, partials, sc);
 }
 
 // p = zp + beta p; ends the CG body: keeps the while-node running until done.

@@ -1,5 +1,6 @@
 // Spatial passes of the preconditioner by FFT, for axis lengths that are powers
-// of two (Alg. 2: transform along y, then x, divide, invert).
+// of two up to 512 (Alg. 2: transform along y, then x, divide, invert; other
+// lengths in k_fft_mixed.cu).
 //
 // One block takes LB real lines of length N (rows of the contiguous y axis, or
 // columns of the x axis), packs them pairwise into CL = LB/2 complex lines
@@ -17,16 +18,11 @@
 // The result equals the dense orthonormal transform of the plan's tables to
 // round-off; the pass reads and writes each element once.
 #include "mfg_internal.cuh"
+#include "fft_common.cuh"
+#include "pcg_tail.cuh"
 #include "reduce.cuh"
 
 namespace mfg {
-
-template <typename T>
-struct __align__(2 * sizeof(T)) cx {
-  T x, y;
-};
-
-enum { FFT_DHT = 0, FFT_DCT2 = 1, FFT_DCT3 = 2 };
 
 // Lines of N >= 256 take radix-8 Stockham stages (N/8 >= 32 butterflies
 // keep every lane of the warp busy), shorter lines radix-4 stages.
@@ -57,29 +53,6 @@ struct FftShape {
   static constexpr int LB = 2 * CL;                                 // real lines per block
   static constexpr int NP = N + 1;  // padded line stride: staging across lines hits distinct banks
   static constexpr size_t smem = 2 * (size_t)CL * NP * sizeof(cx<T>) + (size_t)(N / 2 + N) * sizeof(cx<T>);
-};
-
-// Dot products fused into the last pass of a PCG preconditioner apply: while
-// zp = P^{-1} r is stored, r.zp (and q.zp for the flexible variant) are
-// accumulated and the last block forms beta exactly as k_dot_beta does.
-struct DotFuse {
-  const double* r;
-  const double* q;
-  double* partials;
-  DevScalars* sc;
-  int flex;
-};
-
-// The PCG update fused into the first pass: z += alpha p, r -= alpha q for the
-// elements this block transforms, ||r||^2 accumulated, and the last block runs
-// the convergence test of k_update_zr.  The pass then transforms the new r.
-struct ZrFuse {
-  double* z;
-  double* r;
-  const double* p;
-  const double* q;
-  double* partials;
-  DevScalars* sc;
 };
 
 // tw[m] = (cos 2 pi m/N, sin 2 pi m/N), m < N/2;  dct[k] = (cos pi k/(2N), sin pi k/(2N)).
@@ -381,59 +354,15 @@ __global__ void __launch_bounds__(256) k_fft(const TI* __restrict__ in, TO* __re
       }
     }
   }
-  if constexpr (ZR) {
-    double part[1] = {rr};
-    block_sum<1>(part);
-    if (!publish_and_check_last<1>(part, zf.partials, &zf.sc->counter)) return;
-    double tot[1];
-    gather_partials<1>(zf.partials, tot);
-    if (flat_tid() == 0) {
-      DevScalars* s = zf.sc;
-      s->rr = tot[0];
-      s->cg_it += 1;
-      const double tol = s->cg_tol;
-      if (!isfinite(tot[0])) {
-        s->cg_done = 1;
-        if (s->status == MFG_OK) s->status = MFG_ERR_NONFINITE;
-      } else if (tot[0] <= tol * tol * s->bnorm2) {
-        s->cg_done = 1;
-      } else if (s->cg_it >= s->max_cg) {
-        s->cg_done = 1;
-        if (s->status == MFG_OK) s->status = MFG_ERR_NOT_CONVERGED;
-      }
-      s->counter = 0;
-    }
-  }
-  if constexpr (DOT) {
-    double part[2] = {a0, a1};
-    block_sum<2>(part);
-    if (!publish_and_check_last<2>(part, df.partials, &df.sc->counter)) return;
-    double tot[2];
-    gather_partials<2>(df.partials, tot);
-    if (flat_tid() == 0) {
-      DevScalars* s = df.sc;
-      const double rz_old = s->rz;
-      s->qz = tot[1];
-      s->beta = df.flex ? (-s->alpha * tot[1] / rz_old) : (tot[0] / rz_old);
-      s->rz = tot[0];
-      if (!isfinite(s->beta) || !(tot[0] > 0.0)) {
-        s->cg_done = 1;
-        if (s->status == MFG_OK) s->status = MFG_ERR_NONFINITE;
-      }
-      s->counter = 0;
-    }
-  }
+  if constexpr (ZR) zr_tail(rr, zf.partials, zf.sc);
+  if constexpr (DOT) dot_tail(a0, a1, df.flex, df.partials, df.sc);
 }
 
-bool fft_supported(int N) { return N >= 8 && N <= 512 && (N & (N - 1)) == 0; }
+bool fft_pow2(int N) { return N >= 8 && N <= 512 && (N & (N - 1)) == 0; }
+bool fft_supported(int N) { return fft_pow2(N) || fft_mixed_supported(N); }
 
-// Partial-sum slots the fused-dot y pass needs (2 per block).
-long long fft_dot_partials(const Geom& g) {
-  const long long lb = FftShape<float, 8>::LB;  // lines per block (same for every N and type)
-  static_assert(FftShape<float, 8>::LB == FftShape<double, 512>::LB, "uniform lines per block");
-  const long long nlines = g.n / g.ny;
-  return 2 * ((nlines + lb - 1) / lb);
-}
+// Partial-sum slots the fused-dot y pass needs (2 per block of at least 2 lines).
+long long fft_dot_partials(const Geom& g) { return 2 * ((g.n / g.ny + 1) / 2); }
 
 template <typename T, int N, int MODE, bool CONTIG, typename TI, typename TO, bool DOT = false,
           bool ZR = false>
@@ -483,6 +412,7 @@ static void dispatch(int N, const TI* in, TO* out, const T* tw, const T* dct, lo
 template <typename T>
 void fft_y_forward(int N, int periodic, const double* in, T* out, const T* tw, const T* dct,
                    long long nlines, const DevScalars* sc, cudaStream_t s, const PcgZr* zr) {
+  if (!fft_pow2(N)) return fft_mixed_y_forward<T>(N, periodic, in, out, tw, dct, nlines, sc, s, zr);
   if (zr) {
     ZrFuse zf{zr->z, zr->r, zr->p, zr->q, zr->partials, zr->sc};
     if (periodic)
@@ -501,6 +431,7 @@ void fft_y_forward(int N, int periodic, const double* in, T* out, const T* tw, c
 template <typename T>
 void fft_y_inverse(int N, int periodic, const T* in, double* out, const T* tw, const T* dct,
                    long long nlines, const DevScalars* sc, cudaStream_t s, const PcgDot* dot) {
+  if (!fft_pow2(N)) return fft_mixed_y_inverse<T>(N, periodic, in, out, tw, dct, nlines, sc, s, dot);
   if (dot) {
     DotFuse df{dot->r, dot->q, dot->partials, dot->sc, dot->flex};
     if (periodic)
@@ -518,6 +449,7 @@ void fft_y_inverse(int N, int periodic, const T* in, double* out, const T* tw, c
 template <typename T>
 void fft_x(int N, int periodic, int inverse, const T* in, T* out, const T* tw, const T* dct,
            long long inner, long long outer, const DevScalars* sc, cudaStream_t s) {
+  if (!fft_pow2(N)) return fft_mixed_x<T>(N, periodic, inverse, in, out, tw, dct, inner, outer, sc, s);
   if (periodic)
     dispatch<T, FFT_DHT, false, T, T>(N, in, out, tw, dct, inner, outer, inner, sc, s);
   else if (!inverse)
@@ -562,6 +494,7 @@ int fft_configure() {
   bad |= set_attr_one<double, FFT_DHT, false, double, double>();
   bad |= set_attr_one<double, FFT_DCT2, false, double, double>();
   bad |= set_attr_one<double, FFT_DCT3, false, double, double>();
+  bad |= fft_mixed_configure() != MFG_OK;
   return bad ? MFG_ERR_CUDA : MFG_OK;
 }
 

@@ -16,10 +16,10 @@
 //
 // Passes over the data (ping-pong work buffers, 10n words in total):
 //   y-forward, x-forward, [time forward, divide by S, time inverse] fused,
-//   x-inverse, y-inverse.  A spatial pass is an FFT (k_fft.cu) when the axis
-//   length is a power of two from 8 to 512, otherwise a small dense matrix
-//   applied along the axis (a SIMT GEMM with the transform matrix on the
-//   left); the time pass is a tridiagonal elimination per spatial mode, or the
+//   x-inverse, y-inverse.  A spatial pass is an FFT (k_fft.cu, k_fft_mixed.cu)
+//   when the axis length has no prime factor above 13, otherwise a small dense
+//   matrix applied along the axis (a SIMT GEMM with the transform matrix on
+//   the left); the time pass is a tridiagonal elimination per spatial mode, or the
 //   two dense products on the tensor cores (k_time_tc.cu).
 #include <algorithm>
 #include <cmath>
@@ -183,8 +183,8 @@ int build_prec_tables(const mfg_problem& p, const Geom& g, PrecTables* t, std::s
   auto fft_tables = [&](int N, double** tw64, float** tw32, double** dc64, float** dc32) {
     if (!fft_supported(N)) return true;
     const double pi = 3.14159265358979323846;
-    std::vector<double> tw((size_t)N), dc((size_t)2 * N);
-    for (int m = 0; m < N / 2; ++m) {
+    std::vector<double> tw((size_t)2 * N), dc((size_t)2 * N);
+    for (int m = 0; m < N; ++m) {
       tw[2 * m] = std::cos(2.0 * pi * m / N);
       tw[2 * m + 1] = std::sin(2.0 * pi * m / N);
     }

@@ -122,8 +122,8 @@ struct PrecTables {
   int l = 1;  // time preconditioner (mfg_problem::l)
   double *Hx64, *Hy64, *Vt64, *lamt64, *L1_64, *L2_64;  // device, FP64
   float *Hx32, *Hy32, *Vt32, *lamt32, *L1_32, *L2_32;   // device, FP32
-  // FFT twiddles for power-of-two axes (null otherwise): tw (N/2 complex),
-  // dct (N complex) per axis, both precisions.
+  // FFT twiddles per axis (null where no FFT pass exists), both precisions: tw
+  // (N complex; power-of-two passes read N/2), dct (N complex).
   double *twx64 = nullptr, *dctx64 = nullptr, *twy64 = nullptr, *dcty64 = nullptr;
   float *twx32 = nullptr, *dctx32 = nullptr, *twy32 = nullptr, *dcty32 = nullptr;
   // l = 0 (exact time solve): Thomas factors c_k(s), 1/den_k(s) (n each) and
@@ -188,7 +188,9 @@ void launch_precond_band(const Geom& g, const PrecTables& t, int precision, cons
 int band_configure();
 int precond_configure();
 
-// FFT spatial passes (k_fft.cu).
+// FFT spatial passes (k_fft.cu: powers of two from 8 to 512; k_fft_mixed.cu: other
+// lengths up to 2048 without a prime factor above 13).
+bool fft_pow2(int N);
 bool fft_supported(int N);
 long long fft_dot_partials(const Geom& g);
 int fft_configure();

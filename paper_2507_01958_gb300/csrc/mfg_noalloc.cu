@@ -143,7 +143,7 @@ void carve(double* base, const Geom& g, int l, PrecTables* t, T** w0) {
   T* L2 = p; p += kNaS;
   T* twx = p; T* dctx = p + kNaMaxAxis; p += kNaTw;
   T* twy = p; T* dcty = p + kNaMaxAxis;
-  const bool fx = g.nx > 1 && fft_supported(g.nx), fy = fft_supported(g.ny);
+  const bool fx = g.nx > 1 && fft_pow2(g.nx), fy = fft_pow2(g.ny);
   if (!fx) twx = dctx = nullptr;
   if (!fy) twy = dcty = nullptr;
   if constexpr (sizeof(T) == 8) {
