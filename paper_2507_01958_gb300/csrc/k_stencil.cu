@@ -12,9 +12,20 @@
 // it sits at the matching end of a Neumann axis.
 #include "df64.cuh"
 #include "mfg_internal.cuh"
+#include "pcg_tail.cuh"
 #include "reduce.cuh"
+#include "strip.cuh"
 
 namespace mfg {
+
+// 256-thread blocks per SM that the launch bounds of the strip kernels admit
+constexpr int kCPerSm = 2, kCtPerSm = 3, kUPerSm = 5, kQPerSm = 3;
+
+// Whether C and C^T run in strips: not for viscosity fields, and not where the
+// strips would be less than ~60 % full (the point-by-point kernels issue 28 and 23 FP64
+// instructions per point, the strips 15 and 12 per lane; 200 x 33 x 31: 44 us for C, C^T
+// and AAt point by point, 51 us in strips; 33 x 200 x 31: 40 against 37).
+bool strips_fit(const Geom& g) { return g.kfy == nullptr && (g.ny + 31) / 32 * 32 * 3 <= 5 * g.ny; }
 
 struct Nb {
   int im, ip;
@@ -56,11 +67,121 @@ __device__ __forceinline__ int wrap_or_neg(int i, int N, int per) {
 //         alpha = rz/(pdot.r).
 // mode 3: adjoint right-hand side r = C v; reduces ||r||^2, resets the PCG
 //         state with the fixed tolerance.
-// VN (viscosity field): nu K m becomes K_nu m = sum over the node's faces of
-// kf (m - m_nb), kf the face coefficient of Geom::kfx / kfy; at a Neumann end
-// the neighbour index is the node itself, so the missing face adds nothing.
+//
+// Terms of a point, in face form (each face formed once, see strip.cuh):
+// F = w1_i + w2_{i+1} per face, div_h w = (F_{i+1/2} - F_{i-1/2}) / dx + the y faces, 0
+// past a Neumann end.  FP64 issue bounds the kernel: 13 instructions per point
+// (15 with oblong cells; 2 more with Az) instead of ~28 point by point.
+__device__ __forceinline__ void rhs_tail(double acc, double accb, bool have_b, double* partials, DevScalars* sc) {
+  double part[2] = {acc, accb};
+  block_sum<2>(part);
+  if (!publish_and_check_last<2>(part, partials, &sc->counter)) return;
+  double tot[2];
+  gather_partials<2>(partials, tot);
+  if (flat_tid() == 0) {
+    const double rr0 = tot[0], b2 = have_b ? tot[1] : tot[0];
+    sc->bnorm2 = b2;  // reference of the relative tolerance: ||b||^2 or ||r_0||^2
+    sc->rr = rr0;
+    sc->cg_it = 0;
+    // The paper's adaptive rule, min{1e-4, max{1e-6, 1e-4 r}} (Sec. 5).
+    double tol = sc->cg_tol_fixed;
+    if (sc->cg_rule == MFG_CG_ADAPTIVE) tol = fmin(1e-4, fmax(1e-6, 1e-4 * sc->r_last));
+    sc->cg_tol = tol;
+    // no iteration when r_0 = 0 or r_0 is already inside the tolerance (NaN: flagged below)
+    sc->cg_done = !(rr0 > 0.0) || rr0 <= tol * tol * b2;
+    if (!isfinite(rr0) || !isfinite(b2)) {
+      sc->cg_done = 1;
+      sc->status = MFG_ERR_NONFINITE;
+    }
+    sc->counter = 0;
+  }
+}
+
+template <int ACTX, bool ISO, int MODE>
+__global__ void __launch_bounds__(256, kCPerSm) k_apply_C(Geom g, StripGrid sg, const double* __restrict__ v,
+                                                    double* __restrict__ r, double alpha,
+                                                    const double* __restrict__ m0, const double* __restrict__ pdot,
+                                                    double* partials, DevScalars* sc, double* __restrict__ Az) {
+  if (MODE == 2 && sc->cg_done) return;
+  if (MODE == 1) alpha = sc->sigma;
+  double acc = 0.0, accb = 0.0;
+  int j0, i0, i1, k;
+  if (strip_item(sg, g, j0, i0, i1, k)) {
+    const long long n = g.n, base = (long long)k * g.S;
+    const double* m = v + base;
+    const double* wx1 = v + n + base;
+    const double* wx2 = v + 2 * n + base;
+    const double* wy1 = v + (ACTX ? 3 : 1) * n + base;
+    const double* wy2 = v + (ACTX ? 4 : 2) * n + base;
+    const StripCols c = strip_cols(g, j0);
+    const int lane = threadIdx.x & 31, j = j0 + lane;
+    const bool end_y = !g.pery && j == g.ny - 1;  // no face beyond
+    auto at = [&](int i, int jj) { return i * g.ny + jj; };  // < S, an int
+    const int ir = min(i0 + lane, i1 - 1);
+    const double w2r = wy2[at(ir, c.right)];
+    const double hf = (!g.pery && j0 == 0) ? 0.0 : wy1[at(ir, c.left)] + wy2[at(ir, j0)];
+    double fxm = 0.0;
+    if (ACTX && (g.perx || i0 > 0)) fxm = wx1[at(ghost(i0 - 1, g.nx, g.perx), c.j)] + wx2[at(i0, c.j)];
+    const double ky = alpha * g.nu * g.ay, rho = ACTX ? g.ax / g.ay : 0.0, kc = 2.0 * (1.0 + rho) * ky;
+    const double aix = alpha * g.idx, aiy = alpha * g.idy, aidt = alpha * g.idt;
+    const double* mp = k >= 1 ? m - g.S : m0;  // m of the previous level (plane 0: m0, or 0)
+    struct Row {
+      double wy1, wy2, wx1, wx2, mp, extra;
+    };
+    const bool have_mp = mp != nullptr, have_az = MODE == 1 && Az != nullptr;
+    sum_march<ISO, 2>(
+        g, rho, i0, i1, j0, [&](int i, int jj) { return m[at(i, jj)]; },
+        [&](int i) {
+          const int e = at(i, c.j);
+          Row w{wy1[e], wy2[e], 0.0, 0.0, 0.0, 0.0};
+          if (ACTX) {
+            w.wx1 = wx1[e];
+            w.wx2 = wx2[at(ghost(i + 1, g.nx, g.perx), c.j)];
+          }
+          if (have_mp) w.mp = mp[e];
+          if (MODE == 2) w.extra = pdot[base + e];
+          if (have_az) w.extra = Az[base + e];
+          return w;
+        },
+        [&](int i, double mc, double sum, const Row& w) {
+          double fy = w.wy1 + from_right(w.wy2, w2r, i - i0);
+          if (end_y) fy = 0.0;
+          const double sy = fy - from_left(fy, hf, i - i0);
+          double val = fma(kc, mc, -ky * sum);
+          if (ACTX) {
+            const double fx = (!g.perx && i == g.nx - 1) ? 0.0 : w.wx1 + w.wx2;
+            const double sx = fx - fxm;
+            fxm = fx;
+            val = ISO ? fma(aiy, sx + sy, val) : fma(aix, sx, fma(aiy, sy, val));
+          } else {
+            val = fma(aiy, sy, val);
+          }
+          if (j >= g.ny) return;
+          val = fma(aidt, mc - w.mp, val);
+          const int e = at(i, j);
+          r[base + e] = val;
+          if constexpr (MODE == 2) acc = fma(w.extra, val, acc);
+          if constexpr (MODE == 1 || MODE == 3) acc = fma(val, val, acc);
+          if constexpr (MODE == 1) {
+            if (have_az) {
+              const double b = w.extra + val;
+              Az[base + e] = b;
+              accb = fma(b, b, accb);
+            }
+          }
+        });
+  }
+  if constexpr (MODE == 2) aat_tail(acc, partials, sc);
+  if constexpr (MODE == 1 || MODE == 3) rhs_tail(acc, accb, Az != nullptr, partials, sc);
+}
+
+// The same terms point by point, for viscosity fields and for grids whose rows
+// would leave most of a 32-column strip empty (strips_fit).  VN (viscosity field):
+// nu K m becomes K_nu m = sum over the node's faces of kf (m - m_nb), kf the face
+// coefficient of Geom::kfx / kfy; at a Neumann end the neighbour index is the node
+// itself, so the missing face adds nothing.
 template <int ACTX, bool VN>
-__global__ void __launch_bounds__(kThreads) k_apply_C(Geom g, const double* __restrict__ v,
+__global__ void __launch_bounds__(kThreads) k_apply_C_flat(Geom g, const double* __restrict__ v,
                                                       double* __restrict__ r, double alpha,
                                                       const double* __restrict__ m0,
                                                       const double* __restrict__ pdot,
@@ -127,64 +248,86 @@ __global__ void __launch_bounds__(kThreads) k_apply_C(Geom g, const double* __re
     }
   }
   if (mode == 0) return;
-  double part[2] = {acc, accb};
-  block_sum<2>(part);
-  if (!publish_and_check_last<2>(part, partials, &sc->counter)) return;
-  double tot[2];
-  gather_partials<2>(partials, tot);
-  if (mode == 2) {
-    if (flat_tid() == 0) {
-      sc->pq = tot[0];
-      if (tot[0] > 0.0 && isfinite(tot[0])) {
-        sc->alpha = sc->rz / tot[0];
-      } else {
-        sc->alpha = 0.0;
-        sc->cg_done = 1;
-        if (sc->status == MFG_OK) sc->status = MFG_ERR_NONFINITE;
-      }
-      sc->counter = 0;
-    }
-    return;
-  }
-  if (flat_tid() == 0) {
-    const double rr0 = tot[0], b2 = (Az != nullptr) ? tot[1] : tot[0];
-    sc->bnorm2 = b2;  // reference of the relative tolerance: ||b||^2 or ||r_0||^2
-    sc->rr = rr0;
-    sc->cg_it = 0;
-    // The paper's adaptive rule, min{1e-4, max{1e-6, 1e-4 r}} (Sec. 5).
-    double tol = sc->cg_tol_fixed;
-    if (sc->cg_rule == MFG_CG_ADAPTIVE) tol = fmin(1e-4, fmax(1e-6, 1e-4 * sc->r_last));
-    sc->cg_tol = tol;
-    // no iteration when r_0 = 0 or r_0 is already inside the tolerance (NaN: flagged below)
-    sc->cg_done = !(rr0 > 0.0) || rr0 <= tol * tol * b2;
-    if (!isfinite(rr0) || !isfinite(b2)) {
-      sc->cg_done = 1;
-      sc->status = MFG_ERR_NONFINITE;
-    }
-    sc->counter = 0;
-  }
+  if (mode == 2)
+    aat_tail(acc, partials, sc);
+  else
+    rhs_tail(acc, accb, Az != nullptr, partials, sc);
 }
 
 void launch_apply_C(const Geom& g, const double* v, double* r, double alpha, const double* m0,
                     double* partials, DevScalars* sc, int mode, cudaStream_t s, const double* pdot,
                     double* Az) {
-  const int nb = red_blocks(g.n, g.vec_blocks);
-  const bool vn = g.kfy != nullptr;
-  if (g.actx && vn)
-    k_apply_C<1, true><<<nb, kThreads, 0, s>>>(g, v, r, alpha, m0, pdot, partials, sc, mode, Az);
-  else if (g.actx)
-    k_apply_C<1, false><<<nb, kThreads, 0, s>>>(g, v, r, alpha, m0, pdot, partials, sc, mode, Az);
-  else if (vn)
-    k_apply_C<0, true><<<nb, kThreads, 0, s>>>(g, v, r, alpha, m0, pdot, partials, sc, mode, Az);
+  if (!strips_fit(g)) {
+    const int nb = red_blocks(g.n, g.vec_blocks);
+#define MFG_C_FLAT(A, N) k_apply_C_flat<A, N><<<nb, kThreads, 0, s>>>(g, v, r, alpha, m0, pdot, partials, sc, mode, Az)
+    if (g.kfy != nullptr) { if (g.actx) MFG_C_FLAT(1, true); else MFG_C_FLAT(0, true); }
+    else                  { if (g.actx) MFG_C_FLAT(1, false); else MFG_C_FLAT(0, false); }
+#undef MFG_C_FLAT
+    return;
+  }
+  const StripGrid sg = strip_grid(g, kCPerSm);
+#define MFG_C(A, I, M) \
+  k_apply_C<A, I, M><<<sg.blocks, 32 * sg.warps, 0, s>>>(g, sg, v, r, alpha, m0, pdot, partials, sc, Az)
+#define MFG_C_MODE(A, I)       \
+  switch (mode) {              \
+    case 0: MFG_C(A, I, 0); break; \
+    case 1: MFG_C(A, I, 1); break; \
+    case 2: MFG_C(A, I, 2); break; \
+    default: MFG_C(A, I, 3); break; \
+  }
+  if (!g.actx)
+    MFG_C_MODE(0, false)
+  else if (g.ax == g.ay)
+    MFG_C_MODE(1, true)
   else
-    k_apply_C<0, false><<<nb, kThreads, 0, s>>>(g, v, r, alpha, m0, pdot, partials, sc, mode, Az);
+    MFG_C_MODE(1, false)
+#undef MFG_C_MODE
+#undef MFG_C
 }
 
 // ----------------------------------------------------------------- C^T p --
 // x_m^k = L p^k - p^{k+1}/dt (p^{N_t} := 0),  x_w^k = B^T p^k = -D_h p^k.
-// VN: L = K_nu + I/dt with the face coefficients of Geom::kfx / kfy.
+// Face form: the two flux rows of an axis are the same face differences, one
+// node apart, so each is formed and scaled once (10 FP64 instructions per point
+// instead of ~23; 48 bytes written and 8 read).
+template <int ACTX>
+__global__ void __launch_bounds__(256, kCtPerSm) k_apply_Ct(Geom g, StripGrid sg, const double* __restrict__ p,
+                                                     double* __restrict__ x) {
+  int j0, i0, i1, k;
+  if (!strip_item(sg, g, j0, i0, i1, k)) return;
+  const long long n = g.n, base = (long long)k * g.S;
+  const double* pk = p + base;
+  double* xm = x + base;
+  double* xx1 = x + n + base;
+  double* xx2 = x + 2 * n + base;
+  double* xy1 = x + (ACTX ? 3 : 1) * n + base;
+  double* xy2 = x + (ACTX ? 4 : 2) * n + base;
+  const int j = j0 + (threadIdx.x & 31);
+  const bool last = k + 1 >= g.nt;
+  const double nx = g.nu * g.idx, ny = g.nu * g.idy;  // nu K p from the scaled differences
+  const int jc = j < g.ny ? j : g.ny - 1;
+  diff_march<ACTX, true, 4>(
+      g, i0, i1, j0, [&](int i, int jj) { return pk[i * g.ny + jj]; },
+      [&](int i) { return last ? 0.0 : pk[i * g.ny + jc + g.S]; },
+      [&](int i, double pc, double dyp, double dym, double dxp, double dxm, double pn) {
+        if (j >= g.ny) return;
+        const int e = i * g.ny + j;
+        double m = fma(ny, dyp - dym, (pc - pn) * g.idt);
+        xy1[e] = dyp;
+        xy2[e] = dym;
+        if (ACTX) {
+          m = fma(nx, dxp - dxm, m);
+          xx1[e] = dxp;
+          xx2[e] = dxm;
+        }
+        xm[e] = m;
+      });
+}
+
+// Point by point (see k_apply_C_flat).  VN: L = K_nu + I/dt with the face
+// coefficients of Geom::kfx / kfy.
 template <int ACTX, bool VN>
-__global__ void __launch_bounds__(kThreads) k_apply_Ct(Geom g, const double* __restrict__ p,
+__global__ void __launch_bounds__(kThreads) k_apply_Ct_flat(Geom g, const double* __restrict__ p,
                                                        double* __restrict__ x) {
   const long long n = g.n;
   double* xm = x;
@@ -224,54 +367,117 @@ __global__ void __launch_bounds__(kThreads) k_apply_Ct(Geom g, const double* __r
 }
 
 void launch_apply_Ct(const Geom& g, const double* p, double* x, cudaStream_t s) {
-  const int nb = red_blocks(g.n, g.vec_blocks);
-  const bool vn = g.kfy != nullptr;
-  if (g.actx && vn)
-    k_apply_Ct<1, true><<<nb, kThreads, 0, s>>>(g, p, x);
-  else if (g.actx)
-    k_apply_Ct<1, false><<<nb, kThreads, 0, s>>>(g, p, x);
-  else if (vn)
-    k_apply_Ct<0, true><<<nb, kThreads, 0, s>>>(g, p, x);
+  if (!strips_fit(g)) {
+    const int nb = red_blocks(g.n, g.vec_blocks);
+#define MFG_CT_FLAT(A, N) k_apply_Ct_flat<A, N><<<nb, kThreads, 0, s>>>(g, p, x)
+    if (g.kfy != nullptr) { if (g.actx) MFG_CT_FLAT(1, true); else MFG_CT_FLAT(0, true); }
+    else                  { if (g.actx) MFG_CT_FLAT(1, false); else MFG_CT_FLAT(0, false); }
+#undef MFG_CT_FLAT
+    return;
+  }
+  const StripGrid sg = strip_grid(g, kCtPerSm);
+  if (g.actx)
+    k_apply_Ct<1><<<sg.blocks, 32 * sg.warps, 0, s>>>(g, sg, p, x);
   else
-    k_apply_Ct<0, false><<<nb, kThreads, 0, s>>>(g, p, x);
+    k_apply_Ct<0><<<sg.blocks, 32 * sg.warps, 0, s>>>(g, sg, p, x);
 }
 
 // ---------------------------------------------------------------- C C^T p --
-// Factored form q = C (C^T p).  With xm^k = L p^k - p^{k+1}/dt (the m rows of
-// C^T p) and B B^T = 2K (eq. precstead):
-//   q^k = L xm^k - xm^{k-1}/dt + 2 K p^k        (xm^{-1} := 0).
-//
 // FP64 issue is the limit on GB300 (a warp's FP64 instruction takes 16 SM
-// clocks; memory traffic is far below the HBM bound), so the stencil is laid
-// out for the fewest FP64 instructions per point:
-//   K u = cK u - ax (uW + uE) - ay (uN + uS),   cK = 2 (ax + ay)   (5 ops),
-// and it runs in two halo-free passes over the grid, each point computed once:
-//   pass 1:  kp = K p,   X = dt xm = fma(nu dt, kp, p^k - p^{k+1})        (7 ops)
-//   pass 2:  q = c4 X - c2 (XW + XE) - c1 (XN + XS) - X^{k-1}/dt^2 + 2 kp (7 ops)
-// with c1 = nu ay/dt, c2 = nu ax/dt, c4 = nu cK/dt + 1/dt^2, plus one FMA for
-// p.q.  (A one-pass version that forms xm on a shared-memory tile must
-// recompute it on the tile's halo and needs ~20 FP64 ops per point.)
+// clocks; the bytes moved take a third of that time), so the operator is
+// arranged for the fewest FP64 instructions per point.  With K p = -ay u,
+//   u = (p_S + p_N) + rho (p_W + p_E) - 2 (1 + rho) p,   rho = ax / ay,
+// and BB^T = 2K (eq. precstead), C C^T = L^2 in space, a second difference in
+// time, becomes
+//   q^k = (2 s^k - s^{k-1} - s^{k+1}) / dt^2 + nu^2 ay^2 U(u^k) - 2 ay u^k,
+//   s = p - nu ay dt u,   s^{-1} := p^0,   s^{N_t} := 0,
+// U the operator that takes p to u: two passes over the grid, each point
+// computed once, u and s through memory.
+// Square cells (rho = 1) share the diagonal pair sums A(i, j) = p(i, j+1) + p(i+1, j):
+//   p_N + p_S + p_W + p_E = A(i, j) + A(i-1, j-1),
+// one addition less per point and pass.  FP64 instructions per point: 4 + 8
+// with p.q (6 + 9 when rho != 1), against 15 for the factored form
+// L (L p^k - p^{k+1}/dt) - ... with K p and L p through memory.
 // On a Neumann axis the neighbour index of an end point is the point itself
 // (u_{-1} = u_0, u_N = u_{N-1}), which turns the same formula into the
-// one-sided D^1 (D^1)^T rows of Sec. 4.3, for p and for X alike.
-// Threads own one (i, j) column and march over a chunk of time planes, so
-// p^{k+1} and X^{k-1} stay in registers from one plane to the next.
-constexpr int AJ = 32, AI = 8;  // block = AJ x AI columns
-
+// one-sided D^1 (D^1)^T rows of Sec. 4.3, for p and for u alike.
+//
+// Both passes walk the grid in warp strips (strip.cuh).  512^2 x 128: 949 -> 756 us (11
+// FP64 instructions per point at 78 % of the FP64 pipe; 587 us at all of it).
 struct AatCoef {
-  double ax, ay, cK, ndt;      // pass 1
-  double c1, c2, c4, idt2;     // pass 2
-  double dt, idt;              // viscosity field (VN)
+  double rho, m2r;        // ax / ay, -2 (1 + rho)
+  double alpha;           // nu ay dt
+  double b, gu, idt2;     // nu^2 ay^2, -2 (1 + rho) b - 2 ay, 1/dt^2
+  double ax, ay, cK;      // viscosity field and double-float passes
+  double ndt, c1, c2, c4;
+  double dt, idt;
 };
 
 AatCoef aat_coef(const Geom& g) {
   const double ax = g.actx ? g.ax : 0.0, ay = g.ay, cK = 2.0 * (ax + ay);
-  const double dt = 1.0 / g.idt, idt2 = g.idt * g.idt;
-  return AatCoef{ax, ay, cK, g.nu * dt, g.nu * ay * g.idt, g.nu * ax * g.idt, g.nu * cK * g.idt + idt2, idt2,
-                 dt, g.idt};
+  const double dt = 1.0 / g.idt, idt2 = g.idt * g.idt, rho = ax / ay, b = g.nu * ay * (g.nu * ay);
+  return AatCoef{rho, -2.0 * (1.0 + rho), g.nu * ay * dt, b, -2.0 * (1.0 + rho) * b - 2.0 * ay, idt2, ax, ay, cK,
+                 g.nu * dt, g.nu * ay * g.idt, g.nu * ax * g.idt, g.nu * cK * g.idt + idt2, dt, g.idt};
 }
 
+template <bool ISO>
+__global__ void __launch_bounds__(256, kUPerSm) k_aat_u(Geom g, AatCoef a, StripGrid ag, const double* __restrict__ p,
+                                               double* __restrict__ U, double* __restrict__ Sx,
+                                               const DevScalars* sc, int mode) {
+  if (mode != 0 && sc->cg_done) return;
+  int j0, i0, i1, k;
+  if (!strip_item(ag, g, j0, i0, i1, k)) return;
+  const long long base = (long long)k * g.S;
+  const double* pk = p + base;
+  const int j = j0 + (threadIdx.x & 31);
+  sum_march<ISO, 4>(g, a.rho, i0, i1, j0, [&](int i, int jj) { return pk[i * g.ny + jj]; },
+                    [](int) { return 0; }, [&](int i, double c, double sum, int) {
+                   if (j >= g.ny) return;
+                   const double u = fma(a.m2r, c, sum);
+                   const long long e = base + (long long)i * g.ny + j;
+                   U[e] = u;
+                   Sx[e] = fma(-a.alpha, u, c);
+                 });
+}
 
+// q = AAt p; STEP (PCG step): also reduces p.q and sets alpha = rz/(p.q) in the
+// device scalars.
+template <bool ISO, bool STEP>
+__global__ void __launch_bounds__(256, kQPerSm) k_aat_q2(Geom g, AatCoef a, StripGrid ag, const double* __restrict__ U,
+                                                   const double* __restrict__ Sx, const double* __restrict__ p,
+                                                   double* __restrict__ q, double* partials, DevScalars* sc) {
+  if (STEP && sc->cg_done) return;
+  double acc = 0.0;
+  int j0, i0, i1, k;
+  if (strip_item(ag, g, j0, i0, i1, k)) {
+    const long long base = (long long)k * g.S;
+    const double* uk = U + base;
+    const int j = j0 + (threadIdx.x & 31);
+    const double* sm = k > 0 ? Sx - g.S : p;  // s^{-1} := p^0
+    const bool last = k == g.nt - 1;
+    struct Row {
+      double s0, sm, sp, p;
+    };
+    const int jc = j < g.ny ? j : g.ny - 1;
+    sum_march<ISO, 4>(g, a.rho, i0, i1, j0, [&](int i, int jj) { return uk[i * g.ny + jj]; },
+                      [&](int i) {
+                        const long long e = base + i * g.ny + jc;
+                        return Row{Sx[e], sm[e], last ? 0.0 : Sx[e + g.S], STEP ? p[e] : 0.0};
+                      },
+                      [&](int i, double c, double sum, const Row& w) {
+                        if (j >= g.ny) return;
+                        const double dd = fma(2.0, w.s0, -(w.sm + w.sp));
+                        const double qv = fma(a.gu, c, fma(a.b, sum, a.idt2 * dd));
+                        q[base + i * g.ny + j] = qv;
+                        if constexpr (STEP) acc = fma(qv, w.p, acc);
+                      });
+  }
+  if constexpr (STEP) aat_tail(acc, partials, sc);
+}
+
+// Viscosity field (VN) and double-float passes: threads own one (i, j) column
+// and march over a chunk of time planes, so p^{k+1} and X^{k-1} stay in registers.
+constexpr int AJ = 32, AI = 8;  // block = AJ x AI columns
 
 int aat2_chunk(const Geom& g) {
   const long long cols = (long long)((g.ny + AJ - 1) / AJ) * ((g.nx + AI - 1) / AI);
@@ -320,7 +526,7 @@ __device__ __forceinline__ FaceCoef face_coef(const Geom& g, int i, int j, const
   return f;
 }
 
-template <int ACTX, bool VN>
+template <int ACTX>
 __global__ void __launch_bounds__(AJ * AI) k_aat_x(Geom g, AatCoef a, int kc, const double* __restrict__ p,
                                                    double* __restrict__ X, double* __restrict__ KP,
                                                    const DevScalars* sc, int mode) {
@@ -330,8 +536,7 @@ __global__ void __launch_bounds__(AJ * AI) k_aat_x(Geom g, AatCoef a, int kc, co
   const int k0 = blockIdx.z * kc, k1 = min(g.nt, k0 + kc);
   const Cols nb = aat_cols(g, i, j);
   const long long row = (long long)i * g.ny;
-  FaceCoef fc{0.0, 0.0, 0.0, 0.0};
-  if (VN) fc = face_coef(g, i, j, nb, a.dt);
+  const FaceCoef fc = face_coef(g, i, j, nb, a.dt);
   long long base = (long long)k0 * g.S;
   double c = p[base + row + j];
   for (int k = k0; k < k1; ++k) {
@@ -345,24 +550,17 @@ __global__ void __launch_bounds__(AJ * AI) k_aat_x(Geom g, AatCoef a, int kc, co
       t = fma(a.ax, pW + pE, t);
     }
     const double kp = fma(a.cK, c, -t);
-    if (VN) {
-      double kv = fma(fc.yp, c - pN, fc.ym * (c - pS));  // dt K_nu p
-      if (ACTX) kv = fma(fc.xp, c - pE, fma(fc.xm, c - pW, kv));
-      X[base + row + j] = kv + (c - pn);
-    } else {
-      X[base + row + j] = fma(a.ndt, kp, c - pn);
-    }
+    double kv = fma(fc.yp, c - pN, fc.ym * (c - pS));  // dt K_nu p
+    if (ACTX) kv = fma(fc.xp, c - pE, fma(fc.xm, c - pW, kv));
+    X[base + row + j] = kv + (c - pn);
     KP[base + row + j] = kp;
     c = pn;
     base += g.S;
   }
 }
 
-// mode 0: q = AAt p.  mode 1 (PCG step): also reduces p.q and sets
-// alpha = rz/(p.q) in the device scalars.
-template <int ACTX, bool VN>
-// 2-D: capped at 64 registers (four 256-thread blocks per SM) to hide the load latency
-__global__ void __launch_bounds__(AJ * AI, (ACTX && !VN) ? 4 : 3) k_aat_q(Geom g, AatCoef a, int kc, const double* __restrict__ X,
+template <int ACTX>
+__global__ void __launch_bounds__(AJ * AI, 3) k_aat_q(Geom g, AatCoef a, int kc, const double* __restrict__ X,
                                                    const double* __restrict__ KP, const double* __restrict__ p,
                                                    double* __restrict__ q, double* partials, DevScalars* sc,
                                                    int mode) {
@@ -373,28 +571,18 @@ __global__ void __launch_bounds__(AJ * AI, (ACTX && !VN) ? 4 : 3) k_aat_q(Geom g
     const int k0 = blockIdx.z * kc, k1 = min(g.nt, k0 + kc);
     const Cols nb = aat_cols(g, i, j);
     const long long row = (long long)i * g.ny;
-    FaceCoef fc{0.0, 0.0, 0.0, 0.0};
-    if (VN) fc = face_coef(g, i, j, nb, a.idt);
+    const FaceCoef fc = face_coef(g, i, j, nb, a.idt);
     long long base = (long long)k0 * g.S;
     double xprev = k0 > 0 ? X[base - g.S + row + j] : 0.0;
     for (int k = k0; k < k1; ++k) {
       const double xc = X[base + row + j];
-      double qv;
-      if (VN) {
-        const double xS = X[base + row + nb.jm], xN = X[base + row + nb.jp];
-        double kv = fma(fc.yp, xc - xN, fc.ym * (xc - xS));  // K_nu X / dt
-        if (ACTX) {
-          const double xW = X[base + (long long)nb.im * g.ny + j], xE = X[base + (long long)nb.ip * g.ny + j];
-          kv = fma(fc.xp, xc - xE, fma(fc.xm, xc - xW, kv));
-        }
-        qv = fma(2.0, KP[base + row + j], fma(a.idt2, xc - xprev, kv));
-      } else {
-        double t = a.c1 * (X[base + row + nb.jm] + X[base + row + nb.jp]);
-        if (ACTX) t = fma(a.c2, X[base + (long long)nb.im * g.ny + j] + X[base + (long long)nb.ip * g.ny + j], t);
-        t = fma(a.idt2, xprev, t);
-        t = fma(-2.0, KP[base + row + j], t);
-        qv = fma(a.c4, xc, -t);
+      const double xS = X[base + row + nb.jm], xN = X[base + row + nb.jp];
+      double kv = fma(fc.yp, xc - xN, fc.ym * (xc - xS));  // K_nu X / dt
+      if (ACTX) {
+        const double xW = X[base + (long long)nb.im * g.ny + j], xE = X[base + (long long)nb.ip * g.ny + j];
+        kv = fma(fc.xp, xc - xE, fma(fc.xm, xc - xW, kv));
       }
+      const double qv = fma(2.0, KP[base + row + j], fma(a.idt2, xc - xprev, kv));
       q[base + row + j] = qv;
       if (mode == 1) acc = fma(qv, p[base + row + j], acc);
       xprev = xc;
@@ -402,27 +590,14 @@ __global__ void __launch_bounds__(AJ * AI, (ACTX && !VN) ? 4 : 3) k_aat_q(Geom g
     }
   }
   if (mode == 0) return;
-  double part[1] = {acc};
-  block_sum<1>(part);
-  if (!publish_and_check_last<1>(part, partials, &sc->counter)) return;
-  double tot[1];
-  gather_partials<1>(partials, tot);
-  if (flat_tid() == 0) {
-    sc->pq = tot[0];
-    if (tot[0] > 0.0 && isfinite(tot[0])) {
-      sc->alpha = sc->rz / tot[0];
-    } else {
-      sc->alpha = 0.0;
-      sc->cg_done = 1;
-      if (sc->status == MFG_OK) sc->status = MFG_ERR_NONFINITE;
-    }
-    sc->counter = 0;
-  }
+  aat_tail(acc, partials, sc);
 }
 
+// Blocks of the largest reducing launch of this file (viscosity fields and the
+// double-float stencil use the column grid).
 int aat_blocks(const Geom& g) {
   const dim3 g2 = aat2_grid(g, aat2_chunk(g));
-  return (int)((long long)g2.x * g2.y * g2.z);
+  return std::max({(int)((long long)g2.x * g2.y * g2.z), strip_grid(g, kQPerSm).blocks, strip_grid(g, kCPerSm).blocks});
 }
 
 // The same two passes in double-float arithmetic (df64.cuh, the MFG_MIXED_DF
@@ -492,22 +667,7 @@ __global__ void __launch_bounds__(AJ * AI) k_aat_q_df(Geom g, AatCoef ad, int kc
     }
   }
   if (mode == 0) return;
-  double part[1] = {acc};
-  block_sum<1>(part);
-  if (!publish_and_check_last<1>(part, partials, &sc->counter)) return;
-  double tot[1];
-  gather_partials<1>(partials, tot);
-  if (flat_tid() == 0) {
-    sc->pq = tot[0];
-    if (tot[0] > 0.0 && isfinite(tot[0])) {
-      sc->alpha = sc->rz / tot[0];
-    } else {
-      sc->alpha = 0.0;
-      sc->cg_done = 1;
-      if (sc->status == MFG_OK) sc->status = MFG_ERR_NONFINITE;
-    }
-    sc->counter = 0;
-  }
+  aat_tail(acc, partials, sc);
 }
 
 void launch_AAt(const Geom& g, const double* p, double* q, double* scratch, double* partials,
@@ -527,22 +687,29 @@ void launch_AAt(const Geom& g, const double* p, double* q, double* scratch, doub
     }
     return;
   }
-  double* X = scratch;
-  double* KP = scratch + g.n;
-  const bool vn = g.kfy != nullptr;
-  if (g.actx && vn) {
-    k_aat_x<1, true><<<grid, block, 0, s>>>(g, a, kc, p, X, KP, sc, mode);
-    k_aat_q<1, true><<<grid, block, 0, s>>>(g, a, kc, X, KP, p, q, partials, sc, mode);
-  } else if (g.actx) {
-    k_aat_x<1, false><<<grid, block, 0, s>>>(g, a, kc, p, X, KP, sc, mode);
-    k_aat_q<1, false><<<grid, block, 0, s>>>(g, a, kc, X, KP, p, q, partials, sc, mode);
-  } else if (vn) {
-    k_aat_x<0, true><<<grid, block, 0, s>>>(g, a, kc, p, X, KP, sc, mode);
-    k_aat_q<0, true><<<grid, block, 0, s>>>(g, a, kc, X, KP, p, q, partials, sc, mode);
-  } else {
-    k_aat_x<0, false><<<grid, block, 0, s>>>(g, a, kc, p, X, KP, sc, mode);
-    k_aat_q<0, false><<<grid, block, 0, s>>>(g, a, kc, X, KP, p, q, partials, sc, mode);
+  double* X = scratch;  // u, or X = dt xm of a viscosity field
+  double* KP = scratch + g.n;  // s, or K p
+  if (g.kfy != nullptr) {
+    if (g.actx) {
+      k_aat_x<1><<<grid, block, 0, s>>>(g, a, kc, p, X, KP, sc, mode);
+      k_aat_q<1><<<grid, block, 0, s>>>(g, a, kc, X, KP, p, q, partials, sc, mode);
+    } else {
+      k_aat_x<0><<<grid, block, 0, s>>>(g, a, kc, p, X, KP, sc, mode);
+      k_aat_q<0><<<grid, block, 0, s>>>(g, a, kc, X, KP, p, q, partials, sc, mode);
+    }
+    return;
   }
+  const StripGrid ug = strip_grid(g, kUPerSm), ag = strip_grid(g, kQPerSm);
+  const int nth = 32 * ag.warps;
+  const bool iso = g.actx && g.ax == g.ay, step = mode != 0;
+#define MFG_AAT(I, ST) k_aat_q2<I, ST><<<ag.blocks, nth, 0, s>>>(g, a, ag, X, KP, p, q, partials, sc)
+  if (iso)
+    k_aat_u<true><<<ug.blocks, 32 * ug.warps, 0, s>>>(g, a, ug, p, X, KP, sc, mode);
+  else
+    k_aat_u<false><<<ug.blocks, 32 * ug.warps, 0, s>>>(g, a, ug, p, X, KP, sc, mode);
+  if (iso) { if (step) MFG_AAT(true, true); else MFG_AAT(true, false); }
+  else     { if (step) MFG_AAT(false, true); else MFG_AAT(false, false); }
+#undef MFG_AAT
 }
 
 int aat_kernel_count(int) { return 2; }

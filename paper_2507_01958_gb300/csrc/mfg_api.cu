@@ -412,7 +412,7 @@ double time_us(F&& f, cudaStream_t s, cudaEvent_t a, cudaEvent_t b) {
 //                                    cores (MFG_MIXED_TC); FFT or dense pass per
 //                                    power-of-two axis; timed as the PCG step
 //                                    (fused z, r update and dot products)
-//   AAt stencil target blocks        152 x 4, 8, 16
+//   AAt stencil launch (aat_want)    152 x 4, 8, 16
 int tune_instance(Inst& in, double* zbuf, cudaStream_t s, cudaEvent_t a, cudaEvent_t b) {
   const long long n = in.g.n;
   int rc;
@@ -466,7 +466,7 @@ int tune_instance(Inst& in, double* zbuf, cudaStream_t s, cudaEvent_t a, cudaEve
   {
     double best = 1e300;
     int choice = g.aat_want;
-    for (int want : {152 * 4, 152 * 8, 152 * 16}) {
+    for (int want : kAatWants) {
       Geom c = g;
       c.aat_want = want;
       if ((rc = reset_tune_scalars(in, s))) return rc;
@@ -624,11 +624,14 @@ int mfg_plan(const mfg_problem* probs, int batch, mfg_plan_t* out) {
     in.g.kfy = in.tabs.kfy;
     in.p.nu_field = nullptr;
     const size_t n = (size_t)in.g.n;
-    // partial sums for the largest grids any launch choice may use
-    Geom gmax = in.g;
-    gmax.aat_want = kAatWantMax;
-    size_t npart = (size_t)std::max<long long>(std::max(2 * kVecBlocksMax, aat_blocks(gmax)),
-                                               fft_dot_partials(in.g));
+    // partial sums for the largest grids any launch choice may use (two sums per block)
+    long long most = std::max<long long>(2 * kVecBlocksMax, fft_dot_partials(in.g));
+    for (int want : kAatWants) {
+      Geom gw = in.g;
+      gw.aat_want = want;
+      most = std::max<long long>(most, 2LL * aat_blocks(gw));
+    }
+    const size_t npart = (size_t)most;
     if (cudaMalloc(&in.r, n * 8) != cudaSuccess || cudaMalloc(&in.pv, n * 8) != cudaSuccess ||
         cudaMalloc(&in.q, n * 8) != cudaSuccess || cudaMalloc(&in.zp, n * 8) != cudaSuccess ||
         cudaMalloc(&in.partials, npart * 8) != cudaSuccess)

@@ -15,7 +15,7 @@ constexpr int kThreads = 256;        // threads per block for 1-D launches
 constexpr int kRedBlocks = 152 * 2;
 constexpr int kVecBlocksMax = 152 * 4;   // largest vec_blocks the autotuner tries
 constexpr int kAatWantDefault = 152 * 8;
-constexpr int kAatWantMax = 152 * 16;    // largest aat_want the autotuner tries
+constexpr int kAatWants[3] = {152 * 4, kAatWantDefault, 152 * 16};  // what the autotuner tries
 constexpr int kMaxNt = 256;          // largest N_t of the fused time-transform kernel
 
 // Geometry and coefficients of one instance on the device.  Internally every
@@ -36,7 +36,8 @@ struct Geom {
   // measured ones.  They change launch shapes and pass variants, never the
   // operator a kernel applies.
   int vec_blocks;   // grid cap of the vector and reduction kernels
-  int aat_want;     // target block count of the AAt stencil launch
+  int aat_want;     // twice the blocks of a wave the strip kernels' row chunks are chosen for; target
+                    // block count of the column kernels (viscosity field, double-float)
   int time_simt;    // 1: time pass by elimination on the CUDA cores even where the tensor-core pass applies
   int fft_x, fft_y; // 1: FFT spatial pass where the axis length allows it; 0: dense pass
   // Viscosity field (mfg_problem::nu_field): per node, the coefficient of its

@@ -7,6 +7,26 @@
 
 namespace mfg {
 
+// After q = AAt p: acc = this thread's share of p.q; alpha = rz / (p.q).
+__device__ __forceinline__ void aat_tail(double acc, double* partials, DevScalars* sc) {
+  double part[1] = {acc};
+  block_sum<1>(part);
+  if (!publish_and_check_last<1>(part, partials, &sc->counter)) return;
+  double tot[1];
+  gather_partials<1>(partials, tot);
+  if (flat_tid() == 0) {
+    sc->pq = tot[0];
+    if (tot[0] > 0.0 && isfinite(tot[0])) {
+      sc->alpha = sc->rz / tot[0];
+    } else {
+      sc->alpha = 0.0;
+      sc->cg_done = 1;
+      if (sc->status == MFG_OK) sc->status = MFG_ERR_NONFINITE;
+    }
+    sc->counter = 0;
+  }
+}
+
 // After z += alpha p, r -= alpha q: rr = this thread's share of ||r||^2; the
 // convergence test.
 __device__ __forceinline__ void zr_tail(double rr, double* partials, DevScalars* sc) {

@@ -19,27 +19,31 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// Sum of `v` over the block; the result is valid in thread 0.  Up to 1024 threads.
+// Sum of `v` over the block; the result is valid in thread 0.  Up to 256 threads,
+// whole warps.  Through shared memory: one warp per value adds the threads'
+// columns and ends with one shuffle tree, 5 + (warps - 1) FP64 instructions per
+// value where a tree in every warp takes 5 (warps + 1); on GB300 each of them
+// holds the SM's FP64 unit for 16 cycles, and a block of a reduction kernel has
+// often only tens per thread.
 template <int NV>
 __device__ __forceinline__ void block_sum(double (&v)[NV]) {
-  __shared__ double ws[NV][32];
-  const int tid = flat_tid(), lane = tid & 31, w = tid >> 5, nw = (flat_nthreads() + 31) >> 5;
-#pragma unroll
-  for (int q = 0; q < NV; ++q) v[q] = warp_sum(v[q]);
+  __shared__ double ws[NV][256];
+  const int tid = flat_tid(), lane = tid & 31, w = tid >> 5, nw = flat_nthreads() >> 5;
   __syncthreads();
-  if (lane == 0) {
 #pragma unroll
-    for (int q = 0; q < NV; ++q) ws[q][w] = v[q];
-  }
+  for (int q = 0; q < NV; ++q) ws[q][tid] = v[q];
   __syncthreads();
-  if (w == 0) {
 #pragma unroll
-    for (int q = 0; q < NV; ++q) {
-      double t = lane < nw ? ws[q][lane] : 0.0;
-      v[q] = warp_sum(t);
+  for (int q = 0; q < NV; ++q)
+    if (w == q % nw) {
+      double t = ws[q][lane];
+      for (int i = 1; i < nw; ++i) t += ws[q][lane + 32 * i];
+      t = warp_sum(t);
+      if (lane == 0) ws[q][0] = t;
     }
-  }
   __syncthreads();
+#pragma unroll
+  for (int q = 0; q < NV; ++q) v[q] = ws[q][0];
 }
 
 // Publishes this block's partial sums (valid in thread 0) and returns true in
