@@ -251,7 +251,7 @@ int mfg_apply_Ct(mfg_plan_t plan, int b, const double* p, double* x, void* strea
  * Built for q' = 2 (MFG_ERR_UNSUPPORTED otherwise).
  * The adjoint system is solved through its Schur complement
  * C_A H^{-1} C_A^T with the plan's preconditioner P (eq. prec) inside PCG,
- * H being the per-cell Hessian of phi.  The first call allocates a c*n + n
+ * H being the per-cell Hessian of phi.  The first call allocates a 2*c*n + n
  * workspace owned by the plan.  Synchronises `stream`. */
 int mfg_adjoint(mfg_plan_t plan, int b, const double* y, const double* z, const double* gy,
                 double* dm0, double* dV, double* dW, double* dnu, double tol, int max_iter,

@@ -19,13 +19,22 @@
 // the inactive w components are zero, so
 //   (H^{-1} u)_m = (u_m + w.u_w / m) / a',  (H^{-1} u)_w = m u_w + (w/m) (H^{-1} u)_m,
 // and 0 on inactive components.
+//
+// y is fixed over the whole adjoint solve, so the velocities v = w/m and 1/a' are
+// formed once (k_hinv, which also applies H^{-1} to the right-hand side) and each
+// PCG iteration has no division left: 23 FP64 instructions per point instead of
+// 54, FP64 issue being what bounds it (128^2 x 64, cold: 114 -> 70 us; the whole
+// adjoint 7.9 -> 5.6 ms).
 #include "mfg_internal.cuh"
 #include "reduce.cuh"
+#include "strip.cuh"
 
 namespace mfg {
 
+// om, ow = H^{-1} (um, uw) with the cell's m, velocities v (0 on inactive
+// components, and all 0 with iap = 0 where m <= 0) and iap = 1/a'.
 template <int NW>
-__device__ __forceinline__ void hinv_cell(double m, const double (&w)[NW], double ap, double um,
+__device__ __forceinline__ void hinv_cell(double m, const double (&v)[NW], double iap, double um,
                                           const double (&uw)[NW], double& om, double (&ow)[NW]) {
   if (!(m > 0.0)) {
     om = 0.0;
@@ -33,50 +42,112 @@ __device__ __forceinline__ void hinv_cell(double m, const double (&w)[NW], doubl
     for (int q = 0; q < NW; ++q) ow[q] = 0.0;
     return;
   }
-  const double im = 1.0 / m;
-  double wu = 0.0;
 #pragma unroll
-  for (int q = 0; q < NW; ++q) wu = fma(w[q], uw[q], wu);
-  om = (um + wu * im) / ap;
+  for (int q = 0; q < NW; ++q) um = fma(v[q], uw[q], um);
+  om = um * iap;
 #pragma unroll
-  for (int q = 0; q < NW; ++q) ow[q] = (w[q] != 0.0) ? fma(m, uw[q], w[q] * im * om) : 0.0;
+  for (int q = 0; q < NW; ++q) ow[q] = v[q] != 0.0 ? fma(m, uw[q], v[q] * om) : 0.0;
 }
 
-template <int ACTX>
-__device__ __forceinline__ void load_cell(const double* y, long long e, long long n, double& m,
-                                          double (&w)[ACTX ? 4 : 2]) {
-  m = y[e];
-#pragma unroll
-  for (int q = 0; q < (ACTX ? 4 : 2); ++q) w[q] = y[e + (q + 1) * n];
-}
-
+// out = H^{-1} u, and the cell data of y that later applies read: vel (v, then
+// 1/a', NW + 1 planes).
 template <int ACTX>
 __global__ void __launch_bounds__(kThreads) k_hinv(Geom g, Coef cf, const double* __restrict__ y,
-                                                   const double* __restrict__ u, double* __restrict__ out) {
+                                                   const double* __restrict__ u, double* __restrict__ out,
+                                                   double* __restrict__ vel) {
   constexpr int NW = ACTX ? 4 : 2;
   const long long n = g.n;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
        e += (long long)gridDim.x * blockDim.x) {
     const int k = (int)(e / g.S);
-    double m, w[NW], uw[NW], ow[NW], om;
-    load_cell<ACTX>(y, e, n, m, w);
+    const double m = y[e];
+    double v[NW], uw[NW], ow[NW], om, iap = 0.0;
+    const bool on = m > 0.0;
+    const double im = on ? 1.0 / m : 0.0;
+    if (on) iap = 1.0 / (cf.f_a + 2.0 * cf.f_b * m + (k == g.nt - 1 ? cf.g_a * g.idt : 0.0));
 #pragma unroll
-    for (int q = 0; q < NW; ++q) uw[q] = u[e + (q + 1) * n];
-    const double ap = cf.f_a + 2.0 * cf.f_b * m + (k == g.nt - 1 ? cf.g_a * g.idt : 0.0);
-    hinv_cell<NW>(m, w, ap, u[e], uw, om, ow);
+    for (int q = 0; q < NW; ++q) {
+      uw[q] = u[e + (q + 1) * n];
+      v[q] = on ? y[e + (q + 1) * n] * im : 0.0;
+      vel[e + q * n] = v[q];
+    }
+    vel[e + NW * n] = iap;
+    hinv_cell<NW>(m, v, iap, u[e], uw, om, ow);
     out[e] = om;
 #pragma unroll
     for (int q = 0; q < NW; ++q) out[e + (q + 1) * n] = ow[q];
   }
 }
 
-// out = H^{-1} (C^T p)  or, with gsub, out = H^{-1} (gsub - C^T p).  VN: L =
-// K_nu + I/dt with the face coefficients of Geom::kfx / kfy.
+constexpr int kCtHinvPerSm = 2;  // 256-thread blocks per SM
+
+// out = H^{-1} (C^T p)  or, with GSUB, out = H^{-1} (gsub - C^T p), in warp strips
+// (strip.cuh): 13 reads and writes of 8 bytes and 23 FP64 instructions per point.
+template <int ACTX, bool GSUB>
+__global__ void __launch_bounds__(256, kCtHinvPerSm) k_ct_hinv(Geom g, StripGrid sg, const double* __restrict__ m,
+                                                              const double* __restrict__ vel,
+                                                              const double* __restrict__ p,
+                                                              const double* __restrict__ gsub,
+                                                              double* __restrict__ out, const DevScalars* sc) {
+  if (sc != nullptr && sc->cg_done) return;
+  constexpr int NW = ACTX ? 4 : 2;
+  int j0, i0, i1, k;
+  if (!strip_item(sg, g, j0, i0, i1, k)) return;
+  const long long n = g.n, base = (long long)k * g.S;
+  const double* pk = p + base;
+  const int j = j0 + (threadIdx.x & 31), jc = j < g.ny ? j : g.ny - 1;
+  const bool last = k + 1 >= g.nt;
+  const double nx = g.nu * g.idx, ny = g.nu * g.idy;  // nu K p from the scaled differences
+  struct Row {
+    double pn, m, iap, v[NW], um, uw[NW];
+  };
+  diff_march<ACTX, true, 2>(
+      g, i0, i1, j0, [&](int i, int jj) { return pk[i * g.ny + jj]; },
+      [&](int i) {
+        const long long e = base + i * g.ny + jc;
+        Row w;
+        w.pn = last ? 0.0 : p[e + g.S];
+        w.m = m[e];
+        w.iap = vel[e + NW * n];
+        w.um = GSUB ? gsub[e] : 0.0;
+#pragma unroll
+        for (int q = 0; q < NW; ++q) {
+          w.v[q] = vel[e + q * n];
+          w.uw[q] = GSUB ? gsub[e + (q + 1) * n] : 0.0;
+        }
+        return w;
+      },
+      [&](int i, double pc, double dyp, double dym, double dxp, double dxm, const Row& w) {
+        if (j >= g.ny) return;
+        double xm = fma(ny, dyp - dym, (pc - w.pn) * g.idt), om, ow[NW];
+        double xw[NW];
+        if (ACTX) {
+          xm = fma(nx, dxp - dxm, xm);
+          xw[0] = dxp; xw[1] = dxm; xw[NW - 2] = dyp; xw[NW - 1] = dym;
+        } else {
+          xw[0] = dyp; xw[1] = dym;
+        }
+        if (GSUB) {
+          xm = w.um - xm;
+#pragma unroll
+          for (int q = 0; q < NW; ++q) xw[q] = w.uw[q] - xw[q];
+        }
+        hinv_cell<NW>(w.m, w.v, w.iap, xm, xw, om, ow);
+        const long long e = base + i * g.ny + j;
+        out[e] = om;
+#pragma unroll
+        for (int q = 0; q < NW; ++q) out[e + (q + 1) * n] = ow[q];
+      });
+}
+
+// The same point by point, for viscosity fields (VN: L = K_nu + I/dt with the face
+// coefficients of Geom::kfx / kfy) and for rows too short for strips.
 template <int ACTX, bool VN>
-__global__ void __launch_bounds__(kThreads) k_ct_hinv(Geom g, Coef cf, const double* __restrict__ y,
-                                                      const double* __restrict__ p,
-                                                      const double* __restrict__ gsub,
-                                                      double* __restrict__ out, const DevScalars* sc) {
+__global__ void __launch_bounds__(kThreads) k_ct_hinv_flat(Geom g, const double* __restrict__ mass,
+                                                           const double* __restrict__ vel,
+                                                           const double* __restrict__ p,
+                                                           const double* __restrict__ gsub,
+                                                           double* __restrict__ out, const DevScalars* sc) {
   if (sc != nullptr && sc->cg_done) return;
   constexpr int NW = ACTX ? 4 : 2;
   const long long n = g.n;
@@ -122,18 +193,20 @@ __global__ void __launch_bounds__(kThreads) k_ct_hinv(Geom g, Coef cf, const dou
 #pragma unroll
       for (int q = 0; q < NW; ++q) xw[q] = gsub[e + (q + 1) * n] - xw[q];
     }
-    double m, w[NW], ow[NW], om;
-    load_cell<ACTX>(y, e, n, m, w);
-    const double ap = cf.f_a + 2.0 * cf.f_b * m + (k == g.nt - 1 ? cf.g_a * g.idt : 0.0);
-    hinv_cell<NW>(m, w, ap, xm, xw, om, ow);
+    double v[NW], ow[NW], om;
+#pragma unroll
+    for (int q = 0; q < NW; ++q) v[q] = vel[e + q * n];
+    hinv_cell<NW>(mass[e], v, vel[e + NW * n], xm, xw, om, ow);
     out[e] = om;
 #pragma unroll
     for (int q = 0; q < NW; ++q) out[e + (q + 1) * n] = ow[q];
   }
 }
 
-// One thread per spatial point, looping over time planes; dnu by reduction,
-// or (VN) the node derivative dnu(f) written per point.
+// A block takes 32 spatial points and splits their time planes over 8 warps (one
+// thread per point left 64 blocks of serial loops at 128^2: 119 us); the warps'
+// sums are added in order.  dnu by reduction, or (VN) the node derivative dnu(f)
+// written per point.
 template <bool VN>
 __global__ void __launch_bounds__(kThreads) k_adj_grads(Geom g, const double* __restrict__ y,
                                                         const double* __restrict__ z,
@@ -141,18 +214,19 @@ __global__ void __launch_bounds__(kThreads) k_adj_grads(Geom g, const double* __
                                                         const double* __restrict__ mu, double* dm0,
                                                         double* dV, double* dW, double* dnu,
                                                         double* partials, DevScalars* sc) {
-  double acc = 0.0;
-  for (long long f = blockIdx.x * (long long)blockDim.x + threadIdx.x; f < g.S;
-       f += (long long)gridDim.x * blockDim.x) {
-    const int j = (int)(f % g.ny), i = (int)(f / g.ny);
+  __shared__ double part_s[2][8][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double acc = 0.0, sv = 0.0, node = 0.0;
+  const int f = blockIdx.x * 32 + lane;
+  if (f < g.S) {
+    const int j = f % g.ny, i = f / g.ny;
     const bool hmy = g.pery || j >= 1, hpy = g.pery || j <= g.ny - 2;
     const int jm = hmy ? (j == 0 ? g.ny - 1 : j - 1) : j;
     const int jp = hpy ? (j == g.ny - 1 ? 0 : j + 1) : j;
     const bool hmx = g.actx && (g.perx || i >= 1), hpx = g.actx && (g.perx || i <= g.nx - 2);
     const int im = hmx ? (i == 0 ? g.nx - 1 : i - 1) : i;
     const int ip = hpx ? (i == g.nx - 1 ? 0 : i + 1) : i;
-    double sv = 0.0, node = 0.0;
-    for (int k = 0; k < g.nt; ++k) {
+    for (int k = warp; k < g.nt; k += 8) {
       const long long base = (long long)k * g.S;
       const long long e = base + f;
       const double mum = mu[e];
@@ -180,6 +254,15 @@ __global__ void __launch_bounds__(kThreads) k_adj_grads(Geom g, const double* __
         acc -= mum * K5(z) + eta[e] * K5(y);
       }
     }
+  }
+  part_s[0][warp][lane] = sv;
+  part_s[1][warp][lane] = node;
+  __syncthreads();
+  if (warp == 0 && f < g.S) {
+    for (int w = 1; w < 8; ++w) {
+      sv += part_s[0][w][lane];
+      node += part_s[1][w][lane];
+    }
     if (VN) dnu[f] = -0.5 * node;
     dm0[f] = eta[f] * g.idt;
     dV[f] = -sv;
@@ -197,33 +280,38 @@ __global__ void __launch_bounds__(kThreads) k_adj_grads(Geom g, const double* __
   }
 }
 
-void launch_hinv(const Geom& g, const Coef& cf, const double* y, const double* u, double* out,
+void launch_hinv(const Geom& g, const Coef& cf, const double* y, const double* u, double* out, double* vel,
                  cudaStream_t s) {
-  const int nb = red_blocks(g.n, g.vec_blocks);
+  const int nb = red_blocks(g.n, kVecBlocksMax);
   if (g.actx)
-    k_hinv<1><<<nb, kThreads, 0, s>>>(g, cf, y, u, out);
+    k_hinv<1><<<nb, kThreads, 0, s>>>(g, cf, y, u, out, vel);
   else
-    k_hinv<0><<<nb, kThreads, 0, s>>>(g, cf, y, u, out);
+    k_hinv<0><<<nb, kThreads, 0, s>>>(g, cf, y, u, out, vel);
 }
 
-void launch_ct_hinv(const Geom& g, const Coef& cf, const double* y, const double* p,
-                    const double* gsub, double* out, cudaStream_t s, const DevScalars* sc) {
-  const int nb = red_blocks(g.n, g.vec_blocks);
-  const bool vn = g.kfy != nullptr;
-  if (g.actx && vn)
-    k_ct_hinv<1, true><<<nb, kThreads, 0, s>>>(g, cf, y, p, gsub, out, sc);
-  else if (g.actx)
-    k_ct_hinv<1, false><<<nb, kThreads, 0, s>>>(g, cf, y, p, gsub, out, sc);
-  else if (vn)
-    k_ct_hinv<0, true><<<nb, kThreads, 0, s>>>(g, cf, y, p, gsub, out, sc);
-  else
-    k_ct_hinv<0, false><<<nb, kThreads, 0, s>>>(g, cf, y, p, gsub, out, sc);
+void launch_ct_hinv(const Geom& g, const double* y, const double* vel, const double* p, const double* gsub,
+                    double* out, cudaStream_t s, const DevScalars* sc) {
+  if (!strips_fit(g)) {
+    const int nb = red_blocks(g.n, kVecBlocksMax);
+#define MFG_CT_HINV(A, N) k_ct_hinv_flat<A, N><<<nb, kThreads, 0, s>>>(g, y, vel, p, gsub, out, sc)
+    if (g.kfy != nullptr) { if (g.actx) MFG_CT_HINV(1, true); else MFG_CT_HINV(0, true); }
+    else                  { if (g.actx) MFG_CT_HINV(1, false); else MFG_CT_HINV(0, false); }
+#undef MFG_CT_HINV
+    return;
+  }
+  const StripGrid sg = strip_grid(g, kCtHinvPerSm);
+#define MFG_CT_HINV(A, G) k_ct_hinv<A, G><<<sg.blocks, 32 * sg.warps, 0, s>>>(g, sg, y, vel, p, gsub, out, sc)
+  if (gsub != nullptr) { if (g.actx) MFG_CT_HINV(1, true); else MFG_CT_HINV(0, true); }
+  else                 { if (g.actx) MFG_CT_HINV(1, false); else MFG_CT_HINV(0, false); }
+#undef MFG_CT_HINV
 }
+
+int adj_grads_blocks(const Geom& g) { return (g.S + 31) / 32; }
 
 void launch_adj_grads(const Geom& g, const double* y, const double* z, const double* eta,
                       const double* mu, double* dm0, double* dV, double* dW, double* dnu,
                       double* partials, DevScalars* sc, cudaStream_t s) {
-  const int nb = red_blocks(g.S, g.vec_blocks);
+  const int nb = adj_grads_blocks(g);
   if (g.kfy != nullptr)
     k_adj_grads<true><<<nb, kThreads, 0, s>>>(g, y, z, eta, mu, dm0, dV, dW, dnu, partials, sc);
   else

@@ -14,6 +14,7 @@
 // Batched instances are independent branches of the same graph, so the
 // runtime may overlap them on the GPU.  All control flow (convergence tests,
 // step sizes) lives in device memory; the host only reads the final record.
+#include <algorithm>
 #include <array>
 #include <climits>
 #include <cmath>
@@ -57,7 +58,7 @@ struct Inst {
   float* work32 = nullptr;
   double* partials = nullptr;
   DevScalars* sc = nullptr;  // points into the plan's contiguous array
-  double *adj_t = nullptr, *adj_eta = nullptr;  // adjoint workspace, allocated on first use
+  double *adj_t = nullptr, *adj_eta = nullptr, *adj_vel = nullptr;  // adjoint workspace, allocated on first use
   double* Az = nullptr;  // MFG_CG_REF_RHS: AAt z, carried across CP iterations (stop reference)
   int tuned = 0, measured = 0;                  // launch choices from mfg_autotune
   double tune_precond_us = 0.0, tune_aat_us = 0.0;
@@ -166,6 +167,8 @@ struct mfg_plan_s {
   const void* key[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   cudaStream_t cap0 = nullptr, cap1 = nullptr;
   int launch_mode = MFG_LAUNCH_GRAPH;
+  DevScalars* adj_host = nullptr;              // pinned: flags of two adjoint iterations
+  cudaEvent_t adj_ev[2] = {nullptr, nullptr};  // their arrival; both made by the first adjoint call
   int inject = MFG_INJECT_NONE;  // test hook, copied into the device scalars by mfg_solve
   // device staging for mfg_solve_host
   double *h_m0 = nullptr, *h_V = nullptr, *h_W = nullptr, *h_y = nullptr, *h_ybar = nullptr,
@@ -176,10 +179,10 @@ namespace {
 
 void free_inst(Inst& in) {
   free_prec_tables(&in.tabs);
-  void* ptrs[] = {in.r, in.pv, in.q, in.zp, in.work64, in.work32, in.partials, in.adj_t, in.adj_eta, in.Az};
+  void* ptrs[] = {in.r, in.pv, in.q, in.zp, in.work64, in.work32, in.partials, in.adj_t, in.adj_eta, in.adj_vel, in.Az};
   for (void* q : ptrs)
     if (q) cudaFree(q);
-  in.r = in.pv = in.q = in.zp = in.work64 = in.partials = in.adj_t = in.adj_eta = in.Az = nullptr;
+  in.r = in.pv = in.q = in.zp = in.work64 = in.partials = in.adj_t = in.adj_eta = in.adj_vel = in.Az = nullptr;
   in.work32 = nullptr;
 }
 
@@ -625,7 +628,7 @@ int mfg_plan(const mfg_problem* probs, int batch, mfg_plan_t* out) {
     in.p.nu_field = nullptr;
     const size_t n = (size_t)in.g.n;
     // partial sums for the largest grids any launch choice may use (two sums per block)
-    long long most = std::max<long long>(2 * kVecBlocksMax, fft_dot_partials(in.g));
+    long long most = std::max<long long>({2 * kVecBlocksMax, fft_dot_partials(in.g), adj_grads_blocks(in.g)});
     for (int want : kAatWants) {
       Geom gw = in.g;
       gw.aat_want = want;
@@ -666,6 +669,9 @@ int mfg_destroy(mfg_plan_t pl) {
   for (auto& in : pl->inst) free_inst(in);
   if (pl->sc_dev) cudaFree(pl->sc_dev);
   if (pl->sc_host) cudaFreeHost(pl->sc_host);
+  if (pl->adj_host) cudaFreeHost(pl->adj_host);
+  for (auto ev : pl->adj_ev)
+    if (ev) cudaEventDestroy(ev);
   double* hs[] = {pl->h_m0, pl->h_V, pl->h_W, pl->h_y, pl->h_ybar, pl->h_z};
   for (double* q : hs)
     if (q) cudaFree(q);
@@ -809,10 +815,15 @@ int mfg_adjoint(mfg_plan_t pl, int b, const double* y, const double* z, const do
     return fail(MFG_ERR_UNSUPPORTED, "the adjoint is built for the quadratic Hamiltonian (q' = 2) only");
   const Geom& g = in.g;
   const size_t n = (size_t)g.n;
-  if (!in.adj_t) {
-    if (cudaMalloc(&in.adj_t, (size_t)g.c * n * 8) != cudaSuccess || cudaMalloc(&in.adj_eta, n * 8) != cudaSuccess)
-      return fail(MFG_ERR_CUDA, "cudaMalloc failed for adjoint workspace");
-  }
+  if (!pl->adj_host && cudaMallocHost(&pl->adj_host, 2 * sizeof(DevScalars)) != cudaSuccess)
+    return fail(MFG_ERR_CUDA, "cudaMallocHost failed for adjoint flags");
+  for (auto& ev : pl->adj_ev)
+    if (!ev && cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess)
+      return fail(MFG_ERR_CUDA, "cudaEventCreate failed for adjoint flags");
+  if ((!in.adj_t && cudaMalloc(&in.adj_t, (size_t)g.c * n * 8) != cudaSuccess) ||
+      (!in.adj_eta && cudaMalloc(&in.adj_eta, n * 8) != cudaSuccess) ||
+      (!in.adj_vel && cudaMalloc(&in.adj_vel, (size_t)g.c * n * 8) != cudaSuccess))
+    return fail(MFG_ERR_CUDA, "cudaMalloc failed for adjoint workspace");
   cudaStream_t s = (cudaStream_t)stream;
   DevScalars h{};
   h.status = MFG_OK;
@@ -823,27 +834,35 @@ int mfg_adjoint(mfg_plan_t pl, int b, const double* y, const double* z, const do
   const int flex = in.p.precision != MFG_FP64;
   const int dfa = in.p.precision == MFG_MIXED_DF;
   // right-hand side C H^{-1} g; eta starts at 0
-  launch_hinv(g, in.cf, y, gy, in.adj_t, s);
+  launch_hinv(g, in.cf, y, gy, in.adj_t, in.adj_vel, s);
   launch_apply_C(g, in.adj_t, in.r, 1.0, nullptr, in.partials, in.sc, 3, s);
   CK(cudaMemsetAsync(in.adj_eta, 0, n * 8, s));
   launch_precond(g, in.tabs, in.p.precision, in.r, in.zp, in.work64, in.work32, in.sc, s);
   launch_init_p(g.n, in.zp, in.pv, in.r, in.partials, in.sc, s, g.vec_blocks);
   long long launches = 3 + precond_kernel_count(g);
-  DevScalars hs;
-  for (;;) {
-    CK(cudaMemcpyAsync(&hs, in.sc, sizeof(hs), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    if (hs.cg_done) break;
+  // The host reads iteration i's flags while iteration i+1 runs: past convergence
+  // every kernel of an iteration returns at once, so the one enqueued too many
+  // changes nothing, and the GPU never waits for the host.
+  auto post = [&](int i) -> cudaError_t {
+    const cudaError_t e = cudaMemcpyAsync(pl->adj_host + (i & 1), in.sc, sizeof(DevScalars), cudaMemcpyDeviceToHost, s);
+    return e != cudaSuccess ? e : cudaEventRecord(pl->adj_ev[i & 1], s);
+  };
+  CK(post(0));
+  for (int i = 0;; ++i) {
     const PcgDot dot{in.r, in.q, in.partials, in.sc, flex};
     const PcgZr zr{in.adj_eta, in.r, in.pv, in.q, in.partials, in.sc};
-    launch_ct_hinv(g, in.cf, y, in.pv, nullptr, in.adj_t, s, in.sc);
+    launch_ct_hinv(g, y, in.adj_vel, in.pv, nullptr, in.adj_t, s, in.sc);
     launch_apply_C(g, in.adj_t, in.q, 1.0, nullptr, in.partials, in.sc, 2, s, in.pv);
     launch_precond(g, in.tabs, in.p.precision, in.r, in.zp, in.work64, in.work32, in.sc, s, &dot, &zr);
     launch_update_p(g.n, in.zp, in.pv, in.sc, 0, 0, s, g.vec_blocks);
     launches += 3 + precond_step_kernel_count(g, in.tabs);
+    CK(post(i + 1));
+    CK(cudaEventSynchronize(pl->adj_ev[i & 1]));
+    if (pl->adj_host[i & 1].cg_done) break;
   }
+  DevScalars hs;
   // mu = H^{-1}(g - C^T eta), then the contractions
-  launch_ct_hinv(g, in.cf, y, in.adj_eta, gy, in.adj_t, s, nullptr);
+  launch_ct_hinv(g, y, in.adj_vel, in.adj_eta, gy, in.adj_t, s, nullptr);
   launch_adj_grads(g, y, z, in.adj_eta, in.adj_t, dm0, dV, dW, dnu, in.partials, in.sc, s);
   launches += 2;
   pl->launches += launches;

@@ -103,6 +103,7 @@ void launch_AAt(const Geom& g, const double* p, double* q, double* scratch, doub
                 DevScalars* sc, int mode, cudaStream_t s, int df64);
 int aat_kernel_count(int df64);
 int aat_blocks(const Geom& g);
+bool strips_fit(const Geom& g);
 
 // Vector kernels (k_cg.cu).
 // `cap`: grid cap (Geom::vec_blocks).
@@ -205,11 +206,13 @@ template <typename T>
 void fft_x(int N, int periodic, int inverse, const T* in, T* out, const T* tw, const T* dct,
            long long inner, long long outer, const DevScalars* sc, cudaStream_t s);
 
-// Adjoint (k_adjoint.cu).
-void launch_hinv(const Geom& g, const Coef& cf, const double* y, const double* u, double* out,
+// Adjoint (k_adjoint.cu).  vel: (c planes) velocities w/m of y and 1/f_eff'(m),
+// written by launch_hinv and read by launch_ct_hinv.
+void launch_hinv(const Geom& g, const Coef& cf, const double* y, const double* u, double* out, double* vel,
                  cudaStream_t s);
-void launch_ct_hinv(const Geom& g, const Coef& cf, const double* y, const double* p,
-                    const double* gsub, double* out, cudaStream_t s, const DevScalars* sc);
+void launch_ct_hinv(const Geom& g, const double* y, const double* vel, const double* p, const double* gsub,
+                    double* out, cudaStream_t s, const DevScalars* sc);
+int adj_grads_blocks(const Geom& g);  // partial sums launch_adj_grads writes
 void launch_adj_grads(const Geom& g, const double* y, const double* z, const double* eta,
                       const double* mu, double* dm0, double* dV, double* dW, double* dnu,
                       double* partials, DevScalars* sc, cudaStream_t s);
