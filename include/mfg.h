@@ -345,8 +345,9 @@ int mfg_set_fault_injection(mfg_plan_t plan, int what);
  *     Calls on one stream are ordered and safe.
  *   - r, z: n device doubles, caller-owned, must not alias.  Stream-ordered;
  *     returns after enqueueing.
- *   - Same passes as mfg_apply_precond: FFT spatial passes on power-of-two
- *     axes (twiddles are part of the static array), dense ones otherwise.
+ *   - Same passes as mfg_apply_precond: FFT spatial passes on axes without a
+ *     prime factor above 13 (twiddles are part of the static array), dense ones
+ *     otherwise.
  *     p->precision: MFG_FP64 and MFG_MIXED as in a plan, MFG_MIXED_TC with the
  *     tensor-core time pass as in a plan; MFG_MIXED_DF runs as MFG_MIXED (the
  *     two differ only in the AAt stencil, which this apply does not use).

@@ -55,6 +55,7 @@ template <int ACTX>
 __global__ void __launch_bounds__(kThreads) k_hinv(Geom g, Coef cf, const double* __restrict__ y,
                                                    const double* __restrict__ u, double* __restrict__ out,
                                                    double* __restrict__ vel) {
+  dep_sync();
   constexpr int NW = ACTX ? 4 : 2;
   const long long n = g.n;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
@@ -89,6 +90,7 @@ __global__ void __launch_bounds__(256, kCtHinvPerSm) k_ct_hinv(Geom g, StripGrid
                                                               const double* __restrict__ p,
                                                               const double* __restrict__ gsub,
                                                               double* __restrict__ out, const DevScalars* sc) {
+  dep_sync();
   if (sc != nullptr && sc->cg_done) return;
   constexpr int NW = ACTX ? 4 : 2;
   int j0, i0, i1, k;
@@ -148,6 +150,7 @@ __global__ void __launch_bounds__(kThreads) k_ct_hinv_flat(Geom g, const double*
                                                            const double* __restrict__ p,
                                                            const double* __restrict__ gsub,
                                                            double* __restrict__ out, const DevScalars* sc) {
+  dep_sync();
   if (sc != nullptr && sc->cg_done) return;
   constexpr int NW = ACTX ? 4 : 2;
   const long long n = g.n;
@@ -214,6 +217,7 @@ __global__ void __launch_bounds__(kThreads) k_adj_grads(Geom g, const double* __
                                                         const double* __restrict__ mu, double* dm0,
                                                         double* dV, double* dW, double* dnu,
                                                         double* partials, DevScalars* sc) {
+  dep_sync();
   __shared__ double part_s[2][8][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double acc = 0.0, sv = 0.0, node = 0.0;
@@ -284,23 +288,23 @@ void launch_hinv(const Geom& g, const Coef& cf, const double* y, const double* u
                  cudaStream_t s) {
   const int nb = red_blocks(g.n, kVecBlocksMax);
   if (g.actx)
-    k_hinv<1><<<nb, kThreads, 0, s>>>(g, cf, y, u, out, vel);
+    launch_k(k_hinv<1>, nb, kThreads, 0, s, g, cf, y, u, out, vel);
   else
-    k_hinv<0><<<nb, kThreads, 0, s>>>(g, cf, y, u, out, vel);
+    launch_k(k_hinv<0>, nb, kThreads, 0, s, g, cf, y, u, out, vel);
 }
 
 void launch_ct_hinv(const Geom& g, const double* y, const double* vel, const double* p, const double* gsub,
                     double* out, cudaStream_t s, const DevScalars* sc) {
   if (!strips_fit(g)) {
     const int nb = red_blocks(g.n, kVecBlocksMax);
-#define MFG_CT_HINV(A, N) k_ct_hinv_flat<A, N><<<nb, kThreads, 0, s>>>(g, y, vel, p, gsub, out, sc)
+#define MFG_CT_HINV(A, N) launch_k(k_ct_hinv_flat<A, N>, nb, kThreads, 0, s, g, y, vel, p, gsub, out, sc)
     if (g.kfy != nullptr) { if (g.actx) MFG_CT_HINV(1, true); else MFG_CT_HINV(0, true); }
     else                  { if (g.actx) MFG_CT_HINV(1, false); else MFG_CT_HINV(0, false); }
 #undef MFG_CT_HINV
     return;
   }
   const StripGrid sg = strip_grid(g, kCtHinvPerSm);
-#define MFG_CT_HINV(A, G) k_ct_hinv<A, G><<<sg.blocks, 32 * sg.warps, 0, s>>>(g, sg, y, vel, p, gsub, out, sc)
+#define MFG_CT_HINV(A, G) launch_k(k_ct_hinv<A, G>, sg.blocks, 32 * sg.warps, 0, s, g, sg, y, vel, p, gsub, out, sc)
   if (gsub != nullptr) { if (g.actx) MFG_CT_HINV(1, true); else MFG_CT_HINV(0, true); }
   else                 { if (g.actx) MFG_CT_HINV(1, false); else MFG_CT_HINV(0, false); }
 #undef MFG_CT_HINV
@@ -313,9 +317,9 @@ void launch_adj_grads(const Geom& g, const double* y, const double* z, const dou
                       double* partials, DevScalars* sc, cudaStream_t s) {
   const int nb = adj_grads_blocks(g);
   if (g.kfy != nullptr)
-    k_adj_grads<true><<<nb, kThreads, 0, s>>>(g, y, z, eta, mu, dm0, dV, dW, dnu, partials, sc);
+    launch_k(k_adj_grads<true>, nb, kThreads, 0, s, g, y, z, eta, mu, dm0, dV, dW, dnu, partials, sc);
   else
-    k_adj_grads<false><<<nb, kThreads, 0, s>>>(g, y, z, eta, mu, dm0, dV, dW, dnu, partials, sc);
+    launch_k(k_adj_grads<false>, nb, kThreads, 0, s, g, y, z, eta, mu, dm0, dV, dW, dnu, partials, sc);
 }
 
 }  // namespace mfg

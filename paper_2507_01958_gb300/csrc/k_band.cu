@@ -392,6 +392,7 @@ template <typename TI, typename TO, typename T, bool FROM_BAND, bool TO_BAND>
 __global__ void __launch_bounds__(256) k_time_xf(const TI* __restrict__ in, TO* __restrict__ out,
                                                  const T* __restrict__ V, const int* __restrict__ ipos,
                                                  int nt, int S, const DevScalars* sc) {
+  dep_sync();
   if (sc != nullptr && sc->cg_done) return;
   extern __shared__ __align__(16) unsigned char smraw[];
   T* strip = reinterpret_cast<T*>(smraw);
@@ -495,6 +496,7 @@ template <typename T, bool BWD, int G>
 __global__ void __launch_bounds__(512, 1) k_band_pass(const T* __restrict__ rhs, T* __restrict__ sol,
                                                     const T* __restrict__ F, int S, int w, int stage,
                                                     DevScalars* sc) {
+  dep_sync();
   constexpr int RG = (kBandRing * G + 3) / 4 * 4;     // right-hand-side stages, 16-byte multiple
   if (sc != nullptr && sc->cg_done) return;
   // Fault-injection hook (MFG_INJECT_BAND_NO_COPY): no stage copy and no
@@ -614,7 +616,7 @@ void launch_band_pass(const BandShape& b, int nt, const T* in, T* out, const T* 
   DevScalars* scw = const_cast<DevScalars*>(sc);  // written only when a bounded wait runs out
   switch (b.G) {
 #define MFG_BAND_G(GG) \
-  case GG: k_band_pass<T, BWD, GG><<<nt, b.threads, b.smem, s>>>(in, out, F, S, w, b.stage, scw); break;
+  case GG: launch_k(k_band_pass<T, BWD, GG>, nt, b.threads, b.smem, s, in, out, F, S, w, b.stage, scw); break;
     MFG_BAND_G(32) MFG_BAND_G(16) MFG_BAND_G(8) MFG_BAND_G(4) MFG_BAND_G(2) MFG_BAND_G(1)
 #undef MFG_BAND_G
     default: break;
@@ -627,11 +629,11 @@ void precond_band_typed(const Geom& g, const PrecTables& t, const T* V, const T*
   const int S = g.S, nt = g.nt, w = t.band_w;
   const size_t tsm = sizeof(T) * (size_t)nt * 32;
   const int tb = (S + 31) / 32;
-  k_time_xf<double, T, T, false, true><<<tb, 256, tsm, s>>>(r, w0, V, t.band_perm, nt, S, sc);
+  launch_k(k_time_xf<double, T, T, false, true>, tb, 256, tsm, s, r, w0, V, t.band_perm, nt, S, sc);
   const BandShape b = band_shape<T>(w);
   launch_band_pass<T, false>(b, nt, w0, w1, Fc, S, w, sc, s);
   launch_band_pass<T, true>(b, nt, w1, w0, Fr, S, w, sc, s);
-  k_time_xf<T, double, T, true, false><<<tb, 256, tsm, s>>>(w0, z, V, t.band_perm, nt, S, sc);
+  launch_k(k_time_xf<T, double, T, true, false>, tb, 256, tsm, s, w0, z, V, t.band_perm, nt, S, sc);
 }
 
 template <typename T>

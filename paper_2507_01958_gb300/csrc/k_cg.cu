@@ -53,6 +53,7 @@ __device__ __forceinline__ bool aligned16(const void* a, const void* b = nullptr
 __global__ void __launch_bounds__(kThreads) k_init_p(long long n, const double* __restrict__ zp,
                                                      double* __restrict__ p, const double* __restrict__ r,
                                                      double* partials, DevScalars* sc) {
+  dep_sync();
   if (sc->cg_done) return;
   double acc = 0.0;
   const bool vec = aligned16(zp, p, r);
@@ -88,6 +89,7 @@ __global__ void __launch_bounds__(kThreads) k_update_zr(long long n, double* __r
                                                         double* __restrict__ r, const double* __restrict__ p,
                                                         const double* __restrict__ q, double* partials,
                                                         DevScalars* sc) {
+  dep_sync();
   if (sc->cg_done) return;
   const double alpha = sc->alpha;
   double acc = 0.0;
@@ -120,6 +122,7 @@ __global__ void __launch_bounds__(kThreads) k_dot_beta(long long n, const double
                                                        const double* __restrict__ zp,
                                                        const double* __restrict__ q, double* partials,
                                                        DevScalars* sc) {
+  dep_sync();
   if (sc->cg_done) return;
   double a0 = 0.0, a1 = 0.0;
   const bool vec = aligned16(r, zp, q);
@@ -145,6 +148,7 @@ __global__ void __launch_bounds__(kThreads) k_dot_beta(long long n, const double
 __global__ void __launch_bounds__(kThreads) k_update_p(long long n, const double* __restrict__ zp,
                                                        double* __restrict__ p, DevScalars* sc,
                                                        cudaGraphConditionalHandle h, int use_handle) {
+  dep_sync();
   const int done = sc->cg_done;
   if (use_handle && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(h, done ? 0u : 1u);
   if (done) return;
@@ -161,31 +165,32 @@ __global__ void __launch_bounds__(kThreads) k_update_p(long long n, const double
 
 void launch_init_p(long long n, const double* zp, double* p, const double* r, double* partials,
                    DevScalars* sc, cudaStream_t s, int cap) {
-  k_init_p<<<red_blocks(n, cap), kThreads, 0, s>>>(n, zp, p, r, partials, sc);
+  launch_k(k_init_p, red_blocks(n, cap), kThreads, 0, s, n, zp, p, r, partials, sc);
 }
 void launch_update_zr(long long n, double* z, double* r, const double* p, const double* q,
                       double* partials, DevScalars* sc, cudaStream_t s, int cap) {
-  k_update_zr<<<red_blocks(n, cap), kThreads, 0, s>>>(n, z, r, p, q, partials, sc);
+  launch_k(k_update_zr, red_blocks(n, cap), kThreads, 0, s, n, z, r, p, q, partials, sc);
 }
 void launch_dot_beta(long long n, const double* r, const double* zp, const double* q, int flexible,
                      double* partials, DevScalars* sc, cudaStream_t s, int cap) {
   if (flexible)
-    k_dot_beta<1><<<red_blocks(n, cap), kThreads, 0, s>>>(n, r, zp, q, partials, sc);
+    launch_k(k_dot_beta<1>, red_blocks(n, cap), kThreads, 0, s, n, r, zp, q, partials, sc);
   else
-    k_dot_beta<0><<<red_blocks(n, cap), kThreads, 0, s>>>(n, r, zp, q, partials, sc);
+    launch_k(k_dot_beta<0>, red_blocks(n, cap), kThreads, 0, s, n, r, zp, q, partials, sc);
 }
 void launch_update_p(long long n, const double* zp, double* p, DevScalars* sc,
                      cudaGraphConditionalHandle h, int use_handle, cudaStream_t s, int cap) {
-  k_update_p<<<red_blocks(n, cap), kThreads, 0, s>>>(n, zp, p, sc, h, use_handle);
+  launch_k(k_update_p, red_blocks(n, cap), kThreads, 0, s, n, zp, p, sc, h, use_handle);
 }
 
 // Start of a CP iteration inside the graph: arms the inner while-node.
 __global__ void k_scalars_begin(DevScalars* sc, cudaGraphConditionalHandle h, int use_handle) {
+  dep_sync();
   if (threadIdx.x == 0 && use_handle) cudaGraphSetConditional(h, sc->cg_done ? 0u : 1u);
 }
 void launch_scalars_begin(DevScalars* sc, cudaGraphConditionalHandle h, int use_handle,
                           cudaStream_t s) {
-  k_scalars_begin<<<1, 32, 0, s>>>(sc, h, use_handle);
+  launch_k(k_scalars_begin, 1, 32, 0, s, sc, h, use_handle);
 }
 
 }  // namespace mfg

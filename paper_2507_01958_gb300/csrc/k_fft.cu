@@ -62,6 +62,7 @@ __global__ void __launch_bounds__(256) k_fft(const TI* __restrict__ in, TO* __re
                                              const T* __restrict__ tw, const T* __restrict__ dct,
                                              long long inner, long long nlines, const DevScalars* sc,
                                              DotFuse df, ZrFuse zf) {
+  dep_sync();
   if (sc != nullptr && sc->cg_done) return;
   using Sh = FftShape<T, N>;
   constexpr int CL = Sh::CL, LB = Sh::LB, NP = Sh::NP;
@@ -371,7 +372,7 @@ static void launch_one(const TI* in, TO* out, const T* tw, const T* dct, long lo
                        DotFuse df = DotFuse{}, ZrFuse zf = ZrFuse{}) {
   using Sh = FftShape<T, N>;
   dim3 grid((unsigned)((nlines + Sh::LB - 1) / Sh::LB), CONTIG ? 1u : (unsigned)outer);
-  k_fft<T, N, MODE, CONTIG, TI, TO, DOT, ZR><<<grid, 256, Sh::smem, s>>>(in, out, tw, dct, inner, nlines, sc,
+  launch_k(k_fft<T, N, MODE, CONTIG, TI, TO, DOT, ZR>, grid, 256, Sh::smem, s, in, out, tw, dct, inner, nlines, sc,
                                                                          df, zf);
 }
 

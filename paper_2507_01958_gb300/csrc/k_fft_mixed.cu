@@ -15,6 +15,8 @@
 // leaves the pass bound by its shared-memory stages.  200 x 150 x 60, FP32: four
 // dense passes 300 us -> ~75 us together (P^{-1} 307 -> 87 us, its error against
 // 64 bits 4.8e-7 -> 1.7e-7); 8 is the shortest line that fills a stage.
+#include <cmath>
+
 #include "fft_common.cuh"
 #include "pcg_tail.cuh"
 #include "reduce.cuh"
@@ -22,7 +24,7 @@
 namespace mfg {
 namespace {
 
-constexpr int kMaxN = 2048, kMaxStages = 10, kBlock = 256;
+constexpr int kMaxN = 2048, kMaxStages = 10, kBlock = 256;  // kBlock: most threads per block
 
 // x / d for x * d < 2^32 (m = ceil(2^32 / d); d = 1 has m = 0).
 struct Div {
@@ -34,6 +36,7 @@ Div make_div(int d) { return Div{d == 1 ? 0u : (unsigned)(((1ull << 32) + d - 1)
 struct FftPlan {
   int N, stages, lines;  // lines: complex lines per block
   Div dN;
+  double r1, r2, rh;  // 1/sqrt(N), sqrt(2/N), 1/sqrt(2N): formed on the host, an FP64 root per thread is not free
   int radix[kMaxStages];
   Div dB[kMaxStages];   // by N / R, the butterflies of a line
   int Ns[kMaxStages];
@@ -156,7 +159,7 @@ __device__ __forceinline__ void dft(cx<T> (&a)[R], const cx<T>* w, int nb, T sgn
 template <typename T, int R>
 __device__ void stage(const cx<T>* src, cx<T>* dst, const cx<T>* tw, int N, int lines, int Ns, Div dB, Div dNs, T sgn) {
   const int nb = N / R, step = quot(nb, dNs);
-  for (int idx = threadIdx.x; idx < lines * nb; idx += kBlock) {
+  for (int idx = threadIdx.x; idx < lines * nb; idx += blockDim.x) {
     const int q = quot(idx, dB), j = idx - q * nb, b = quot(j, dNs), k = j - b * Ns;
     const cx<T>* sp = src + q * (N + 1) + j;
     cx<T> a[R];
@@ -210,15 +213,16 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 2 : 3) k_fft_mixed(co
                                                       const __grid_constant__ FftPlan P, int mode, int llb,
                                                       long long inner, long long nlines, const DevScalars* sc,
                                                       DotFuse df, ZrFuse zf) {
+  dep_sync();
   if (sc != nullptr && sc->cg_done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int N = P.N, NP = N + 1, CL = P.lines, LB = 2 * CL, tid = threadIdx.x;
+  const int N = P.N, NP = N + 1, CL = P.lines, LB = 2 * CL, tid = threadIdx.x, nth = blockDim.x;
   cx<T>* buf0 = reinterpret_cast<cx<T>*>(smem_raw);
   cx<T>* buf1 = buf0 + CL * NP;
   T* real1 = reinterpret_cast<T*>(buf1);  // [LB][NP] real staging
   cx<T>* tws = buf1 + CL * NP;
   cx<T>* dcs = tws + N;
-  for (int q = tid; q < N; q += kBlock) {
+  for (int q = tid; q < N; q += nth) {
     tws[q] = cx<T>{tw[2 * q], tw[2 * q + 1]};
     if (mode != FFT_DHT) dcs[q] = cx<T>{dct[2 * q], dct[2 * q + 1]};
   }
@@ -242,12 +246,12 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 2 : 3) k_fft_mixed(co
   const double alpha = ZR ? zf.sc->alpha : 0.0;
   // loads in batches, all of a batch issued before the first is used
   constexpr int BL = ZR ? 4 : 8;
-  for (int e0 = tid; e0 < total; e0 += kBlock * BL) {
+  for (int e0 = tid; e0 < total; e0 += nth * BL) {
     int ls[BL], is[BL];
     long long ad[BL];
     bool lv[BL];
 #pragma unroll
-    for (int u = 0; u < BL; ++u) lv[u] = element(e0 + kBlock * u, ls[u], is[u], ad[u]);
+    for (int u = 0; u < BL; ++u) lv[u] = element(e0 + nth * u, ls[u], is[u], ad[u]);
     if constexpr (ZR) {
       double zv[BL], pv[BL], rv[BL], qv[BL];
 #pragma unroll
@@ -265,7 +269,7 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 2 : 3) k_fft_mixed(co
           zf.r[ad[u]] = rn;
         }
         rr = fma(rn, rn, rr);
-        if (e0 + kBlock * u < total) put(ls[u], is[u], (T)rn);
+        if (e0 + nth * u < total) put(ls[u], is[u], (T)rn);
       }
     } else {
       T v[BL];
@@ -273,14 +277,14 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 2 : 3) k_fft_mixed(co
       for (int u = 0; u < BL; ++u) v[u] = lv[u] ? (T)in[ad[u]] : T(0);
 #pragma unroll
       for (int u = 0; u < BL; ++u)
-        if (e0 + kBlock * u < total) put(ls[u], is[u], v[u]);
+        if (e0 + nth * u < total) put(ls[u], is[u], v[u]);
     }
   }
   __syncthreads();
   if (mode == FFT_DCT3) {
     // exp(i th_k) (X_k - i X_{N-k}) with X = C/c, times 1/N of the inverse FFT
-    const T s0 = T(1) / sqrt(T(N)), s1 = T(1) / sqrt(T(2 * N));
-    for (int idx = tid; idx < CL * N; idx += kBlock) {
+    const T s0 = (T)P.r1, s1 = (T)P.rh;
+    for (int idx = tid; idx < CL * N; idx += nth) {
       const int q = quot(idx, P.dN), k = idx - q * N;
       const T* xa = real1 + (2 * q) * NP;
       const T* xb = xa + NP;
@@ -295,8 +299,8 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 2 : 3) k_fft_mixed(co
   const int odd = fft_stages<T>(P, mode == FFT_DCT3 ? T(1) : T(-1));
   const cx<T>* Z = odd ? buf1 : buf0;
   T* R = reinterpret_cast<T*>(odd ? buf0 : buf1);  // real outputs [LB][NP]
-  const T rsn = T(1) / sqrt(T(N)), rs2 = sqrt(T(2) / T(N));
-  for (int idx = tid; idx < CL * N; idx += kBlock) {
+  const T rsn = (T)P.r1, rs2 = (T)P.r2;
+  for (int idx = tid; idx < CL * N; idx += nth) {
     const int q = quot(idx, P.dN), k = idx - q * N;
     T* ra = R + (2 * q) * NP + k;
     if (mode == FFT_DCT3) {
@@ -320,14 +324,14 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 2 : 3) k_fft_mixed(co
   __syncthreads();
   double a0 = 0.0, a1 = 0.0;
   constexpr int BS = DOT ? 4 : 8;
-  for (int e0 = tid; e0 < total; e0 += kBlock * BS) {
+  for (int e0 = tid; e0 < total; e0 += nth * BS) {
     int ls[BS], is[BS];
     long long ad[BS];
     bool lv[BS];
     double dr[DOT ? BS : 1], dq[DOT ? BS : 1];
 #pragma unroll
     for (int u = 0; u < BS; ++u) {
-      lv[u] = element(e0 + kBlock * u, ls[u], is[u], ad[u]);
+      lv[u] = element(e0 + nth * u, ls[u], is[u], ad[u]);
       if constexpr (DOT) {
         dr[u] = lv[u] ? df.r[ad[u]] : 0.0;
         dq[u] = (lv[u] && df.flex) ? df.q[ad[u]] : 0.0;
@@ -357,6 +361,9 @@ void launch_mixed(int N, int mode, const TI* in, TO* out, const T* tw, const T* 
   P.N = N;
   P.stages = factor(N, P.radix);
   P.dN = make_div(N);
+  P.r1 = 1.0 / std::sqrt((double)N);
+  P.r2 = std::sqrt(2.0 / N);
+  P.rh = 1.0 / std::sqrt(2.0 * N);
   for (int i = 0, Ns = 1; i < P.stages; Ns *= P.radix[i], ++i) {
     P.dB[i] = make_div(N / P.radix[i]);
     P.Ns[i] = Ns;
@@ -370,9 +377,10 @@ void launch_mixed(int N, int mode, const TI* in, TO* out, const T* tw, const T* 
     --llb;
   }
   P.lines = lines;
+  int nth = kBlock;  // four elements of the complex lines per thread, at least two warps
+  while (nth > 64 && lines * N <= 2 * nth) nth >>= 1;
   const dim3 grid((unsigned)((nlines + 2 * lines - 1) / (2 * lines)), (unsigned)outer);
-  k_fft_mixed<T, TI, TO, CONTIG, DOT, ZR>
-      <<<grid, kBlock, smem_bytes<T>(N, lines), s>>>(in, out, tw, dct, P, mode, llb, inner, nlines, sc, df, zf);
+  launch_k(k_fft_mixed<T, TI, TO, CONTIG, DOT, ZR>, grid, nth, smem_bytes<T>(N, lines), s, in, out, tw, dct, P, mode, llb, inner, nlines, sc, df, zf);
 }
 
 template <typename T>

@@ -236,6 +236,7 @@ template <typename TI, typename T, typename TO, bool CONTIG>
 __global__ void __launch_bounds__(256) k_axis(const TI* __restrict__ in, TO* __restrict__ out,
                                               const T* __restrict__ M, int N, long long inner,
                                               long long ncols, int trans, const DevScalars* sc) {
+  dep_sync();
   if (sc != nullptr && sc->cg_done) return;
   __shared__ T As[BK][BM + 1];
   __shared__ T Bs[BK][BN + 1];
@@ -312,9 +313,9 @@ static void axis_pass(const TI* in, TO* out, const T* M, int N, long long inner,
   const long long ncols = inner * outer;
   dim3 grid((unsigned)((ncols + BN - 1) / BN), (N + BM - 1) / BM);
   if (inner == 1)
-    k_axis<TI, T, TO, true><<<grid, 256, 0, s>>>(in, out, M, N, inner, ncols, trans, sc);
+    launch_k(k_axis<TI, T, TO, true>, grid, 256, 0, s, in, out, M, N, inner, ncols, trans, sc);
   else
-    k_axis<TI, T, TO, false><<<grid, 256, 0, s>>>(in, out, M, N, inner, ncols, trans, sc);
+    launch_k(k_axis<TI, T, TO, false>, grid, 256, 0, s, in, out, M, N, inner, ncols, trans, sc);
 }
 
 // ------------------------------------------------------------ time pass --
@@ -366,6 +367,7 @@ template <typename T>
 __global__ void __launch_bounds__(128) k_time_tri(const T* __restrict__ in, T* __restrict__ out,
                                                   const T* __restrict__ L1, const T* __restrict__ L2, int l,
                                                   int nt, int S, const DevScalars* sc) {
+  dep_sync();
   if (sc != nullptr && sc->cg_done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int bd = blockDim.x, s = blockIdx.x * bd + threadIdx.x;
@@ -437,7 +439,7 @@ template <typename T>
 static void time_pass(const T* in, T* out, const T* L1, const T* L2, int l, int nt, int S, const DevScalars* sc,
                       cudaStream_t s) {
   const int bd = tri_threads<T>(nt, S);
-  k_time_tri<T><<<(S + bd - 1) / bd, bd, 2 * sizeof(T) * (size_t)nt * bd, s>>>(in, out, L1, L2, l, nt, S, sc);
+  launch_k(k_time_tri<T>, (S + bd - 1) / bd, bd, 2 * sizeof(T) * (size_t)nt * bd, s, in, out, L1, L2, l, nt, S, sc);
 }
 
 // Exact time solve of the l = 0 variant: per spatial mode s, the tridiagonal
@@ -449,6 +451,7 @@ __global__ void __launch_bounds__(256) k_thomas(const T* __restrict__ in, T* __r
                                                 const T* __restrict__ cf, const T* __restrict__ idn,
                                                 const T* __restrict__ off, int nt, int S,
                                                 const DevScalars* sc) {
+  dep_sync();
   if (sc != nullptr && sc->cg_done) return;
   for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < S; s += gridDim.x * blockDim.x) {
     const T o = off[s];
@@ -496,7 +499,7 @@ static void precond_typed(const Geom& g, const T* Hx, const T* Hy, const T* V, c
     T* t = a; a = b; b = t;
   }
   if (thc != nullptr) {
-    k_thomas<T><<<(int)((S + 255) / 256), 256, 0, s>>>(a, b, thc, thd, tho, g.nt, (int)S, sc);
+    launch_k(k_thomas<T>, (int)((S + 255) / 256), 256, 0, s, a, b, thc, thd, tho, g.nt, (int)S, sc);
   } else if constexpr (sizeof(T) == 4) {
     if (tc && !g.time_simt && time_tc_supported(g.nt))
       launch_time_tc(a, b, V, lamt, L1, L2, g.nt, (int)S, sc, s);

@@ -363,6 +363,7 @@ __global__ void __launch_bounds__(kThreads) k_prox_cp(Geom g, Coef cf, const dou
                                                       DevScalars* sc, cudaGraphConditionalHandle h,
                                                       int use_handle, double* __restrict__ Az,
                                                       const double* __restrict__ rfin) {
+  dep_sync();
   constexpr int NW = ACTX ? 4 : 2;
   const long long n = g.n;
   const double tau = sc->tau, theta = sc->theta;
@@ -465,6 +466,7 @@ __global__ void __launch_bounds__(kThreads) k_prox_plain(Geom g, Coef cf, double
                                                          const double* v, double* y,
                                                          const double* __restrict__ V,
                                                          const double* __restrict__ W) {
+  dep_sync();
   constexpr int NW = ACTX ? 4 : 2;
   const long long n = g.n;
   const ProxK K = prox_consts(tau, 0.5 / tau, cf.f_b);
@@ -524,7 +526,7 @@ void launch_prox_cp(const Geom& g, const Coef& cf, const double* z, double* y, d
   // the general-q' root finder and the viscosity field are their own
   // instantiations, so the q' = 2, constant-nu kernel keeps its registers
 #define MFG_PROX_CP(A, Q, N) \
-  k_prox_cp<A, Q, N><<<nb, kThreads, 0, s>>>(g, cf, z, y, ybar, V, W, partials, sc, h, use_handle, Az, rfin)
+  launch_k(k_prox_cp<A, Q, N>, nb, kThreads, 0, s, g, cf, z, y, ybar, V, W, partials, sc, h, use_handle, Az, rfin)
   const bool gq = cf.qprime != 2.0, vn = g.kfy != nullptr;
   if (g.actx) {
     if (gq) { if (vn) MFG_PROX_CP(1, true, true); else MFG_PROX_CP(1, true, false); }
@@ -541,13 +543,13 @@ void launch_prox_plain(const Geom& g, const Coef& cf, double tau, const double* 
   const int nb = red_blocks(g.n, g.vec_blocks);
   if (cf.qprime != 2.0) {
     if (g.actx)
-      k_prox_plain<1, true><<<nb, kThreads, 0, s>>>(g, cf, tau, v, y, V, W);
+      launch_k(k_prox_plain<1, true>, nb, kThreads, 0, s, g, cf, tau, v, y, V, W);
     else
-      k_prox_plain<0, true><<<nb, kThreads, 0, s>>>(g, cf, tau, v, y, V, W);
+      launch_k(k_prox_plain<0, true>, nb, kThreads, 0, s, g, cf, tau, v, y, V, W);
   } else if (g.actx) {
-    k_prox_plain<1, false><<<nb, kThreads, 0, s>>>(g, cf, tau, v, y, V, W);
+    launch_k(k_prox_plain<1, false>, nb, kThreads, 0, s, g, cf, tau, v, y, V, W);
   } else {
-    k_prox_plain<0, false><<<nb, kThreads, 0, s>>>(g, cf, tau, v, y, V, W);
+    launch_k(k_prox_plain<0, false>, nb, kThreads, 0, s, g, cf, tau, v, y, V, W);
   }
 }
 

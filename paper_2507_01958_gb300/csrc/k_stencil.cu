@@ -102,6 +102,7 @@ __global__ void __launch_bounds__(256, kCPerSm) k_apply_C(Geom g, StripGrid sg, 
                                                     double* __restrict__ r, double alpha,
                                                     const double* __restrict__ m0, const double* __restrict__ pdot,
                                                     double* partials, DevScalars* sc, double* __restrict__ Az) {
+  dep_sync();
   if (MODE == 2 && sc->cg_done) return;
   if (MODE == 1) alpha = sc->sigma;
   double acc = 0.0, accb = 0.0;
@@ -187,6 +188,7 @@ __global__ void __launch_bounds__(kThreads) k_apply_C_flat(Geom g, const double*
                                                       const double* __restrict__ pdot,
                                                       double* partials, DevScalars* sc, int mode,
                                                       double* __restrict__ Az) {
+  dep_sync();
   if (mode == 2 && sc->cg_done) return;
   if (mode == 1) alpha = sc->sigma;
   const long long n = g.n;
@@ -259,7 +261,7 @@ void launch_apply_C(const Geom& g, const double* v, double* r, double alpha, con
                     double* Az) {
   if (!strips_fit(g)) {
     const int nb = red_blocks(g.n, g.vec_blocks);
-#define MFG_C_FLAT(A, N) k_apply_C_flat<A, N><<<nb, kThreads, 0, s>>>(g, v, r, alpha, m0, pdot, partials, sc, mode, Az)
+#define MFG_C_FLAT(A, N) launch_k(k_apply_C_flat<A, N>, nb, kThreads, 0, s, g, v, r, alpha, m0, pdot, partials, sc, mode, Az)
     if (g.kfy != nullptr) { if (g.actx) MFG_C_FLAT(1, true); else MFG_C_FLAT(0, true); }
     else                  { if (g.actx) MFG_C_FLAT(1, false); else MFG_C_FLAT(0, false); }
 #undef MFG_C_FLAT
@@ -267,7 +269,7 @@ void launch_apply_C(const Geom& g, const double* v, double* r, double alpha, con
   }
   const StripGrid sg = strip_grid(g, kCPerSm);
 #define MFG_C(A, I, M) \
-  k_apply_C<A, I, M><<<sg.blocks, 32 * sg.warps, 0, s>>>(g, sg, v, r, alpha, m0, pdot, partials, sc, Az)
+  launch_k(k_apply_C<A, I, M>, sg.blocks, 32 * sg.warps, 0, s, g, sg, v, r, alpha, m0, pdot, partials, sc, Az)
 #define MFG_C_MODE(A, I)       \
   switch (mode) {              \
     case 0: MFG_C(A, I, 0); break; \
@@ -293,6 +295,7 @@ void launch_apply_C(const Geom& g, const double* v, double* r, double alpha, con
 template <int ACTX>
 __global__ void __launch_bounds__(256, kCtPerSm) k_apply_Ct(Geom g, StripGrid sg, const double* __restrict__ p,
                                                      double* __restrict__ x) {
+  dep_sync();
   int j0, i0, i1, k;
   if (!strip_item(sg, g, j0, i0, i1, k)) return;
   const long long n = g.n, base = (long long)k * g.S;
@@ -329,6 +332,7 @@ __global__ void __launch_bounds__(256, kCtPerSm) k_apply_Ct(Geom g, StripGrid sg
 template <int ACTX, bool VN>
 __global__ void __launch_bounds__(kThreads) k_apply_Ct_flat(Geom g, const double* __restrict__ p,
                                                        double* __restrict__ x) {
+  dep_sync();
   const long long n = g.n;
   double* xm = x;
   double* xx1 = x + n;
@@ -369,7 +373,7 @@ __global__ void __launch_bounds__(kThreads) k_apply_Ct_flat(Geom g, const double
 void launch_apply_Ct(const Geom& g, const double* p, double* x, cudaStream_t s) {
   if (!strips_fit(g)) {
     const int nb = red_blocks(g.n, g.vec_blocks);
-#define MFG_CT_FLAT(A, N) k_apply_Ct_flat<A, N><<<nb, kThreads, 0, s>>>(g, p, x)
+#define MFG_CT_FLAT(A, N) launch_k(k_apply_Ct_flat<A, N>, nb, kThreads, 0, s, g, p, x)
     if (g.kfy != nullptr) { if (g.actx) MFG_CT_FLAT(1, true); else MFG_CT_FLAT(0, true); }
     else                  { if (g.actx) MFG_CT_FLAT(1, false); else MFG_CT_FLAT(0, false); }
 #undef MFG_CT_FLAT
@@ -377,9 +381,9 @@ void launch_apply_Ct(const Geom& g, const double* p, double* x, cudaStream_t s) 
   }
   const StripGrid sg = strip_grid(g, kCtPerSm);
   if (g.actx)
-    k_apply_Ct<1><<<sg.blocks, 32 * sg.warps, 0, s>>>(g, sg, p, x);
+    launch_k(k_apply_Ct<1>, sg.blocks, 32 * sg.warps, 0, s, g, sg, p, x);
   else
-    k_apply_Ct<0><<<sg.blocks, 32 * sg.warps, 0, s>>>(g, sg, p, x);
+    launch_k(k_apply_Ct<0>, sg.blocks, 32 * sg.warps, 0, s, g, sg, p, x);
 }
 
 // ---------------------------------------------------------------- C C^T p --
@@ -424,6 +428,7 @@ template <bool ISO>
 __global__ void __launch_bounds__(256, kUPerSm) k_aat_u(Geom g, AatCoef a, StripGrid ag, const double* __restrict__ p,
                                                double* __restrict__ U, double* __restrict__ Sx,
                                                const DevScalars* sc, int mode) {
+  dep_sync();
   if (mode != 0 && sc->cg_done) return;
   int j0, i0, i1, k;
   if (!strip_item(ag, g, j0, i0, i1, k)) return;
@@ -446,6 +451,7 @@ template <bool ISO, bool STEP>
 __global__ void __launch_bounds__(256, kQPerSm) k_aat_q2(Geom g, AatCoef a, StripGrid ag, const double* __restrict__ U,
                                                    const double* __restrict__ Sx, const double* __restrict__ p,
                                                    double* __restrict__ q, double* partials, DevScalars* sc) {
+  dep_sync();
   if (STEP && sc->cg_done) return;
   double acc = 0.0;
   int j0, i0, i1, k;
@@ -530,6 +536,7 @@ template <int ACTX>
 __global__ void __launch_bounds__(AJ * AI) k_aat_x(Geom g, AatCoef a, int kc, const double* __restrict__ p,
                                                    double* __restrict__ X, double* __restrict__ KP,
                                                    const DevScalars* sc, int mode) {
+  dep_sync();
   if (mode != 0 && sc->cg_done) return;
   const int j = blockIdx.x * AJ + threadIdx.x, i = blockIdx.y * AI + threadIdx.y;
   if (i >= g.nx || j >= g.ny) return;
@@ -564,6 +571,7 @@ __global__ void __launch_bounds__(AJ * AI, 3) k_aat_q(Geom g, AatCoef a, int kc,
                                                    const double* __restrict__ KP, const double* __restrict__ p,
                                                    double* __restrict__ q, double* partials, DevScalars* sc,
                                                    int mode) {
+  dep_sync();
   if (mode != 0 && sc->cg_done) return;
   const int j = blockIdx.x * AJ + threadIdx.x, i = blockIdx.y * AI + threadIdx.y;
   double acc = 0.0;
@@ -612,6 +620,7 @@ template <int ACTX>
 __global__ void __launch_bounds__(AJ * AI) k_aat_x_df(Geom g, AatCoef ad, int kc, const double* __restrict__ p,
                                                       df* __restrict__ X, df* __restrict__ KP,
                                                       const DevScalars* sc, int mode) {
+  dep_sync();
   if (mode != 0 && sc->cg_done) return;
   const int j = blockIdx.x * AJ + threadIdx.x, i = blockIdx.y * AI + threadIdx.y;
   if (i >= g.nx || j >= g.ny) return;
@@ -641,6 +650,7 @@ __global__ void __launch_bounds__(AJ * AI) k_aat_q_df(Geom g, AatCoef ad, int kc
                                                       const df* __restrict__ KP, const double* __restrict__ p,
                                                       double* __restrict__ q, double* partials, DevScalars* sc,
                                                       int mode) {
+  dep_sync();
   if (mode != 0 && sc->cg_done) return;
   const int j = blockIdx.x * AJ + threadIdx.x, i = blockIdx.y * AI + threadIdx.y;
   double acc = 0.0;
@@ -679,11 +689,11 @@ void launch_AAt(const Geom& g, const double* p, double* q, double* scratch, doub
     df* X = reinterpret_cast<df*>(scratch);
     df* KP = X + g.n;
     if (g.actx) {
-      k_aat_x_df<1><<<grid, block, 0, s>>>(g, a, kc, p, X, KP, sc, mode);
-      k_aat_q_df<1><<<grid, block, 0, s>>>(g, a, kc, X, KP, p, q, partials, sc, mode);
+      launch_k(k_aat_x_df<1>, grid, block, 0, s, g, a, kc, p, X, KP, sc, mode);
+      launch_k(k_aat_q_df<1>, grid, block, 0, s, g, a, kc, X, KP, p, q, partials, sc, mode);
     } else {
-      k_aat_x_df<0><<<grid, block, 0, s>>>(g, a, kc, p, X, KP, sc, mode);
-      k_aat_q_df<0><<<grid, block, 0, s>>>(g, a, kc, X, KP, p, q, partials, sc, mode);
+      launch_k(k_aat_x_df<0>, grid, block, 0, s, g, a, kc, p, X, KP, sc, mode);
+      launch_k(k_aat_q_df<0>, grid, block, 0, s, g, a, kc, X, KP, p, q, partials, sc, mode);
     }
     return;
   }
@@ -691,22 +701,22 @@ void launch_AAt(const Geom& g, const double* p, double* q, double* scratch, doub
   double* KP = scratch + g.n;  // s, or K p
   if (g.kfy != nullptr) {
     if (g.actx) {
-      k_aat_x<1><<<grid, block, 0, s>>>(g, a, kc, p, X, KP, sc, mode);
-      k_aat_q<1><<<grid, block, 0, s>>>(g, a, kc, X, KP, p, q, partials, sc, mode);
+      launch_k(k_aat_x<1>, grid, block, 0, s, g, a, kc, p, X, KP, sc, mode);
+      launch_k(k_aat_q<1>, grid, block, 0, s, g, a, kc, X, KP, p, q, partials, sc, mode);
     } else {
-      k_aat_x<0><<<grid, block, 0, s>>>(g, a, kc, p, X, KP, sc, mode);
-      k_aat_q<0><<<grid, block, 0, s>>>(g, a, kc, X, KP, p, q, partials, sc, mode);
+      launch_k(k_aat_x<0>, grid, block, 0, s, g, a, kc, p, X, KP, sc, mode);
+      launch_k(k_aat_q<0>, grid, block, 0, s, g, a, kc, X, KP, p, q, partials, sc, mode);
     }
     return;
   }
   const StripGrid ug = strip_grid(g, kUPerSm), ag = strip_grid(g, kQPerSm);
   const int nth = 32 * ag.warps;
   const bool iso = g.actx && g.ax == g.ay, step = mode != 0;
-#define MFG_AAT(I, ST) k_aat_q2<I, ST><<<ag.blocks, nth, 0, s>>>(g, a, ag, X, KP, p, q, partials, sc)
+#define MFG_AAT(I, ST) launch_k(k_aat_q2<I, ST>, ag.blocks, nth, 0, s, g, a, ag, X, KP, p, q, partials, sc)
   if (iso)
-    k_aat_u<true><<<ug.blocks, 32 * ug.warps, 0, s>>>(g, a, ug, p, X, KP, sc, mode);
+    launch_k(k_aat_u<true>, ug.blocks, 32 * ug.warps, 0, s, g, a, ug, p, X, KP, sc, mode);
   else
-    k_aat_u<false><<<ug.blocks, 32 * ug.warps, 0, s>>>(g, a, ug, p, X, KP, sc, mode);
+    launch_k(k_aat_u<false>, ug.blocks, 32 * ug.warps, 0, s, g, a, ug, p, X, KP, sc, mode);
   if (iso) { if (step) MFG_AAT(true, true); else MFG_AAT(true, false); }
   else     { if (step) MFG_AAT(false, true); else MFG_AAT(false, false); }
 #undef MFG_AAT

@@ -136,6 +136,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     k_time_tc(const float* __restrict__ in, float* __restrict__ out, const float* __restrict__ V,
               const float* __restrict__ lamt, const float* __restrict__ L1, const float* __restrict__ L2,
               int S, DevScalars* sc) {
+  dep_sync();
   if (sc != nullptr && sc->cg_done) return;
   // Fault-injection hook (MFG_INJECT_TC_NO_COMMIT): the elected thread issues
   // neither the MMAs nor their commit, so no tensor-core work is ever in flight
@@ -359,7 +360,7 @@ void launch_tc(const float* in, float* out, const float* V, const float* lamt, c
   const int per_sm = g_tc_blocks_per_sm[NT == 32 ? 0 : (NT == 64 ? 1 : 2)];
   const int cap = 152 * per_sm;  // one wave of resident blocks; each walks strips
   const int blocks = nstrips < cap ? nstrips : cap;
-  k_time_tc<NT><<<blocks, kTcThreads, TcShape<NT>::smem, s>>>(in, out, V, lamt, L1, L2, S, sc);
+  launch_k(k_time_tc<NT>, blocks, kTcThreads, TcShape<NT>::smem, s, in, out, V, lamt, L1, L2, S, sc);
 }
 
 }  // namespace

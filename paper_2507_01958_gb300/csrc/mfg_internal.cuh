@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <cstdint>
 #include <string>
+#include <utility>
 
 #include "../../include/mfg.h"
 
@@ -88,6 +89,34 @@ int set_error(int code, const std::string& msg);
 inline int red_blocks(long long n, int cap = kRedBlocks) {
   long long b = (n + kThreads - 1) / kThreads;
   return (int)(b < cap ? (b > 0 ? b : 1) : cap);
+}
+
+// Kernel launches.  A solve is a chain of short kernels on one stream (or graph
+// branch), so every launch is allowed to be set up while its predecessor ends
+// (programmatic dependent launch): its blocks wait in dep_sync, the first statement
+// of every kernel, until the predecessor's work is complete and visible; nothing is
+// read or written before it.  No kernel triggers its successor early: blocks of the
+// next grid resident beside the last wave spread it unevenly over the SMs (the 512^2 x
+// 128 solve 139 -> 144 ms with a trigger at the start, 140 without; C, C^T and AAt on
+// 200 x 33 x 31 45 us launched plainly, 56 with, 38 without).  P^{-1} 200 x 150 x 60: 87 -> 77
+// us, the 128^2 x 64 adjoint 5.6 -> 5.1 ms; inside the solve's graph no difference.
+__device__ __forceinline__ void dep_sync() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <typename... KA, typename... A>
+void launch_k(void (*kernel)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, kernel, std::forward<A>(args)...);
 }
 
 // ---------------------------------------------------------------- kernels --

@@ -33,9 +33,9 @@ constexpr size_t kNaWork = 2 * (size_t)kNaMaxN;
 constexpr size_t kNaH = (size_t)kNaMaxAxis * kNaMaxAxis;
 constexpr size_t kNaV = (size_t)kNaMaxNt * kNaMaxNt;
 constexpr size_t kNaS = (size_t)kNaMaxAxis * kNaMaxAxis;
-// FFT twiddles of a power-of-two axis: N/2 complex (cos, sin)(2 pi m/N) and N
-// complex (cos, sin)(pi k/(2N)), i.e. 3N values per axis
-constexpr size_t kNaTw = 3 * (size_t)kNaMaxAxis;
+// FFT twiddles of an axis: N complex (cos, sin)(2 pi m/N) and N complex
+// (cos, sin)(pi k/(2N)), i.e. 4N values per axis
+constexpr size_t kNaTw = 4 * (size_t)kNaMaxAxis;
 constexpr size_t kNaDoubles = kNaWork + 2 * kNaH + kNaV + kNaMaxNt + 2 * kNaS + 2 * kNaTw;  // 6.4 MB
 
 __device__ __align__(256) double g_noalloc_scratch[kNaDoubles];
@@ -51,16 +51,16 @@ __device__ double axis_lambda(int a, int N, int per) {
   return 2.0 - 2.0 * cospi((per ? 2.0 : 1.0) * a / N);
 }
 
-// Twiddles of the FFT spatial passes for a power-of-two axis of length N
-// (same definitions as the plan's): tw[m] = (cos, sin)(2 pi m/N), m < N/2;
+// Twiddles of the FFT spatial passes for an axis of length N (same definitions as
+// the plan's): tw[m] = (cos, sin)(2 pi m/N), m < N;
 // dct[k] = (cos, sin)(pi k/(2N)), k < N; interleaved (cos, sin) pairs.
 template <typename T>
 __device__ void fft_twiddle(long long q, int N, T* tw, T* dct) {
-  if (q < N) {
+  if (q < 2 * N) {
     const int m = (int)(q >> 1);
     tw[q] = (T)((q & 1) ? sinpi(2.0 * m / N) : cospi(2.0 * m / N));
   } else {
-    q -= N;
+    q -= 2 * N;
     const int k = (int)(q >> 1);
     dct[q] = (T)((q & 1) ? sinpi(k / (2.0 * N)) : cospi(k / (2.0 * N)));
   }
@@ -68,14 +68,15 @@ __device__ void fft_twiddle(long long q, int N, T* tw, T* dct) {
 
 // Fills the tables of eq. pstrec (same definitions as the plan's host tables:
 // Hartley / DCT-II in space, DCT-VIII / DST-I in time, Lambda_1, Lambda_2, and
-// the FFT twiddles of power-of-two axes; twx/twy null otherwise), evaluated on
+// the FFT twiddles of axes with an FFT pass; twx/twy null otherwise), evaluated on
 // the device with cospi/sinpi.
 template <typename T>
 __global__ void k_noalloc_tables(Geom g, int l, T* Hx, T* Hy, T* V, T* lamt, T* L1, T* L2, T* twx, T* dctx,
                                  T* twy, T* dcty) {
+  dep_sync();
   const long long nHx = (long long)g.nx * g.nx, nHy = (long long)g.ny * g.ny;
   const long long nV = (long long)g.nt * g.nt;
-  const long long nTx = twx ? 3LL * g.nx : 0, nTy = twy ? 3LL * g.ny : 0;
+  const long long nTx = twx ? 4LL * g.nx : 0, nTy = twy ? 4LL * g.ny : 0;
   const long long total = nHx + nHy + nV + g.nt + g.S + nTx + nTy;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
        e += (long long)gridDim.x * blockDim.x) {
@@ -141,9 +142,9 @@ void carve(double* base, const Geom& g, int l, PrecTables* t, T** w0) {
   T* lamt = p; p += kNaMaxNt;
   T* L1 = p; p += kNaS;
   T* L2 = p; p += kNaS;
-  T* twx = p; T* dctx = p + kNaMaxAxis; p += kNaTw;
-  T* twy = p; T* dcty = p + kNaMaxAxis;
-  const bool fx = g.nx > 1 && fft_pow2(g.nx), fy = fft_pow2(g.ny);
+  T* twx = p; T* dctx = p + 2 * kNaMaxAxis; p += kNaTw;
+  T* twy = p; T* dcty = p + 2 * kNaMaxAxis;
+  const bool fx = g.nx > 1 && fft_supported(g.nx), fy = fft_supported(g.ny);
   if (!fx) twx = dctx = nullptr;
   if (!fy) twy = dcty = nullptr;
   if constexpr (sizeof(T) == 8) {
@@ -198,7 +199,7 @@ extern "C" int mfg_apply_precond_noalloc(const mfg_problem* p, const double* r, 
   cudaStream_t s = (cudaStream_t)stream;
   PrecTables t{};
   const long long ntab = (long long)g.nx * g.nx + (long long)g.ny * g.ny + (long long)g.nt * g.nt + g.nt + g.S +
-                         3LL * (g.nx + g.ny);
+                         4LL * (g.nx + g.ny);
   const int nb = (int)std::min<long long>((ntab + kThreads - 1) / kThreads, 1024);
   if (p->precision != MFG_FP64) {
     // FP32 transforms; MFG_MIXED_TC takes the tensor-core time pass as in the
@@ -206,13 +207,13 @@ extern "C" int mfg_apply_precond_noalloc(const mfg_problem* p, const double* r, 
     // runs as MFG_MIXED
     float* w0 = nullptr;
     carve<float>(base, g, p->l, &t, &w0);
-    k_noalloc_tables<float><<<nb, kThreads, 0, s>>>(g, p->l, t.Hx32, t.Hy32, t.Vt32, t.lamt32, t.L1_32, t.L2_32,
+    launch_k(k_noalloc_tables<float>, nb, kThreads, 0, s, g, p->l, t.Hx32, t.Hy32, t.Vt32, t.lamt32, t.L1_32, t.L2_32,
                                                      t.twx32, t.dctx32, t.twy32, t.dcty32);
     launch_precond(g, t, p->precision == MFG_MIXED_TC ? MFG_MIXED_TC : MFG_MIXED, r, z, nullptr, w0, nullptr, s);
   } else {
     double* w0 = nullptr;
     carve<double>(base, g, p->l, &t, &w0);
-    k_noalloc_tables<double><<<nb, kThreads, 0, s>>>(g, p->l, t.Hx64, t.Hy64, t.Vt64, t.lamt64, t.L1_64,
+    launch_k(k_noalloc_tables<double>, nb, kThreads, 0, s, g, p->l, t.Hx64, t.Hy64, t.Vt64, t.lamt64, t.L1_64,
                                                       t.L2_64, t.twx64, t.dctx64, t.twy64, t.dcty64);
     launch_precond(g, t, MFG_FP64, r, z, w0, nullptr, nullptr, s);
   }
