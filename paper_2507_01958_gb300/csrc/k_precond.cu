@@ -99,6 +99,8 @@ static T* upload(const std::vector<double>& h, std::string* err) {
   return d;
 }
 
+__global__ void k_tri_table(double* G, const double* L1, const double* L2, int l, int nt, int S);
+
 int build_prec_tables(const mfg_problem& p, const Geom& g, PrecTables* t, std::string* err) {
   *t = PrecTables{};
   t->nx = g.nx;
@@ -205,6 +207,19 @@ int build_prec_tables(const mfg_problem& p, const Geom& g, PrecTables* t, std::s
     free_prec_tables(t);
     return MFG_ERR_CUDA;
   }
+  if (p.precision == MFG_FP64 && p.l != 0 && p.nu_field == nullptr) {
+    if (cudaMalloc(&t->tri64, sizeof(double) * (size_t)g.n) != cudaSuccess) {
+      *err = "cudaMalloc failed for the time elimination's factors";
+      free_prec_tables(t);
+      return MFG_ERR_CUDA;
+    }
+    launch_k(k_tri_table, (g.S + 127) / 128, 128, 0, (cudaStream_t) nullptr, t->tri64, t->L1_64, t->L2_64, p.l, g.nt, g.S);
+    if (cudaStreamSynchronize(nullptr) != cudaSuccess) {
+      *err = "building the time elimination's factors failed";
+      free_prec_tables(t);
+      return MFG_ERR_CUDA;
+    }
+  }
   if (p.nu_field != nullptr) {
     const int rc = build_band_tables(p, g, lt.data(), t, err);
     if (rc != MFG_OK) {
@@ -219,7 +234,7 @@ void free_prec_tables(PrecTables* t) {
   void* ptrs[] = {t->Hx64, t->Hy64, t->Vt64, t->lamt64, t->L1_64, t->L2_64, t->Hx32, t->Hy32,
                   t->Vt32, t->lamt32, t->L1_32, t->L2_32, t->twx64, t->twx32, t->dctx64, t->dctx32,
                   t->twy64, t->twy32, t->dcty64, t->dcty32, t->thc64, t->thd64, t->tho64,
-                  t->thc32, t->thd32, t->tho32, t->kfx, t->kfy, t->band_perm, t->bandc64,
+                  t->thc32, t->thd32, t->tho32, t->tri64, t->kfx, t->kfy, t->band_perm, t->bandc64,
                   t->bandr64, t->bandc32, t->bandr32};
   for (void* q : ptrs)
     if (q) cudaFree(q);
@@ -339,7 +354,7 @@ static void axis_pass(const TI* in, TO* out, const T* M, int N, long long inner,
 // thread reads another's column, so nothing synchronises.  512^2 x 128 FP32:
 // 169 us (dense products on the tensor cores) -> 64 us, with a tenth of the
 // apply's error (3e-6 -> 3e-7 against 64 bits); 256^2 x 64 FP64: 973 us (dense
-// products on the CUDA cores) -> ~105 us.
+// products on the CUDA cores) -> 41 us with the plan's g_k.
 template <typename T>
 __device__ __forceinline__ void cp_async_elem(T* smem, const T* gmem) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
@@ -363,10 +378,30 @@ __device__ __forceinline__ double recip(double x) {
   return fma(y, fma(e, e, e), y);
 }
 
-template <typename T>
+// The g_k of every mode, [nt][S]: FP64 plans keep them (8 bytes per element read
+// instead of 6 of the 9 FP64 instructions; in FP32 they cost less than their bytes).
+// P^{-1} 256^2 x 64 740 -> 678 us; the 64-point 1-D solve 7.9 -> 6.9 ms, where the g_k
+// were a serial chain in front of every pass.
+__global__ void __launch_bounds__(128) k_tri_table(double* __restrict__ G, const double* __restrict__ L1,
+                                                   const double* __restrict__ L2, int l, int nt, int S) {
+  dep_sync();
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= S) return;
+  const double rho = L1[s] / L2[s];
+  double d = (double)(l - 1) + rho;
+  for (int k = 0;; ++k) {
+    const double g = recip(1.0 + d);
+    G[(long long)k * S + s] = g;
+    if (k + 1 == nt) break;
+    d = fma(d, g, rho);
+  }
+}
+
+template <typename T, bool TAB>
 __global__ void __launch_bounds__(128) k_time_tri(const T* __restrict__ in, T* __restrict__ out,
-                                                  const T* __restrict__ L1, const T* __restrict__ L2, int l,
-                                                  int nt, int S, const DevScalars* sc) {
+                                                  const T* __restrict__ L1, const T* __restrict__ L2,
+                                                  const T* __restrict__ tab, int l, int nt, int S,
+                                                  const DevScalars* sc) {
   dep_sync();
   if (sc != nullptr && sc->cg_done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -376,16 +411,24 @@ __global__ void __launch_bounds__(128) k_time_tri(const T* __restrict__ in, T* _
   if (s >= S) return;
   const T* src = in + s;
 #pragma unroll 8
-  for (int k = 0; k < nt; ++k) cp_async_elem(E + k * bd, src + (long long)k * S);
+  for (int k = 0; k < nt; ++k) {
+    cp_async_elem(E + k * bd, src + (long long)k * S);
+    if constexpr (TAB) cp_async_elem(G + k * bd, tab + (long long)k * S + s);
+  }
   asm volatile("cp.async.commit_group;\n" ::: "memory");
-  const T l2 = L2[s], rho = L1[s] / l2, il2 = T(1) / l2;
-  T d = T(l - 1) + rho, g = recip(T(1) + d);
-  G[0] = g;
-#pragma unroll 4
-  for (int k = 1; k < nt; ++k) {
-    d = fma(d, g, rho);
+  const T l2 = L2[s], il2 = T(1) / l2;
+  T g;
+  if constexpr (!TAB) {
+    const T rho = L1[s] / l2;
+    T d = T(l - 1) + rho;
     g = recip(T(1) + d);
-    G[k * bd] = g;
+    G[0] = g;
+#pragma unroll 4
+    for (int k = 1; k < nt; ++k) {
+      d = fma(d, g, rho);
+      g = recip(T(1) + d);
+      G[k * bd] = g;
+    }
   }
   asm volatile("cp.async.wait_group 0;\n" ::: "memory");
   // eight steps at a time: their shared loads are issued together, ahead of
@@ -436,10 +479,14 @@ static int tri_threads(int nt, int S) {
 }
 
 template <typename T>
-static void time_pass(const T* in, T* out, const T* L1, const T* L2, int l, int nt, int S, const DevScalars* sc,
-                      cudaStream_t s) {
-  const int bd = tri_threads<T>(nt, S);
-  launch_k(k_time_tri<T>, (S + bd - 1) / bd, bd, 2 * sizeof(T) * (size_t)nt * bd, s, in, out, L1, L2, l, nt, S, sc);
+static void time_pass(const T* in, T* out, const T* L1, const T* L2, const T* tab, int l, int nt, int S,
+                      const DevScalars* sc, cudaStream_t s) {
+  const int bd = tri_threads<T>(nt, S), nb = (S + bd - 1) / bd;
+  const size_t sm = 2 * sizeof(T) * (size_t)nt * bd;
+  if (tab != nullptr)
+    launch_k(k_time_tri<T, true>, nb, bd, sm, s, in, out, L1, L2, tab, l, nt, S, sc);
+  else
+    launch_k(k_time_tri<T, false>, nb, bd, sm, s, in, out, L1, L2, tab, l, nt, S, sc);
 }
 
 // Exact time solve of the l = 0 variant: per spatial mode s, the tridiagonal
@@ -475,7 +522,7 @@ __global__ void __launch_bounds__(256) k_thomas(const T* __restrict__ in, T* __r
 template <typename T>
 static void precond_typed(const Geom& g, const T* Hx, const T* Hy, const T* V, const T* lamt,
                           const T* L1, const T* L2, const T* twx, const T* dctx, const T* twy,
-                          const T* dcty, const T* thc, const T* thd, const T* tho, int l,
+                          const T* dcty, const T* thc, const T* thd, const T* tho, const T* tri, int l,
                           const double* r, double* z, T* w0, T* w1,
                           const DevScalars* sc, cudaStream_t s, const PcgDot* dot,
                           const PcgZr* zr, bool tc = false) {
@@ -504,9 +551,9 @@ static void precond_typed(const Geom& g, const T* Hx, const T* Hy, const T* V, c
     if (tc && !g.time_simt && time_tc_supported(g.nt))
       launch_time_tc(a, b, V, lamt, L1, L2, g.nt, (int)S, sc, s);
     else
-      time_pass<T>(a, b, L1, L2, l, g.nt, (int)S, sc, s);
+      time_pass<T>(a, b, L1, L2, tri, l, g.nt, (int)S, sc, s);
   } else {
-    time_pass<T>(a, b, L1, L2, l, g.nt, (int)S, sc, s);
+    time_pass<T>(a, b, L1, L2, tri, l, g.nt, (int)S, sc, s);
   }
   { T* t = a; a = b; b = t; }
   if (g.nx > 1) {
@@ -535,11 +582,11 @@ void launch_precond(const Geom& g, const PrecTables& t, int precision, const dou
   }
   if (precision == MFG_MIXED || precision == MFG_MIXED_DF || precision == MFG_MIXED_TC)
     precond_typed<float>(g, t.Hx32, t.Hy32, t.Vt32, t.lamt32, t.L1_32, t.L2_32, t.twx32, t.dctx32,
-                         t.twy32, t.dcty32, t.thc32, t.thd32, t.tho32, t.l, r, z, work32, work32 + g.n,
+                         t.twy32, t.dcty32, t.thc32, t.thd32, t.tho32, nullptr, t.l, r, z, work32, work32 + g.n,
                          sc, s, dot, zr, precision == MFG_MIXED_TC);
   else
     precond_typed<double>(g, t.Hx64, t.Hy64, t.Vt64, t.lamt64, t.L1_64, t.L2_64, t.twx64, t.dctx64,
-                          t.twy64, t.dcty64, t.thc64, t.thd64, t.tho64, t.l, r, z, work64, work64 + g.n,
+                          t.twy64, t.dcty64, t.thc64, t.thd64, t.tho64, t.tri64, t.l, r, z, work64, work64 + g.n,
                           sc, s, dot, zr);
 }
 
@@ -557,9 +604,11 @@ int precond_step_kernel_count(const Geom& g, const PrecTables& t) {
 int precond_configure() {
   // one warp's columns of the longest time axis
   const int tri = 2 * kMaxNt * 32;
-  int bad = cudaFuncSetAttribute(k_time_tri<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  int bad = cudaFuncSetAttribute(k_time_tri<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  std::max(65536, tri * (int)sizeof(double))) != cudaSuccess;
-  bad |= cudaFuncSetAttribute(k_time_tri<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  bad |= cudaFuncSetAttribute(k_time_tri<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 std::max(65536, tri * (int)sizeof(double))) != cudaSuccess;
+  bad |= cudaFuncSetAttribute(k_time_tri<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               std::max(65536, tri * (int)sizeof(float))) != cudaSuccess;
   bad |= fft_configure() != MFG_OK;
   bad |= band_configure() != MFG_OK;

@@ -601,11 +601,13 @@ __global__ void __launch_bounds__(AJ * AI, 3) k_aat_q(Geom g, AatCoef a, int kc,
   aat_tail(acc, partials, sc);
 }
 
-// Blocks of the largest reducing launch of this file (viscosity fields and the
-// double-float stencil use the column grid).
+// Blocks of the largest reducing launch over the grid, in strips (for any blocks
+// per SM) or in columns (viscosity fields, the double-float stencil).
 int aat_blocks(const Geom& g) {
   const dim3 g2 = aat2_grid(g, aat2_chunk(g));
-  return std::max({(int)((long long)g2.x * g2.y * g2.z), strip_grid(g, kQPerSm).blocks, strip_grid(g, kCPerSm).blocks});
+  int most = (int)((long long)g2.x * g2.y * g2.z);
+  for (int per_sm = 1; per_sm <= 6; ++per_sm) most = std::max(most, strip_grid(g, per_sm).blocks);
+  return most;
 }
 
 // The same two passes in double-float arithmetic (df64.cuh, the MFG_MIXED_DF

@@ -161,6 +161,7 @@ struct PrecTables {
   // the off-diagonal per mode (S); null otherwise.
   double *thc64 = nullptr, *thd64 = nullptr, *tho64 = nullptr;
   float *thc32 = nullptr, *thd32 = nullptr, *tho32 = nullptr;
+  double* tri64 = nullptr;  // FP64 plans, l = 1, 2: factors of the time elimination (n); else null
   // Viscosity field: face coefficients (Geom::kfx, kfy) and the banded Cholesky
   // factors of the per-frequency systems (k_band.cu); null otherwise.
   double *kfx = nullptr, *kfy = nullptr;
