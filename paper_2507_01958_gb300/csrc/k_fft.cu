@@ -74,8 +74,14 @@ __global__ void __launch_bounds__(256) k_fft(const TI* __restrict__ in, TO* __re
   cx<T>* dcs = tws + N / 2;               // DCT phases, N
   const int tid = threadIdx.x;
   for (int q = tid; q < N / 2; q += 256) tws[q] = cx<T>{tw[2 * q], tw[2 * q + 1]};
+  // phases with the transform's scale folded in: c_k / 2 (DCT-II, the 1/2 of the
+  // separation), 1/(N c_k) (DCT-III; both operands of a k > 0 have the same c)
+  const T rsn = T(1) / sqrt(T(N));
   if (MODE != FFT_DHT)
-    for (int q = tid; q < N; q += 256) dcs[q] = cx<T>{dct[2 * q], dct[2 * q + 1]};
+    for (int q = tid; q < N; q += 256) {
+      const T f = MODE == FFT_DCT2 ? (q == 0 ? T(0.5) * rsn : T(0.5) * sqrt(T(2) / T(N))) : (q == 0 ? rsn : T(1) / sqrt(T(2 * N)));
+      dcs[q] = cx<T>{f * dct[2 * q], f * dct[2 * q + 1]};
+    }
   const long long line0 = (long long)blockIdx.x * LB;
   const long long o = blockIdx.y;
 
@@ -144,15 +150,13 @@ __global__ void __launch_bounds__(256) k_fft(const TI* __restrict__ in, TO* __re
   }
   __syncthreads();
   if (MODE == FFT_DCT3) {
-    // W = exp(i th_k) (X_k - i X_{N-k}) with X = C/c, times 1/N of the inverse FFT.
-    const T s0 = T(1) / sqrt(T(N)), s1 = T(1) / sqrt(T(2 * N));
+    // W = exp(i th_k) (X_k - i X_{N-k}) with X = C/c, times 1/N of the inverse FFT
     for (int idx = tid; idx < CL * N; idx += 256) {
       const int q = idx / N, k = idx % N;
       const T* xa = real1 + (2 * q) * NP;
       const T* xb = real1 + (2 * q + 1) * NP;
-      const T sk = k == 0 ? s0 : s1, sm = s1;  // N-k > 0 whenever k > 0
-      const T ak = xa[k] * sk, bk = xb[k] * sk;
-      const T am = k == 0 ? T(0) : xa[N - k] * sm, bm = k == 0 ? T(0) : xb[N - k] * sm;
+      const T ak = xa[k], bk = xb[k];
+      const T am = k == 0 ? T(0) : xa[N - k], bm = k == 0 ? T(0) : xb[N - k];
       const T c = dcs[k].x, s = dcs[k].y;
       const T war = c * ak + s * am, wai = s * ak - c * am;
       const T wbr = c * bk + s * bm, wbi = s * bk - c * bm;
@@ -294,7 +298,6 @@ __global__ void __launch_bounds__(256) k_fft(const TI* __restrict__ in, TO* __re
   T* R = reinterpret_cast<T*>(odd ? buf0 : buf1);  // real output staging [LB][NP]
 
   // ---- separate the packed pairs and finish the transform
-  const T rsn = T(1) / sqrt(T(N));
   for (int idx = tid; idx < CL * N; idx += 256) {
     const int q = idx / N, k = idx % N;
     if (MODE == FFT_DCT3) {
@@ -306,16 +309,15 @@ __global__ void __launch_bounds__(256) k_fft(const TI* __restrict__ in, TO* __re
     } else {
       const cx<T> zk = Z[q * NP + swz<N>(k)];
       const cx<T> zm = Z[q * NP + swz<N>((N - k) & (N - 1))];
-      const T sr = T(0.5) * (zk.x + zm.x), si = T(0.5) * (zk.y - zm.y);  // X_a
-      const T dr = T(0.5) * (zk.y + zm.y), di = T(0.5) * (zm.x - zk.x);  // X_b
+      const T sr = zk.x + zm.x, si = zk.y - zm.y;  // 2 X_a
+      const T dr = zk.y + zm.y, di = zm.x - zk.x;  // 2 X_b
       if (MODE == FFT_DHT) {
-        R[(2 * q) * NP + k] = (sr - si) * rsn;
-        R[(2 * q + 1) * NP + k] = (dr - di) * rsn;
+        R[(2 * q) * NP + k] = (sr - si) * (T(0.5) * rsn);
+        R[(2 * q + 1) * NP + k] = (dr - di) * (T(0.5) * rsn);
       } else {
-        const T ck = k == 0 ? T(1) / sqrt(T(N)) : sqrt(T(2) / T(N));
         const T c = dcs[k].x, s = dcs[k].y;
-        R[(2 * q) * NP + k] = ck * (c * sr + s * si);
-        R[(2 * q + 1) * NP + k] = ck * (c * dr + s * di);
+        R[(2 * q) * NP + k] = c * sr + s * si;
+        R[(2 * q + 1) * NP + k] = c * dr + s * di;
       }
     }
   }

@@ -224,7 +224,10 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 2 : 3) k_fft_mixed(co
   cx<T>* dcs = tws + N;
   for (int q = tid; q < N; q += nth) {
     tws[q] = cx<T>{tw[2 * q], tw[2 * q + 1]};
-    if (mode != FFT_DHT) dcs[q] = cx<T>{dct[2 * q], dct[2 * q + 1]};
+    if (mode != FFT_DHT) {  // phases with the transform's scale, as in k_fft.cu
+      const T f = mode == FFT_DCT2 ? T(0.5) * (q == 0 ? (T)P.r1 : (T)P.r2) : (q == 0 ? (T)P.r1 : (T)P.rh);
+      dcs[q] = cx<T>{f * dct[2 * q], f * dct[2 * q + 1]};
+    }
   }
   const long long line0 = (long long)blockIdx.x * LB, o = blockIdx.y;
   const int total = LB * N;
@@ -283,14 +286,12 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 2 : 3) k_fft_mixed(co
   __syncthreads();
   if (mode == FFT_DCT3) {
     // exp(i th_k) (X_k - i X_{N-k}) with X = C/c, times 1/N of the inverse FFT
-    const T s0 = (T)P.r1, s1 = (T)P.rh;
     for (int idx = tid; idx < CL * N; idx += nth) {
       const int q = quot(idx, P.dN), k = idx - q * N;
       const T* xa = real1 + (2 * q) * NP;
       const T* xb = xa + NP;
-      const T sk = k == 0 ? s0 : s1;
-      const T ak = xa[k] * sk, bk = xb[k] * sk;
-      const T am = k == 0 ? T(0) : xa[N - k] * s1, bm = k == 0 ? T(0) : xb[N - k] * s1;
+      const T ak = xa[k], bk = xb[k];
+      const T am = k == 0 ? T(0) : xa[N - k], bm = k == 0 ? T(0) : xb[N - k];
       const T c = dcs[k].x, s = dcs[k].y;
       buf0[q * NP + k] = cx<T>{(c * ak + s * am) - (s * bk - c * bm), (s * ak - c * am) + (c * bk + s * bm)};
     }
@@ -299,7 +300,7 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 2 : 3) k_fft_mixed(co
   const int odd = fft_stages<T>(P, mode == FFT_DCT3 ? T(1) : T(-1));
   const cx<T>* Z = odd ? buf1 : buf0;
   T* R = reinterpret_cast<T*>(odd ? buf0 : buf1);  // real outputs [LB][NP]
-  const T rsn = (T)P.r1, rs2 = (T)P.r2;
+  const T hrs = T(0.5) * (T)P.r1;
   for (int idx = tid; idx < CL * N; idx += nth) {
     const int q = quot(idx, P.dN), k = idx - q * N;
     T* ra = R + (2 * q) * NP + k;
@@ -309,15 +310,15 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 2 : 3) k_fft_mixed(co
       ra[NP] = v.y;
     } else {
       const cx<T> zk = Z[q * NP + k], zm = Z[q * NP + (k == 0 ? 0 : N - k)];
-      const T sr = T(0.5) * (zk.x + zm.x), si = T(0.5) * (zk.y - zm.y);  // X_a
-      const T dr = T(0.5) * (zk.y + zm.y), di = T(0.5) * (zm.x - zk.x);  // X_b
+      const T sr = zk.x + zm.x, si = zk.y - zm.y;  // 2 X_a
+      const T dr = zk.y + zm.y, di = zm.x - zk.x;  // 2 X_b
       if (mode == FFT_DHT) {
-        ra[0] = (sr - si) * rsn;
-        ra[NP] = (dr - di) * rsn;
+        ra[0] = (sr - si) * hrs;
+        ra[NP] = (dr - di) * hrs;
       } else {
-        const T ck = k == 0 ? rsn : rs2, c = dcs[k].x, s = dcs[k].y;
-        ra[0] = ck * (c * sr + s * si);
-        ra[NP] = ck * (c * dr + s * di);
+        const T c = dcs[k].x, s = dcs[k].y;
+        ra[0] = c * sr + s * si;
+        ra[NP] = c * dr + s * di;
       }
     }
   }
