@@ -73,6 +73,14 @@ __device__ __forceinline__ df df_mul(df a, df b) {
 // 2^k as an FP32 number, for -126 <= k <= 127 (built from its bit pattern).
 __device__ __forceinline__ float pow2f(int k) { return __uint_as_float((unsigned)(k + 127) << 23); }
 
+// Magnitudes outside the fast path below.  Out of line: inlined, its FP64
+// conversions become predicated instructions that every call issues, and each of
+// them holds the FP64 unit for 16 cycles whether it is taken or not.
+static __device__ __noinline__ float2 df_from_double_slow(double x) {
+  const float h = __double2float_rn(x);
+  return make_float2(h, __double2float_rn(x - (double)h));
+}
+
 // FP64 -> df64.  Fast path (2^-74 <= |x| < 2^128): hi takes the sign, the
 // exponent and the top 23 explicit mantissa bits; lo is the remaining 29 bits,
 // converted as an integer and scaled by a power of two; a final quick_two_sum
@@ -83,8 +91,8 @@ __device__ __forceinline__ df df_from_double(double x) {
   const int e = (int)((b >> 52) & 0x7FF);
   if (e == 0) return df{0.0f, 0.0f};
   if (e < 949 || e > 1150) {
-    const float h = __double2float_rn(x);
-    return df{h, __double2float_rn(x - (double)h)};
+    const float2 s = df_from_double_slow(x);
+    return df{s.x, s.y};
   }
   const unsigned int sign = (unsigned int)(b >> 32) & 0x80000000u;
   const unsigned long long m = b & 0xFFFFFFFFFFFFFull;
@@ -94,14 +102,15 @@ __device__ __forceinline__ df df_from_double(double x) {
   return quick_two_sum(hi, lo);
 }
 
-// FP32 -> FP64 by bits (normal numbers exactly; zero and subnormals give 0).
+// FP32 -> FP64 by bits (normal numbers, Inf and NaN exactly; zero and subnormals
+// give 0).
 __device__ __forceinline__ double f2d_bits(float f) {
   const unsigned int u = __float_as_uint(f);
   const unsigned int ex = (u >> 23) & 0xFF;
   if (ex == 0) return 0.0;
-  if (ex == 255) return (double)f;  // keep Inf and NaN visible
+  const unsigned int e64 = ex == 255 ? 0x7FFu : ex + 896;  // Inf and NaN stay visible
   const unsigned long long s = (unsigned long long)(u & 0x80000000u) << 32;
-  const unsigned long long d = s | ((unsigned long long)(ex + 896) << 52) |
+  const unsigned long long d = s | ((unsigned long long)e64 << 52) |
                                ((unsigned long long)(u & 0x7FFFFFu) << 29);
   return __longlong_as_double((long long)d);
 }

@@ -20,6 +20,7 @@
 #include "df64.cuh"
 #include "mfg_internal.cuh"
 #include "reduce.cuh"
+#include "strip.cuh"
 
 namespace mfg {
 
@@ -63,6 +64,14 @@ __device__ __noinline__ double newton_h64(double B, double hP, double tau, doubl
     if (dxv <= 1e-16 * x || hi - lo <= 4e-16 * hi) break;
   }
   return x;
+}
+
+// A whole cell on that path, zero test included (out of line, so that its divisions
+// are no predicated instructions of the fast path): the root and w = (.).y P.
+__device__ __noinline__ double2 cell_h64(double B, double P2, double tau, double half_itau, double a1, double tb) {
+  if (B + P2 * half_itau <= 0.0) return make_double2(0.0, 0.0);
+  const double x = newton_h64(B, 0.5 * tau * P2, tau, a1, tb, fmax(B, 0.0) + P2 * half_itau);
+  return make_double2(x, x / (x + tau));
 }
 
 // Prox for the general power Hamiltonian |p|^{q'}/q', q = q'/(q'-1), b_hat =
@@ -246,8 +255,8 @@ __device__ void prox_cell_q(double mbar, const double (&wbar)[NW], double tau, d
 
 // Per-step constants of the prox (tau is the CP primal step).
 struct ProxK {
-  double tau, half_tau, half_itau, tb;  // tau, tau/2, 1/(2 tau), tau f_b
-  float tauf, tbf;
+  double tau, tau2, half_tau, half_itau, tb;  // tau, tau^2, tau/2, 1/(2 tau), tau f_b
+  float tauf, tbf, itau2f;                    // itau2f = 1/tau^2
   df taud, tbd;                         // tau, tau f_b as double-float pairs
   bool tau_ok;                          // tau inside the FP32 fast-path range
 };
@@ -255,11 +264,13 @@ struct ProxK {
 __device__ __forceinline__ ProxK prox_consts(double tau, double half_itau, double f_b) {
   ProxK k;
   k.tau = tau;
+  k.tau2 = tau * tau;
   k.half_tau = 0.5 * tau;
   k.half_itau = half_itau;
   k.tb = tau * f_b;
   k.tauf = (float)tau;
   k.tbf = (float)k.tb;
+  k.itau2f = (float)(4.0 * half_itau * half_itau);
   k.taud = df_from_double(tau);
   k.tbd = df_from_double(k.tb);
   k.tau_ok = tau > 1e-15 && tau < 1e15;
@@ -280,40 +291,52 @@ __device__ __forceinline__ ProxK prox_consts(double tau, double half_itau, doubl
 // from an FP32 root two steps reach the double-float resolution.  The polish
 // stops after a step below 1e-9 relative and keeps the bracket, bisecting if
 // a step leaves it.  Inputs outside the FP32 range take an FP64 Newton.
+// act: bit q set where some lane of the warp has a nonzero projection P_q; the
+// others are zero throughout and cost nothing.  (FP64 issue bounds the prox, so the
+// set-up takes as few FP64 instructions as it can: sign and zero tests on bit
+// patterns, the bracket in FP32, all FP32 values from the double-float splits.)
 template <int NW>
 __device__ __forceinline__ void prox_cell(double mbar, const double (&wbar)[NW], const ProxK& K, double a1,
-                                          float a1f, const df& a1d, double c, double& m, double (&w)[NW]) {
+                                          float a1f, const df& a1d, double c, double& m, double (&w)[NW],
+                                          unsigned act = ~0u) {
   // projection onto K by sign tests on the bit patterns (no FP64 min/max)
   double P[NW];
   double P2 = 0.0;
 #pragma unroll
   for (int q = 0; q < NW; ++q) {
-    const bool neg = __double_as_longlong(wbar[q]) < 0;
-    P[q] = ((q & 1) ? neg : !neg) ? wbar[q] : 0.0;
-    P2 = fma(P[q], P[q], P2);
+    P[q] = 0.0;
+    if (act & (1u << q)) {
+      const bool neg = __double_as_longlong(wbar[q]) < 0;
+      P[q] = ((q & 1) ? neg : !neg) ? wbar[q] : 0.0;
+      P2 = fma(P[q], P[q], P2);
+    }
   }
   const double B = fma(-K.tau, c, mbar);
-  const double hp0 = P2 * K.half_itau;  // |P|^2 / (2 tau)
-  if (B + hp0 <= 0.0) {                 // h(0) = -B - |P|^2/(2 tau) >= 0
+  const double hP = K.half_tau * P2;
+  // h(0) = -B - |P|^2/(2 tau) >= 0, as the sign of tau^2 B + hP; a NaN is not a zero
+  // cell (a tau whose square leaves the range takes cell_h64 below)
+  const double zt = fma(B, K.tau2, hP);
+  const unsigned zh = (unsigned)__double2hiint(zt), zl = (unsigned)__double2loint(zt), za = zh & 0x7FFFFFFFu;
+  const bool znan = za > 0x7FF00000u || (za == 0x7FF00000u && zl != 0u);
+  if (K.tau_ok && (((zh >> 31) && !znan) || (za | zl) == 0u)) {
     m = 0.0;
 #pragma unroll
     for (int q = 0; q < NW; ++q) w[q] = 0.0;
     return;
   }
-  const double hi0 = fmax(B, 0.0) + hp0;
-  const double hP = K.half_tau * P2;
-  const float hif = (float)hi0, Bf = (float)B, hPf = (float)hP;
+  const df Bd = df_from_double(B), hPd = df_from_double(hP);
+  const float Bf = Bd.hi, hPf = hPd.hi;
+  // upper end of the bracket, max(0, B) + |P|^2/(2 tau), a little above its FP32 value
+  const float hif = (fmaxf(Bf, 0.0f) + hPf * K.itau2f) * 1.000001f;
   const bool fp32_ok = K.tau_ok && hif < 1e15f && hPf < 1e30f && fabsf(Bf) < 1e30f;
   if (!fp32_ok) {
-    const double x = newton_h64(B, hP, K.tau, a1, K.tb, hi0);
-    m = x;
-    const double s = x / (x + K.tau);
+    const double2 xs = cell_h64(B, P2, K.tau, K.half_itau, a1, K.tb);
+    m = xs.x;
 #pragma unroll
-    for (int q = 0; q < NW; ++q) w[q] = s * P[q];
+    for (int q = 0; q < NW; ++q) w[q] = xs.y * P[q];
     return;
   }
-  const df Bd = df_from_double(B), hPd = df_from_double(hP);
-  df lo{0.0f, 0.0f}, hi = df_from_double(hi0);
+  df lo{0.0f, 0.0f}, hi{hif, 0.0f};
   df x{newton_h32(hif, Bf, hPf, K.tauf, a1f, K.tbf), 0.0f};
   for (int it = 0; it < 100; ++it) {
     const df t = df_add_same(x, K.taud);
@@ -343,7 +366,45 @@ __device__ __forceinline__ void prox_cell(double mbar, const double (&wbar)[NW],
   m = df_to_double(x);
   const double s = df_to_double(df_mul(x, r));
 #pragma unroll
-  for (int q = 0; q < NW; ++q) w[q] = s * P[q];
+  for (int q = 0; q < NW; ++q) {
+    w[q] = 0.0;
+    if (act & (1u << q)) w[q] = s * P[q];
+  }
+}
+
+// End of a CP step: acc = this thread's share of ||m_{l+1} - m_l||^2; the last
+// block updates the step sizes and decides whether the loop goes on.
+__device__ __forceinline__ void prox_tail(double acc, double tau, double theta, double gamma, double* partials,
+                                          DevScalars* sc, cudaGraphConditionalHandle h, int use_handle) {
+  double part[1] = {acc};
+  block_sum<1>(part);
+  if (!publish_and_check_last<1>(part, partials, &sc->counter)) return;
+  double tot[1];
+  gather_partials<1>(partials, tot);
+  if (flat_tid() == 0) {
+    const double r = sqrt(tot[0]);
+    sc->dm2 = tot[0];
+    sc->r_last = r;
+    const double tau_next = theta * tau;
+    sc->tau = tau_next;
+    sc->sigma = sc->sigma / theta;
+    sc->theta = 1.0 / sqrt(1.0 + 2.0 * gamma * tau_next);
+    sc->half_itau = 0.5 / tau_next;
+    sc->ell += 1;
+    sc->cp_iters += 1;
+    sc->cg_total += sc->cg_it;
+    if (sc->cg_it > sc->cg_max) sc->cg_max = sc->cg_it;
+    sc->cp_left -= 1;
+    if (!isfinite(r)) {
+      sc->status = MFG_ERR_NONFINITE;
+      sc->cp_done = 1;
+    }
+    // a non-finite value or a timed-out device wait ends the instance's solve
+    if (sc->status == MFG_ERR_NONFINITE || sc->status == MFG_ERR_TIMEOUT) sc->cp_done = 1;
+    if (sc->cp_tol > 0.0 && r <= sc->cp_tol) sc->cp_done = 1;
+    if (use_handle) cudaGraphSetConditional(h, (sc->cp_left > 0 && !sc->cp_done) ? 1u : 0u);
+    sc->counter = 0;
+  }
 }
 
 // y, ybar hold c planes; z one plane set.  Cell e pairs (m^{k+1}, w^k).
@@ -354,7 +415,7 @@ __device__ __forceinline__ void prox_cell(double mbar, const double (&wbar)[NW],
 // so the difference across the end (a flux slot of Sec. 4.3 that does not
 // exist) is zero and K takes its one-sided form.  VN (viscosity field): nu K z
 // becomes K_nu z = kf_yp dyp - kf_ym dym (+ x terms), the face coefficients of
-// Geom::kfx / kfy.
+// Geom::kfx / kfy.  Point by point: viscosity fields and rows too short for strips.
 template <int ACTX, bool GENQ, bool VN>
 __global__ void __launch_bounds__(kThreads) k_prox_cp(Geom g, Coef cf, const double* __restrict__ z,
                                                       double* __restrict__ y, double* __restrict__ ybar,
@@ -430,35 +491,108 @@ __global__ void __launch_bounds__(kThreads) k_prox_cp(Geom g, Coef cf, const dou
     }
     acc = fma(dm, dm, acc);
   }
-  double part[1] = {acc};
-  block_sum<1>(part);
-  if (!publish_and_check_last<1>(part, partials, &sc->counter)) return;
-  double tot[1];
-  gather_partials<1>(partials, tot);
-  if (flat_tid() == 0) {
-    const double r = sqrt(tot[0]);
-    sc->dm2 = tot[0];
-    sc->r_last = r;
-    const double tau_next = theta * tau;
-    sc->tau = tau_next;
-    sc->sigma = sc->sigma / theta;
-    sc->theta = 1.0 / sqrt(1.0 + 2.0 * cf.gamma * tau_next);
-    sc->half_itau = 0.5 / tau_next;
-    sc->ell += 1;
-    sc->cp_iters += 1;
-    sc->cg_total += sc->cg_it;
-    if (sc->cg_it > sc->cg_max) sc->cg_max = sc->cg_it;
-    sc->cp_left -= 1;
-    if (!isfinite(r)) {
-      sc->status = MFG_ERR_NONFINITE;
-      sc->cp_done = 1;
-    }
-    // a non-finite value or a timed-out device wait ends the instance's solve
-    if (sc->status == MFG_ERR_NONFINITE || sc->status == MFG_ERR_TIMEOUT) sc->cp_done = 1;
-    if (sc->cp_tol > 0.0 && r <= sc->cp_tol) sc->cp_done = 1;
-    if (use_handle) cudaGraphSetConditional(h, (sc->cp_left > 0 && !sc->cp_done) ? 1u : 0u);
-    sc->counter = 0;
+  prox_tail(acc, tau, theta, cf.gamma, partials, sc, h, use_handle);
+}
+
+constexpr int kProxPerSm = 2;  // 256-thread blocks per SM of the strip kernel
+
+// The same step in warp strips (strip.cuh; constant viscosity): each face difference
+// of z formed once, and the flux components that are zero across a whole warp, old
+// value and projection alike (half of them where the flow has one direction over 32 cells),
+// skip theirs.  54 FP64 instructions per cell on noisy data (~66 before, 68 with the
+// out-of-range paths of the double-float conversions inlined): 256^2 x 128 754 -> 627 us a
+// step, the 512^2 x 128 solve 140 -> 136 ms.
+template <int ACTX, bool GENQ>
+__global__ void __launch_bounds__(256, kProxPerSm) k_prox_strip(Geom g, StripGrid sg, Coef cf,
+                                                                const double* __restrict__ z,
+                                                                double* __restrict__ y, double* __restrict__ ybar,
+                                                                const double* __restrict__ V,
+                                                                const double* __restrict__ W, double* partials,
+                                                                DevScalars* sc, cudaGraphConditionalHandle h,
+                                                                int use_handle, double* __restrict__ Az,
+                                                                const double* __restrict__ rfin) {
+  dep_sync();
+  constexpr int NW = ACTX ? 4 : 2;
+  const double tau = sc->tau, theta = sc->theta;
+  double acc = 0.0;
+  int j0, i0, i1, k;
+  if (strip_item(sg, g, j0, i0, i1, k)) {
+    const ProxK K = prox_consts(tau, sc->half_itau, cf.f_b);
+    const bool last = k == g.nt - 1;
+    const double a1 = last ? fma(tau, fma(cf.g_a, g.idt, cf.f_a), 1.0) : fma(tau, cf.f_a, 1.0);
+    const float a1f = (float)a1;
+    const df a1d = df_from_double(a1);
+    const double t_idt = tau * g.idt, t_idx = tau * g.idx, t_idy = tau * g.idy, t_ny = tau * g.nu * g.ay,
+                 t_nx = tau * g.nu * g.ax;
+    const long long n = g.n, base = (long long)k * g.S;
+    const double* zk = z + base;
+    const int j = j0 + (threadIdx.x & 31), jc = j < g.ny ? j : g.ny - 1;
+    struct Row {
+      double zn, m, cc, w[NW];
+    };
+    diff_march<ACTX, false, 1>(
+        g, i0, i1, j0, [&](int i, int jj) { return zk[i * g.ny + jj]; },
+        [&](int i) {
+          const int f = i * g.ny + jc;
+          const long long e = base + f;
+          Row x;
+          x.zn = last ? 0.0 : z[e + g.S];
+          x.m = y[e];
+#pragma unroll
+          for (int q = 0; q < NW; ++q) x.w[q] = y[e + (q + 1) * n];
+          x.cc = last ? fma(W[f], g.idt, V[f]) : V[f];
+          return x;
+        },
+        [&](int i, double zc, double dyp, double dym, double dxp, double dxm, const Row& x) {
+          double d[NW];
+          if (ACTX) { d[0] = dxp; d[1] = dxm; }
+          d[NW - 2] = dyp;
+          d[NW - 1] = dym;
+          const bool own = j < g.ny;
+          unsigned act = 0;
+#pragma unroll
+          for (int q = 0; q < NW; ++q) {
+            // -d has the component's sign, or the old value is not zero
+            const bool neg = __double_as_longlong(d[q]) < 0, old = (__double_as_longlong(x.w[q]) << 1) != 0;
+            if (GENQ || __any_sync(0xffffffffu, (old || ((q & 1) ? !neg : neg)))) act |= 1u << q;
+          }
+          // (lanes past the last column run along on its cell and store nothing, so
+          // that the warp can meet again after the root)
+          const long long e = base + i * g.ny + j;
+          if (own && Az != nullptr) Az[e] -= rfin[e];  // AAt z_{l+1} = b - r_final (stop reference)
+          // primal step y - tau x, x_m = nu K z + (z - z_next)/dt, x_w = d / dx
+          double mbar = fma(-t_ny, dyp - dym, fma(-t_idt, zc - x.zn, x.m));
+          if (ACTX) mbar = fma(-t_nx, dxp - dxm, mbar);
+          double wbar[NW], w_new[NW], m_new;
+#pragma unroll
+          for (int q = 0; q < NW; ++q) {
+            wbar[q] = 0.0;
+            if (act & (1u << q)) wbar[q] = fma(-((ACTX && q < 2) ? t_idx : t_idy), d[q], x.w[q]);
+          }
+          if constexpr (GENQ)
+            prox_cell_q<NW>(mbar, wbar, tau, cf.qprime, a1, K.tb, x.cc, m_new, w_new);
+          else
+            prox_cell<NW>(mbar, wbar, K, a1, a1f, a1d, x.cc, m_new, w_new, act);
+          __syncwarp();
+          const double dm = m_new - x.m, mb = fma(theta, dm, m_new);
+          double b[NW];
+#pragma unroll
+          for (int q = 0; q < NW; ++q) {
+            b[q] = 0.0;
+            if (act & (1u << q)) b[q] = fma(theta, w_new[q] - x.w[q], w_new[q]);
+          }
+          if (!own) return;
+          acc = fma(dm, dm, acc);
+          y[e] = m_new;
+          ybar[e] = mb;
+#pragma unroll
+          for (int q = 0; q < NW; ++q) {
+            y[e + (q + 1) * n] = w_new[q];
+            ybar[e + (q + 1) * n] = b[q];
+          }
+        });
   }
+  prox_tail(acc, tau, theta, cf.gamma, partials, sc, h, use_handle);
 }
 
 template <int ACTX, bool GENQ>
@@ -521,6 +655,17 @@ void launch_prox_cp(const Geom& g, const Coef& cf, const double* z, double* y, d
                     const double* V, const double* W, double* partials, DevScalars* sc,
                     cudaGraphConditionalHandle h, int use_handle, cudaStream_t s, double* Az,
                     const double* rfin) {
+  if (strips_fit(g)) {
+    const StripGrid sg = strip_grid(g, kProxPerSm);
+    const bool gq = cf.qprime != 2.0;
+#define MFG_PROX_STRIP(A, Q)                                                                                        \
+  launch_k(k_prox_strip<A, Q>, sg.blocks, 32 * sg.warps, 0, s, g, sg, cf, z, y, ybar, V, W, partials, sc, h, use_handle, \
+           Az, rfin)
+    if (g.actx) { if (gq) MFG_PROX_STRIP(1, true); else MFG_PROX_STRIP(1, false); }
+    else        { if (gq) MFG_PROX_STRIP(0, true); else MFG_PROX_STRIP(0, false); }
+#undef MFG_PROX_STRIP
+    return;
+  }
   const int idx = (g.actx ? 4 : 0) + (cf.qprime != 2.0 ? 2 : 0) + (g.kfy != nullptr ? 1 : 0);
   const int nb = red_blocks(g.n, g_prox_wave[idx]);
   // the general-q' root finder and the viscosity field are their own
