@@ -9,8 +9,9 @@ One step = one fixed-count solve: 300 accelerated Chambolle-Pock iterations
 (each with its preconditioned AAt solve to relative tolerance 1e-10 against
 ||b||, and the per-cell prox) from the initial iterate, one CUDA-graph launch.
 Metric: CP iterations per second (each CP iteration is one preconditioned AAt
-solve).  Precision (default): the preconditioner in FP32 with its dense time
-transforms on the tensor cores (tcgen05, split TF32), inside FP64 flexible
+solve).  Precision (default): the preconditioner in FP32, its time pass by dense
+transforms on the tensor cores (tcgen05, split TF32) or by elimination, whichever the
+autotuner finds faster, inside FP64 flexible
 PCG with an FP64 AAt, FP64 residuals and dot products and the FP64 prox.
 
 The JSON line also carries: the same metric through the host-buffer entry
@@ -51,13 +52,13 @@ CG_TOL = 1e-10
 METRIC = "CP iterations/s (preconditioned AAt solves/s), 2-D Neumann 512^2 x 128"
 WORKLOAD = ("2-D Neumann unit square 512x512, N_t=128 (n=33,554,432), nu=1e-2, "
             "300 CP iterations per step from the initial iterate")
-# Precision of the timed solve and of the extras: FP32 preconditioner with the
-# time transforms on the tensor cores (tcgen05, split TF32), FP64 elsewhere.
+# Precision of the timed solve and of the extras: FP32 preconditioner, its time
+# pass on the tensor cores (tcgen05, split TF32) or by elimination, FP64 elsewhere.
 PRECISION = "mixed_tc"
 # Algorithmic FP64 flops of one AAt apply per unknown in the factored form
 # q = C (C^T p): K p (4 differences, 2 adds, 2 scalings, 1 add = 9),
 # xm = nu Kp + (p - p')/dt (4), q = nu K xm + (xm - xm')/dt + 2 Kp (10 + 2 + 2)
-# -> 27.  (The kernels issue 15 FP64 instructions per unknown, mostly FMAs.)
+# -> 27.  (The kernels issue 12 FP64 instructions per unknown, mostly FMAs.)
 AAT_FLOPS_PER_UNKNOWN = 27
 # Algorithmic bytes of one AAt apply: read p, write q (2 FP64 words per unknown).
 AAT_BYTES_PER_UNKNOWN = 16
@@ -325,7 +326,7 @@ def kernels_measure(L, dev, stream, peak_gbs):
 
     out = {"workload": "2-D Neumann 512^2 x N_t 128, nu = 1e-2 (n = 33,554,432)"}
     plan = L.mfg_plan(dict(p, precision="mixed"))
-    out["AAt apply (k_aat_x + k_aat_q)"] = entry(
+    out["AAt apply (k_aat_u + k_aat_q2)"] = entry(
         timed(lambda: L.mfg_apply_AAt(plan, 0, r, z, stream=stream)), 16 * n, 56 * n, "FP64 issue")
     out["C apply (k_apply_C)"] = entry(timed(lambda: L.mfg_apply_C(plan, 0, y, z, stream=stream)),
                                        48 * n, 48 * n, "FP64 issue")
@@ -598,7 +599,7 @@ def run_gpu(args):  # noqa: C901
     err_mixed = float(torch.linalg.norm(fm.y - f64.y) / torch.linalg.norm(f64.y))
     del f64, fm
 
-    # Dominant kernel: the AAt apply (k_aat_x + k_aat_q, FP64 issue bound), timed
+    # Dominant kernel: the AAt apply (k_aat_u + k_aat_q2, FP64 issue bound), timed
     # with CUDA events on the stream it is launched on, same launch shapes as in
     # the solve graph.
     p_in = torch.randn(n_per, dtype=torch.float64, device=dev)
@@ -662,7 +663,7 @@ def run_gpu(args):  # noqa: C901
                           "headline_precision_same_count": rm["value"]},
             "mixed_vs_fp64_speedup": rm["value"] / r64["value"],
             "mixed_rel_err_vs_fp64_path": err_mixed,
-            "roofline": {"kernel": "AAt apply: k_aat_x + k_aat_q (C C^T stencil, FP64)", "bound": "alu",
+            "roofline": {"kernel": "AAt apply: k_aat_u + k_aat_q2 (C C^T stencil, FP64)", "bound": "alu",
                          "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                          "frac": achieved / FP64_PEAK_TFLOPS, "traffic": traffic,
                          "algorithmic_flops_per_launch": flops, "algorithmic_bytes_per_launch":

@@ -58,9 +58,10 @@ enum { MFG_PERIODIC = 0, MFG_NEUMANN = 1 };
  * AAt stencil evaluated in double-float arithmetic (pairs of FP32 numbers,
  * ~48 significant bits) from FP64 inputs to FP64 outputs; residuals, dot
  * products and the prox stay FP64.  MFG_MIXED_TC: as MFG_MIXED, with the
- * preconditioner's dense time transforms (DCT-VIII / DST-I products, Sec. 4.2)
+ * preconditioner's time transforms (DCT-VIII / DST-I, Sec. 4.2) as dense products
  * on the tensor cores (tcgen05, TF32 operands split in three products for
- * ~FP32 accuracy) when N_t is 32, 64 or 128, on the CUDA cores otherwise.
+ * ~FP32 accuracy) when N_t is 32, 64 or 128, unless mfg_autotune finds the
+ * elimination that every other plan takes faster.
  * GB300 issues FP32 at ~58x its FP64 rate. */
 enum { MFG_FP64 = 0, MFG_MIXED = 1, MFG_MIXED_DF = 2, MFG_MIXED_TC = 3 };
 /* PCG tolerance: fixed cg_tol, or the paper's rule
@@ -291,9 +292,9 @@ typedef struct {
  * `stream`) the candidate launch choices and keeps the fastest:
  *   - grid cap of the vector and reduction kernels: 152, 304 or 608 blocks;
  *   - the preconditioner step (Alg. 1/2 with the fused PCG vector work): time
- *     pass on the tensor cores or the CUDA cores (MFG_MIXED_TC with N_t in
+ *     pass on the tensor cores or by elimination (MFG_MIXED_TC with N_t in
  *     {32, 64, 128}), FFT or dense transform pass on each power-of-two axis;
- *   - AAt stencil launch: 152 x 4, 8 or 16 target blocks.
+ *   - AAt stencil launch: 152 x 4, 8 or 16 (row chunks of the strips).
  * The choice is cached per process by instance shape (grid, N_t, boundary
  * conditions, precision, l): a later plan with the same shape takes it
  * without timing.  Uses the plan's workspace and a temporary n-double buffer
