@@ -219,10 +219,12 @@ void launch_stop_reference_start(const Inst& in, const double* z, cudaStream_t s
 // (constant viscosity, FP64 stencil), two direction buffers alternating; else
 // k_update_p updates the one.  From 2^22 points on, where the vectors no longer stay
 // in L2 between passes: the 512^2 x 128 solve 136.3 -> 133.9 ms; four 128^2 x 64 tori
-// 23.9 -> 24.2 ms, so smaller instances keep the separate pass.
-bool forms_dir(const Inst& in) {
+// 23.9 -> 24.2 ms, so smaller instances keep the separate pass, and so does one whose
+// second buffer no longer fits beside the rest of the plan.
+bool wants_dir(const Inst& in) {
   return in.g.kfy == nullptr && in.p.precision != MFG_MIXED_DF && in.g.n >= (1LL << 22);
 }
+bool forms_dir(const Inst& in) { return in.pv2 != nullptr; }
 PcgDir pcg_dir(const Inst& in) { return PcgDir{in.zp, {in.pv, in.pv2}}; }
 PcgZr pcg_zr(const Inst& in, double* z) {
   return PcgZr{z, in.r, {in.pv, forms_dir(in) ? in.pv2 : in.pv}, in.q, in.partials, in.sc};
@@ -656,8 +658,6 @@ int mfg_plan(const mfg_problem* probs, int batch, mfg_plan_t* out) {
         cudaMalloc(&in.q, n * 8) != cudaSuccess || cudaMalloc(&in.zp, n * 8) != cudaSuccess ||
         cudaMalloc(&in.partials, npart * 8) != cudaSuccess)
       return bail(MFG_ERR_CUDA, "cudaMalloc failed for solver workspace");
-    if (forms_dir(in) && cudaMalloc(&in.pv2, n * 8) != cudaSuccess)
-      return bail(MFG_ERR_CUDA, "cudaMalloc failed for solver workspace");
     if (in.p.precision != MFG_FP64) {
       if (cudaMalloc(&in.work32, 2 * n * 4) != cudaSuccess)
         return bail(MFG_ERR_CUDA, "cudaMalloc failed for FP32 workspace");
@@ -678,6 +678,11 @@ int mfg_plan(const mfg_problem* probs, int batch, mfg_plan_t* out) {
   if (cudaStreamCreateWithFlags(&pl->cap0, cudaStreamNonBlocking) != cudaSuccess ||
       cudaStreamCreateWithFlags(&pl->cap1, cudaStreamNonBlocking) != cudaSuccess)
     return bail(MFG_ERR_CUDA, "cudaStreamCreate failed");
+  for (auto& in : pl->inst)
+    if (wants_dir(in) && cudaMalloc(&in.pv2, (size_t)in.g.n * 8) != cudaSuccess) {
+      in.pv2 = nullptr;
+      cudaGetLastError();  // no room: the separate pass
+    }
   *out = pl;
   return MFG_OK;
 }
