@@ -335,10 +335,10 @@ def kernels_measure(L, dev, stream, peak_gbs):
         L.mfg_prox_step(plan, 0, 0.5, zd, y, ybar, V, W, stream=stream)
     # the in-solve primal step: reads z, y; writes y, ybar (y is overwritten in
     # place each repetition, which keeps the values in the same range)
-    out["prox step (k_prox_cp, in-solve)"] = entry(timed(prox_step), 128 * n, 128 * n, "FP64 issue")
+    out["prox step (k_prox_strip, in-solve)"] = entry(timed(prox_step), 128 * n, 128 * n, "FP64 issue")
     # P^-1 in 3 passes' worth of algorithmic bytes (FP64 in, FP64 out, FP32 in between:
     # 8 + 4 + 4 + 4 + 4 + 8); the five passes move 48 B per unknown
-    out["P^-1 apply, FP32, CUDA-core time pass"] = entry(
+    out["P^-1 apply, FP32, eliminated time pass"] = entry(
         timed(lambda: L.mfg_apply_precond(plan, 0, r, z, stream=stream)), 32 * n, 48 * n, "HBM / latency")
     plan_tc = L.mfg_plan(dict(p, precision="mixed_tc"))
     out["P^-1 apply, FP32, tensor-core time pass"] = entry(
