@@ -578,7 +578,8 @@ __global__ void __launch_bounds__(256, kProxPerSm) k_prox_strip(Geom g, StripGri
           double b[NW];
 #pragma unroll
           for (int q = 0; q < NW; ++q) {
-            b[q] = 0.0;
+            // a skipped component: old value 0, new value 0, or NaN in a cell whose m is NaN
+            b[q] = w_new[q];
             if (act & (1u << q)) b[q] = fma(theta, w_new[q] - x.w[q], w_new[q]);
           }
           if (!own) return;
