@@ -69,7 +69,10 @@ __global__ void __launch_bounds__(kThreads) k_hinv(Geom g, Coef cf, const double
 #pragma unroll
     for (int q = 0; q < NW; ++q) {
       uw[q] = u[e + (q + 1) * n];
-      v[q] = on ? y[e + (q + 1) * n] * im : 0.0;
+      const double w = y[e + (q + 1) * n];
+      v[q] = on ? w * im : 0.0;
+      // w != 0 marks an active component: a quotient that underflows keeps the mark
+      if (on && w != 0.0 && v[q] == 0.0) v[q] = __longlong_as_double(1);
       vel[e + q * n] = v[q];
     }
     vel[e + NW * n] = iap;
