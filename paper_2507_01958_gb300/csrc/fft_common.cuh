@@ -30,7 +30,7 @@ struct DotFuse {
 struct ZrFuse {
   double* z;
   double* r;
-  const double* p[2];  // even and odd iterations (PcgZr)
+  const double* p;
   const double* q;
   double* partials;
   DevScalars* sc;

@@ -86,13 +86,11 @@ __global__ void __launch_bounds__(kThreads) k_init_p(long long n, const double* 
 
 // z += alpha p; r -= alpha q; rr = r.r; convergence test.
 __global__ void __launch_bounds__(kThreads) k_update_zr(long long n, double* __restrict__ z,
-                                                        double* __restrict__ r, const double* __restrict__ p0,
-                                                        const double* __restrict__ p1,
+                                                        double* __restrict__ r, const double* __restrict__ p,
                                                         const double* __restrict__ q, double* partials,
                                                         DevScalars* sc) {
   dep_sync();
   if (sc->cg_done) return;
-  const double* __restrict__ p = (sc->cg_it & 1) ? p1 : p0;
   const double alpha = sc->alpha;
   double acc = 0.0;
   const bool vec = aligned16(z, r, p, q);
@@ -169,8 +167,9 @@ void launch_init_p(long long n, const double* zp, double* p, const double* r, do
                    DevScalars* sc, cudaStream_t s, int cap) {
   launch_k(k_init_p, red_blocks(n, cap), kThreads, 0, s, n, zp, p, r, partials, sc);
 }
-void launch_update_zr(long long n, const PcgZr& zr, cudaStream_t s, int cap) {
-  launch_k(k_update_zr, red_blocks(n, cap), kThreads, 0, s, n, zr.z, zr.r, zr.p[0], zr.p[1], zr.q, zr.partials, zr.sc);
+void launch_update_zr(long long n, double* z, double* r, const double* p, const double* q,
+                      double* partials, DevScalars* sc, cudaStream_t s, int cap) {
+  launch_k(k_update_zr, red_blocks(n, cap), kThreads, 0, s, n, z, r, p, q, partials, sc);
 }
 void launch_dot_beta(long long n, const double* r, const double* zp, const double* q, int flexible,
                      double* partials, DevScalars* sc, cudaStream_t s, int cap) {
@@ -184,8 +183,7 @@ void launch_update_p(long long n, const double* zp, double* p, DevScalars* sc,
   launch_k(k_update_p, red_blocks(n, cap), kThreads, 0, s, n, zp, p, sc, h, use_handle);
 }
 
-// Inside the graph: arms the inner while-node (start of a CP iteration) and keeps
-// it running (end of a PCG iteration whose AAt pass forms the next direction).
+// Start of a CP iteration inside the graph: arms the inner while-node.
 __global__ void k_scalars_begin(DevScalars* sc, cudaGraphConditionalHandle h, int use_handle) {
   dep_sync();
   if (threadIdx.x == 0 && use_handle) cudaGraphSetConditional(h, sc->cg_done ? 0u : 1u);

@@ -109,7 +109,6 @@ __global__ void __launch_bounds__(256) k_fft(const TI* __restrict__ in, TO* __re
   };
   double rr = 0.0;
   const double alpha = ZR ? zf.sc->alpha : 0.0;
-  const double* __restrict__ zp_dir = ZR ? ((zf.sc->cg_it & 1) ? zf.p[1] : zf.p[0]) : nullptr;
 #pragma unroll 1
   for (int b0 = 0; b0 < PER; b0 += BL) {
     int ls[BL], is[BL];
@@ -126,7 +125,7 @@ __global__ void __launch_bounds__(256) k_fft(const TI* __restrict__ in, TO* __re
 #pragma unroll
       for (int u = 0; u < BL; ++u) {
         zv[u] = lv[u] ? zf.z[ad[u]] : 0.0;
-        pv[u] = lv[u] ? zp_dir[ad[u]] : 0.0;
+        pv[u] = lv[u] ? zf.p[ad[u]] : 0.0;
         rv[u] = lv[u] ? zf.r[ad[u]] : 0.0;
         qv[u] = lv[u] ? zf.q[ad[u]] : 0.0;
       }
@@ -418,7 +417,7 @@ void fft_y_forward(int N, int periodic, const double* in, T* out, const T* tw, c
                    long long nlines, const DevScalars* sc, cudaStream_t s, const PcgZr* zr) {
   if (!fft_pow2(N)) return fft_mixed_y_forward<T>(N, periodic, in, out, tw, dct, nlines, sc, s, zr);
   if (zr) {
-    ZrFuse zf{zr->z, zr->r, {zr->p[0], zr->p[1]}, zr->q, zr->partials, zr->sc};
+    ZrFuse zf{zr->z, zr->r, zr->p, zr->q, zr->partials, zr->sc};
     if (periodic)
       dispatch<T, FFT_DHT, true, double, T, false, true>(N, in, out, tw, dct, 1, 1, nlines, sc, s, DotFuse{}, zf);
     else

@@ -247,7 +247,6 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 2 : 3) k_fft_mixed(co
   };
   double rr = 0.0;
   const double alpha = ZR ? zf.sc->alpha : 0.0;
-  const double* __restrict__ zp_dir = ZR ? ((zf.sc->cg_it & 1) ? zf.p[1] : zf.p[0]) : nullptr;
   // loads in batches, all of a batch issued before the first is used
   constexpr int BL = ZR ? 4 : 8;
   for (int e0 = tid; e0 < total; e0 += nth * BL) {
@@ -261,7 +260,7 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 2 : 3) k_fft_mixed(co
 #pragma unroll
       for (int u = 0; u < BL; ++u) {
         zv[u] = lv[u] ? zf.z[ad[u]] : 0.0;
-        pv[u] = lv[u] ? zp_dir[ad[u]] : 0.0;
+        pv[u] = lv[u] ? zf.p[ad[u]] : 0.0;
         rv[u] = lv[u] ? zf.r[ad[u]] : 0.0;
         qv[u] = lv[u] ? zf.q[ad[u]] : 0.0;
       }
@@ -415,7 +414,7 @@ void fft_mixed_y_forward(int N, int periodic, const double* in, T* out, const T*
   const int mode = periodic ? FFT_DHT : FFT_DCT2;
   if (zr)
     launch_mixed<T, double, T, true, false, true>(N, mode, in, out, tw, dct, 1, 1, nlines, sc, s, DotFuse{},
-                                                  ZrFuse{zr->z, zr->r, {zr->p[0], zr->p[1]}, zr->q, zr->partials, zr->sc});
+                                                  ZrFuse{zr->z, zr->r, zr->p, zr->q, zr->partials, zr->sc});
   else
     launch_mixed<T, double, T, true>(N, mode, in, out, tw, dct, 1, 1, nlines, sc, s);
 }

@@ -533,7 +533,7 @@ static void precond_typed(const Geom& g, const T* Hx, const T* Hy, const T* V, c
   if (fy) {
     fft_y_forward<T>(g.ny, g.pery, r, w0, twy, dcty, n / g.ny, sc, s, zr);
   } else {
-    if (zr) launch_update_zr(n, *zr, s, g.vec_blocks);
+    if (zr) launch_update_zr(n, zr->z, zr->r, zr->p, zr->q, zr->partials, zr->sc, s, g.vec_blocks);
     axis_pass<double, T, T>(r, w0, Hy, g.ny, 1, n / g.ny, 0, sc, s);
   }
   T* a = w0;
@@ -575,7 +575,7 @@ void launch_precond(const Geom& g, const PrecTables& t, int precision, const dou
                     double* work64, float* work32, const DevScalars* sc, cudaStream_t s,
                     const PcgDot* dot, const PcgZr* zr) {
   if (t.band_w > 0) {  // viscosity field: time transforms around banded per-frequency solves
-    if (zr) launch_update_zr(g.n, *zr, s, g.vec_blocks);
+    if (zr) launch_update_zr(g.n, zr->z, zr->r, zr->p, zr->q, zr->partials, zr->sc, s, g.vec_blocks);
     launch_precond_band(g, t, precision, r, z, work64, work32, sc, s);
     if (dot) launch_dot_beta(g.n, dot->r, z, dot->q, dot->flex, dot->partials, dot->sc, s, g.vec_blocks);
     return;

@@ -19,7 +19,7 @@
 namespace mfg {
 
 // 256-thread blocks per SM that the launch bounds of the strip kernels admit
-constexpr int kCPerSm = 2, kCtPerSm = 3, kUPerSm = 5, kUDirPerSm = 3, kQPerSm = 3;
+constexpr int kCPerSm = 2, kCtPerSm = 3, kUPerSm = 5, kQPerSm = 3;
 
 // Whether C and C^T run in strips: not for viscosity fields, and not where the
 // strips would be less than ~60 % full (the point-by-point kernels issue 28 and 23 FP64
@@ -424,60 +424,35 @@ AatCoef aat_coef(const Geom& g) {
                  g.nu * dt, g.nu * ay * g.idt, g.nu * ax * g.idt, g.nu * cK * g.idt + idt2, dt, g.idt};
 }
 
-// DIR (PCG): p is formed on the way, zp + beta p_{it-1} per value loaded (again for the
-// strip's borders), and stored; a separate pass over zp and p cost 24 bytes per point
-// and a launch (512^2 x 128: 155 us).
-template <bool ISO, bool DIR>
-__global__ void __launch_bounds__(256, DIR ? kUDirPerSm : kUPerSm) k_aat_u(Geom g, AatCoef a, StripGrid ag,
-                                                                          const double* __restrict__ p,
-                                                                          PcgDir dir, double* __restrict__ U,
-                                                                          double* __restrict__ Sx,
-                                                                          const DevScalars* sc, int mode) {
+template <bool ISO>
+__global__ void __launch_bounds__(256, kUPerSm) k_aat_u(Geom g, AatCoef a, StripGrid ag, const double* __restrict__ p,
+                                               double* __restrict__ U, double* __restrict__ Sx,
+                                               const DevScalars* sc, int mode) {
   dep_sync();
   if (mode != 0 && sc->cg_done) return;
   int j0, i0, i1, k;
   if (!strip_item(ag, g, j0, i0, i1, k)) return;
   const long long base = (long long)k * g.S;
+  const double* pk = p + base;
   const int j = j0 + (threadIdx.x & 31);
-  const int it = DIR ? sc->cg_it : 0;
-  if (DIR && it > 0) {
-    const double beta = sc->beta;
-    const double* zk = dir.zp + base;
-    const double* po = ((it & 1) ? dir.p[0] : dir.p[1]) + base;
-    double* pn = ((it & 1) ? dir.p[1] : dir.p[0]) + base;
-    sum_march<ISO, 4>(g, a.rho, i0, i1, j0,
-                      [&](int i, int jj) { return fma(beta, po[i * g.ny + jj], zk[i * g.ny + jj]); },
-                      [](int) { return 0; }, [&](int i, double c, double sum, int) {
-                        if (j >= g.ny) return;
-                        const double u = fma(a.m2r, c, sum);
-                        const int f = i * g.ny + j;
-                        pn[f] = c;
-                        U[base + f] = u;
-                        Sx[base + f] = fma(-a.alpha, u, c);
-                      });
-    return;
-  }
-  const double* pk = (DIR ? dir.p[0] : p) + base;
   sum_march<ISO, 4>(g, a.rho, i0, i1, j0, [&](int i, int jj) { return pk[i * g.ny + jj]; },
                     [](int) { return 0; }, [&](int i, double c, double sum, int) {
-                      if (j >= g.ny) return;
-                      const double u = fma(a.m2r, c, sum);
-                      const int f = i * g.ny + j;
-                      U[base + f] = u;
-                      Sx[base + f] = fma(-a.alpha, u, c);
-                    });
+                   if (j >= g.ny) return;
+                   const double u = fma(a.m2r, c, sum);
+                   const long long e = base + (long long)i * g.ny + j;
+                   U[e] = u;
+                   Sx[e] = fma(-a.alpha, u, c);
+                 });
 }
 
 // q = AAt p; STEP (PCG step): also reduces p.q and sets alpha = rz/(p.q) in the
 // device scalars.
 template <bool ISO, bool STEP>
 __global__ void __launch_bounds__(256, kQPerSm) k_aat_q2(Geom g, AatCoef a, StripGrid ag, const double* __restrict__ U,
-                                                   const double* __restrict__ Sx, const double* __restrict__ p0,
-                                                   const double* __restrict__ p1, double* __restrict__ q,
-                                                   double* partials, DevScalars* sc) {
+                                                   const double* __restrict__ Sx, const double* __restrict__ p,
+                                                   double* __restrict__ q, double* partials, DevScalars* sc) {
   dep_sync();
   if (STEP && sc->cg_done) return;
-  const double* __restrict__ p = STEP && (sc->cg_it & 1) ? p1 : p0;
   double acc = 0.0;
   int j0, i0, i1, k;
   if (strip_item(ag, g, j0, i0, i1, k)) {
@@ -708,7 +683,7 @@ __global__ void __launch_bounds__(AJ * AI) k_aat_q_df(Geom g, AatCoef ad, int kc
 }
 
 void launch_AAt(const Geom& g, const double* p, double* q, double* scratch, double* partials,
-                DevScalars* sc, int mode, cudaStream_t s, int df64, const PcgDir* dir) {
+                DevScalars* sc, int mode, cudaStream_t s, int df64) {
   const AatCoef a = aat_coef(g);
   const int kc = aat2_chunk(g);
   const dim3 grid = aat2_grid(g, kc), block(AJ, AI);
@@ -736,19 +711,17 @@ void launch_AAt(const Geom& g, const double* p, double* q, double* scratch, doub
     }
     return;
   }
-  const StripGrid ug = strip_grid(g, dir ? kUDirPerSm : kUPerSm), ag = strip_grid(g, kQPerSm);
+  const StripGrid ug = strip_grid(g, kUPerSm), ag = strip_grid(g, kQPerSm);
+  const int nth = 32 * ag.warps;
   const bool iso = g.actx && g.ax == g.ay, step = mode != 0;
-  const double* p0 = dir ? dir->p[0] : p;
-  const double* p1 = dir ? dir->p[1] : p;
-  const PcgDir d = dir ? *dir : PcgDir{};
-#define MFG_AAT_U(I, D) launch_k(k_aat_u<I, D>, ug.blocks, 32 * ug.warps, 0, s, g, a, ug, p, d, X, KP, sc, mode)
-#define MFG_AAT(I, ST) launch_k(k_aat_q2<I, ST>, ag.blocks, 32 * ag.warps, 0, s, g, a, ag, X, KP, p0, p1, q, partials, sc)
-  if (iso) { if (dir) MFG_AAT_U(true, true); else MFG_AAT_U(true, false); }
-  else     { if (dir) MFG_AAT_U(false, true); else MFG_AAT_U(false, false); }
+#define MFG_AAT(I, ST) launch_k(k_aat_q2<I, ST>, ag.blocks, nth, 0, s, g, a, ag, X, KP, p, q, partials, sc)
+  if (iso)
+    launch_k(k_aat_u<true>, ug.blocks, 32 * ug.warps, 0, s, g, a, ug, p, X, KP, sc, mode);
+  else
+    launch_k(k_aat_u<false>, ug.blocks, 32 * ug.warps, 0, s, g, a, ug, p, X, KP, sc, mode);
   if (iso) { if (step) MFG_AAT(true, true); else MFG_AAT(true, false); }
   else     { if (step) MFG_AAT(false, true); else MFG_AAT(false, false); }
 #undef MFG_AAT
-#undef MFG_AAT_U
 }
 
 int aat_kernel_count(int) { return 2; }

@@ -8,8 +8,8 @@
 //   zp = P^{-1} r                     preconditioner passes (Alg. 1 + Alg. 2)
 //   p = zp, rz = r.zp                 k_init_p
 //   arm the inner while-node          k_scalars_begin
-//   while (!converged): p = zp + beta p (from the second iteration) in the first AAt
-//                       pass; q = AAt p; z += alpha p, r -= alpha q; zp = P^{-1} r; beta
+//   while (!converged): q = AAt p; z += alpha p, r -= alpha q; zp = P^{-1} r;
+//                       beta; p = zp + beta p
 //   prox + extrapolation + step sizes k_prox_cp (decides whether to loop again)
 // Batched instances are independent branches of the same graph, so the
 // runtime may overlap them on the GPU.  All control flow (convergence tests,
@@ -54,7 +54,7 @@ struct Inst {
   Coef cf{};
   PrecTables tabs{};
   size_t field_off = 0, primal_off = 0, dual_off = 0;
-  double *r = nullptr, *pv = nullptr, *pv2 = nullptr, *q = nullptr, *zp = nullptr, *work64 = nullptr;
+  double *r = nullptr, *pv = nullptr, *q = nullptr, *zp = nullptr, *work64 = nullptr;
   float* work32 = nullptr;
   double* partials = nullptr;
   DevScalars* sc = nullptr;  // points into the plan's contiguous array
@@ -179,10 +179,10 @@ namespace {
 
 void free_inst(Inst& in) {
   free_prec_tables(&in.tabs);
-  void* ptrs[] = {in.r, in.pv, in.pv2, in.q, in.zp, in.work64, in.work32, in.partials, in.adj_t, in.adj_eta, in.adj_vel, in.Az};
+  void* ptrs[] = {in.r, in.pv, in.q, in.zp, in.work64, in.work32, in.partials, in.adj_t, in.adj_eta, in.adj_vel, in.Az};
   for (void* q : ptrs)
     if (q) cudaFree(q);
-  in.r = in.pv = in.pv2 = in.q = in.zp = in.work64 = in.partials = in.adj_t = in.adj_eta = in.adj_vel = in.Az = nullptr;
+  in.r = in.pv = in.q = in.zp = in.work64 = in.partials = in.adj_t = in.adj_eta = in.adj_vel = in.Az = nullptr;
   in.work32 = nullptr;
 }
 
@@ -214,20 +214,6 @@ int launches_solve(const Inst& in) { return in.Az ? aat_kernel_count(in.p.precis
 void launch_stop_reference_start(const Inst& in, const double* z, cudaStream_t s) {
   if (!in.Az) return;
   launch_AAt(in.g, z, in.Az, in.work64, in.partials, in.sc, 0, s, in.p.precision == MFG_MIXED_DF);
-}
-// Whether the AAt pass of a PCG iteration forms the search direction itself
-// (constant viscosity, FP64 stencil), two direction buffers alternating; else
-// k_update_p updates the one.  From 2^22 points on, where the vectors no longer stay
-// in L2 between passes: the 512^2 x 128 solve 136.3 -> 133.9 ms; four 128^2 x 64 tori
-// 23.9 -> 24.2 ms, so smaller instances keep the separate pass, and so does one whose
-// second buffer no longer fits beside the rest of the plan.
-bool wants_dir(const Inst& in) {
-  return in.g.kfy == nullptr && in.p.precision != MFG_MIXED_DF && in.g.n >= (1LL << 22);
-}
-bool forms_dir(const Inst& in) { return in.pv2 != nullptr; }
-PcgDir pcg_dir(const Inst& in) { return PcgDir{in.zp, {in.pv, in.pv2}}; }
-PcgZr pcg_zr(const Inst& in, double* z) {
-  return PcgZr{z, in.r, {in.pv, forms_dir(in) ? in.pv2 : in.pv}, in.q, in.partials, in.sc};
 }
 int launches_cg(const Inst& in) {
   return 1 + aat_kernel_count(in.p.precision == MFG_MIXED_DF) + precond_step_kernel_count(in.g, in.tabs);
@@ -290,14 +276,10 @@ int add_instance(mfg_plan_t pl, Inst& in, cudaGraph_t top, const double* m0, con
   cudaStream_t s2 = pl->cap1;
   CK(cudaStreamBeginCaptureToGraph(s2, body_cg, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
   const PcgDot dot{in.r, in.q, in.partials, in.sc, flex};
-  const PcgZr zr = pcg_zr(in, z);
-  const PcgDir dir = pcg_dir(in);
-  launch_AAt(g, in.pv, in.q, in.work64, in.partials, in.sc, 1, s2, dfa, forms_dir(in) ? &dir : nullptr);
+  const PcgZr zr{z, in.r, in.pv, in.q, in.partials, in.sc};
+  launch_AAt(g, in.pv, in.q, in.work64, in.partials, in.sc, 1, s2, dfa);
   launch_precond(g, in.tabs, in.p.precision, in.r, in.zp, in.work64, in.work32, in.sc, s2, &dot, &zr);
-  if (forms_dir(in))
-    launch_scalars_begin(in.sc, hg, 1, s2);
-  else
-    launch_update_p(g.n, in.zp, in.pv, in.sc, hg, 1, s2, g.vec_blocks);
+  launch_update_p(g.n, in.zp, in.pv, in.sc, hg, 1, s2, g.vec_blocks);
   CK(cudaStreamEndCapture(s2, &body_cg));
   return MFG_OK;
 }
@@ -354,12 +336,11 @@ int solve_eager(mfg_plan_t pl, const double* m0, const double* V, const double* 
         CK(cudaStreamSynchronize(s));
         if (hs.cg_done) break;
         const PcgDot dot{in.r, in.q, in.partials, in.sc, flex};
-        const PcgZr zr = pcg_zr(in, zb);
-        const PcgDir dir = pcg_dir(in);
-        launch_AAt(g, in.pv, in.q, in.work64, in.partials, in.sc, 1, s, dfa, forms_dir(in) ? &dir : nullptr);
+        const PcgZr zr{zb, in.r, in.pv, in.q, in.partials, in.sc};
+        launch_AAt(g, in.pv, in.q, in.work64, in.partials, in.sc, 1, s, dfa);
         launch_precond(g, in.tabs, in.p.precision, in.r, in.zp, in.work64, in.work32, in.sc, s, &dot, &zr);
-        if (!forms_dir(in)) launch_update_p(g.n, in.zp, in.pv, in.sc, 0, 0, s, g.vec_blocks);
-        pl->launches += launches_cg(in) - (forms_dir(in) ? 1 : 0);  // nothing arms a graph node
+        launch_update_p(g.n, in.zp, in.pv, in.sc, 0, 0, s, g.vec_blocks);
+        pl->launches += launches_cg(in);
       }
       launch_prox_cp(g, in.cf, zb, yb, ybb, Vb, Wb, in.partials, in.sc, 0, 0, s, in.Az, in.r);
       pl->launches += 1;
@@ -474,7 +455,7 @@ int tune_instance(Inst& in, double* zbuf, cudaStream_t s, cudaEvent_t a, cudaEve
           c.fft_y = fy;
           c.fft_x = fx;
           const PcgDot dot{in.r, in.q, in.partials, in.sc, flex};
-          const PcgZr zr{zbuf, in.r, {in.pv, in.pv}, in.q, in.partials, in.sc};
+          const PcgZr zr{zbuf, in.r, in.pv, in.q, in.partials, in.sc};
           if ((rc = reset_tune_scalars(in, s))) return rc;
           const double t = time_us([&] {
             launch_precond(c, in.tabs, in.p.precision, in.r, in.zp, in.work64, in.work32, in.sc, s, &dot, &zr);
@@ -678,11 +659,6 @@ int mfg_plan(const mfg_problem* probs, int batch, mfg_plan_t* out) {
   if (cudaStreamCreateWithFlags(&pl->cap0, cudaStreamNonBlocking) != cudaSuccess ||
       cudaStreamCreateWithFlags(&pl->cap1, cudaStreamNonBlocking) != cudaSuccess)
     return bail(MFG_ERR_CUDA, "cudaStreamCreate failed");
-  for (auto& in : pl->inst)
-    if (wants_dir(in) && cudaMalloc(&in.pv2, (size_t)in.g.n * 8) != cudaSuccess) {
-      in.pv2 = nullptr;
-      cudaGetLastError();  // no room: the separate pass
-    }
   *out = pl;
   return MFG_OK;
 }
@@ -874,7 +850,7 @@ int mfg_adjoint(mfg_plan_t pl, int b, const double* y, const double* z, const do
   CK(post(0));
   for (int i = 0;; ++i) {
     const PcgDot dot{in.r, in.q, in.partials, in.sc, flex};
-    const PcgZr zr{in.adj_eta, in.r, {in.pv, in.pv}, in.q, in.partials, in.sc};
+    const PcgZr zr{in.adj_eta, in.r, in.pv, in.q, in.partials, in.sc};
     launch_ct_hinv(g, y, in.adj_vel, in.pv, nullptr, in.adj_t, s, in.sc);
     launch_apply_C(g, in.adj_t, in.q, 1.0, nullptr, in.partials, in.sc, 2, s, in.pv);
     launch_precond(g, in.tabs, in.p.precision, in.r, in.zp, in.work64, in.work32, in.sc, s, &dot, &zr);

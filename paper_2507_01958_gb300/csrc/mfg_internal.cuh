@@ -119,14 +119,6 @@ void launch_k(void (*kernel)(KA...), dim3 grid, dim3 block, size_t smem, cudaStr
   cudaLaunchKernelEx(&c, kernel, std::forward<A>(args)...);
 }
 
-// Search directions of a PCG loop whose AAt pass forms p_it = zp + beta p_{it-1}
-// itself: iteration it (DevScalars::cg_it) has its direction in p[it & 1] (the pass reads
-// neighbours of p_{it-1}, so it cannot be overwritten in place); p_0 is there on entry.
-struct PcgDir {
-  const double* zp;
-  double* p[2];
-};
-
 // ---------------------------------------------------------------- kernels --
 // Stencils (k_stencil.cu).
 // Az (mode 1 only, MFG_CG_REF_RHS): AAt z_l on entry, b = AAt z_l + r on exit.
@@ -136,10 +128,8 @@ void launch_apply_C(const Geom& g, const double* v, double* r, double alpha, con
 void launch_apply_Ct(const Geom& g, const double* p, double* x, cudaStream_t s);
 // df64 != 0 selects the double-float variant of the stencil (MFG_MIXED_DF).
 // q = AAt p.  scratch: 2 n doubles.  mode 0: plain apply; 1: PCG step (p.q, alpha).
-// dir != nullptr (mode 1, constant viscosity, no double-float): the step also forms
-// its search direction, p = zp + beta p (see PcgDir).
 void launch_AAt(const Geom& g, const double* p, double* q, double* scratch, double* partials,
-                DevScalars* sc, int mode, cudaStream_t s, int df64, const PcgDir* dir = nullptr);
+                DevScalars* sc, int mode, cudaStream_t s, int df64);
 int aat_kernel_count(int df64);
 int aat_blocks(const Geom& g);
 bool strips_fit(const Geom& g);
@@ -148,8 +138,8 @@ bool strips_fit(const Geom& g);
 // `cap`: grid cap (Geom::vec_blocks).
 void launch_init_p(long long n, const double* zp, double* p, const double* r, double* partials,
                    DevScalars* sc, cudaStream_t s, int cap = kRedBlocks);
-struct PcgZr;
-void launch_update_zr(long long n, const PcgZr& zr, cudaStream_t s, int cap = kRedBlocks);
+void launch_update_zr(long long n, double* z, double* r, const double* p, const double* q,
+                      double* partials, DevScalars* sc, cudaStream_t s, int cap = kRedBlocks);
 void launch_dot_beta(long long n, const double* r, const double* zp, const double* q, int flexible,
                      double* partials, DevScalars* sc, cudaStream_t s, int cap = kRedBlocks);
 void launch_update_p(long long n, const double* zp, double* p, DevScalars* sc,
@@ -205,7 +195,7 @@ struct PcgDot {
 struct PcgZr {
   double* z;
   double* r;
-  const double* p[2];  // direction of even and odd iterations (PcgDir; both the same otherwise)
+  const double* p;
   const double* q;
   double* partials;
   DevScalars* sc;
