@@ -19,7 +19,7 @@
 namespace mfg {
 
 // 256-thread blocks per SM that the launch bounds of the strip kernels admit
-constexpr int kCPerSm = 2, kCtPerSm = 3, kUPerSm = 5, kQPerSm = 3;
+constexpr int kCPerSm = 2, kCtPerSm = 3, kUPerSm = 4, kQPerSm = 3;
 
 // Whether C and C^T run in strips: not for viscosity fields, and not where the
 // strips would be less than ~60 % full (the point-by-point kernels issue 28 and 23 FP64
@@ -389,67 +389,74 @@ void launch_apply_Ct(const Geom& g, const double* p, double* x, cudaStream_t s) 
 // ---------------------------------------------------------------- C C^T p --
 // FP64 issue is the limit on GB300 (a warp's FP64 instruction takes 16 SM
 // clocks; the bytes moved take a third of that time), so the operator is
-// arranged for the fewest FP64 instructions per point.  With K p = -ay u,
-//   u = (p_S + p_N) + rho (p_W + p_E) - 2 (1 + rho) p,   rho = ax / ay,
-// and BB^T = 2K (eq. precstead), C C^T = L^2 in space, a second difference in
-// time, becomes
-//   q^k = (2 s^k - s^{k-1} - s^{k+1}) / dt^2 + nu^2 ay^2 U(u^k) - 2 ay u^k,
-//   s = p - nu ay dt u,   s^{-1} := p^0,   s^{N_t} := 0,
-// U the operator that takes p to u: two passes over the grid, each point
-// computed once, u and s through memory.
+// arranged for the fewest FP64 instructions per point.  Factored form
+// q = C (C^T p): with x^k = L p^k - p^{k+1}/dt (the m rows of C^T p, p^{N_t} := 0)
+// and BB^T = 2K (eq. precstead),
+//   q^k = L x^k - x^{k-1}/dt + 2 K p^k        (x^{-1} := 0),
+// in two passes over the grid, each point computed once.  With K p = -ay u,
+//   u = (p_S + p_N) + rho (p_W + p_E) - 2 (1 + rho) p,   rho = ax / ay:
+//   pass 1:  u,  X = dt x = (p^k - p^{k+1}) - nu ay dt u
+//   pass 2:  q = c4 X - (X^{k-1}/dt^2 + c1 sum(X) + 2 ay u),   c1 = nu ay/dt,
+//            c4 = 2 (1 + rho) c1 + 1/dt^2, sum the neighbour sum of u's formula.
+// The time differences are formed from neighbouring planes of p, exactly where p
+// varies slowly; a second difference of p - nu ay dt u (the same number of
+// instructions) rounds at the size of p/dt^2, 10 to 35 times as far off for fields
+// smooth in time on grids with 1/dt^2 >> ay (8^2 x 200: 2e-16 against 8e-15).
 // Square cells (rho = 1) share the diagonal pair sums A(i, j) = p(i, j+1) + p(i+1, j):
 //   p_N + p_S + p_W + p_E = A(i, j) + A(i-1, j-1),
-// one addition less per point and pass.  FP64 instructions per point: 4 + 8
-// with p.q (6 + 9 when rho != 1), against 15 for the factored form
-// L (L p^k - p^{k+1}/dt) - ... with K p and L p through memory.
+// one addition less per point and pass.  FP64 instructions per point: 5 + 7
+// with p.q (6 + 8 when rho != 1).
 // On a Neumann axis the neighbour index of an end point is the point itself
 // (u_{-1} = u_0, u_N = u_{N-1}), which turns the same formula into the
-// one-sided D^1 (D^1)^T rows of Sec. 4.3, for p and for u alike.
+// one-sided D^1 (D^1)^T rows of Sec. 4.3, for p and for X alike.
 //
-// Both passes walk the grid in warp strips (strip.cuh).  512^2 x 128: 949 -> 756 us (11
-// FP64 instructions per point at 78 % of the FP64 pipe; 587 us at all of it).
+// Both passes walk the grid in warp strips (strip.cuh).  512^2 x 128: 748 us, 12 FP64
+// instructions per point (949 us one column per thread, 15 instructions).
 struct AatCoef {
   double rho, m2r;        // ax / ay, -2 (1 + rho)
   double alpha;           // nu ay dt
-  double b, gu, idt2;     // nu^2 ay^2, -2 (1 + rho) b - 2 ay, 1/dt^2
+  double ay2, c1, idt2, c4r;  // 2 ay, nu ay/dt, 1/dt^2, 2 (1 + rho) c1 + 1/dt^2
   double ax, ay, cK;      // viscosity field and double-float passes
-  double ndt, c1, c2, c4;
+  double ndt, c2, c4;
   double dt, idt;
 };
 
 AatCoef aat_coef(const Geom& g) {
   const double ax = g.actx ? g.ax : 0.0, ay = g.ay, cK = 2.0 * (ax + ay);
-  const double dt = 1.0 / g.idt, idt2 = g.idt * g.idt, rho = ax / ay, b = g.nu * ay * (g.nu * ay);
-  return AatCoef{rho, -2.0 * (1.0 + rho), g.nu * ay * dt, b, -2.0 * (1.0 + rho) * b - 2.0 * ay, idt2, ax, ay, cK,
-                 g.nu * dt, g.nu * ay * g.idt, g.nu * ax * g.idt, g.nu * cK * g.idt + idt2, dt, g.idt};
+  const double dt = 1.0 / g.idt, idt2 = g.idt * g.idt, rho = ax / ay, c1 = g.nu * ay * g.idt;
+  return AatCoef{rho, -2.0 * (1.0 + rho), g.nu * ay * dt, 2.0 * ay, c1, idt2, 2.0 * (1.0 + rho) * c1 + idt2, ax, ay, cK,
+                 g.nu * dt, g.nu * ax * g.idt, g.nu * cK * g.idt + idt2, dt, g.idt};
 }
 
 template <bool ISO>
 __global__ void __launch_bounds__(256, kUPerSm) k_aat_u(Geom g, AatCoef a, StripGrid ag, const double* __restrict__ p,
-                                               double* __restrict__ U, double* __restrict__ Sx,
-                                               const DevScalars* sc, int mode) {
+                                                        double* __restrict__ U, double* __restrict__ X,
+                                                        const DevScalars* sc, int mode) {
   dep_sync();
   if (mode != 0 && sc->cg_done) return;
   int j0, i0, i1, k;
   if (!strip_item(ag, g, j0, i0, i1, k)) return;
   const long long base = (long long)k * g.S;
+  const int j = j0 + (threadIdx.x & 31), jc = j < g.ny ? j : g.ny - 1;
+  const bool last = k + 1 >= g.nt;
   const double* pk = p + base;
-  const int j = j0 + (threadIdx.x & 31);
+  const double* pkn = pk + (last ? 0 : g.S);
   sum_march<ISO, 4>(g, a.rho, i0, i1, j0, [&](int i, int jj) { return pk[i * g.ny + jj]; },
-                    [](int) { return 0; }, [&](int i, double c, double sum, int) {
-                   if (j >= g.ny) return;
-                   const double u = fma(a.m2r, c, sum);
-                   const long long e = base + (long long)i * g.ny + j;
-                   U[e] = u;
-                   Sx[e] = fma(-a.alpha, u, c);
-                 });
+                    [&](int i) { return last ? 0.0 : pkn[i * g.ny + jc]; },
+                    [&](int i, double c, double sum, double next) {
+                      if (j >= g.ny) return;
+                      const double u = fma(a.m2r, c, sum);
+                      const int f = i * g.ny + j;
+                      U[base + f] = u;
+                      X[base + f] = fma(-a.alpha, u, c - next);
+                    });
 }
 
 // q = AAt p; STEP (PCG step): also reduces p.q and sets alpha = rz/(p.q) in the
 // device scalars.
 template <bool ISO, bool STEP>
 __global__ void __launch_bounds__(256, kQPerSm) k_aat_q2(Geom g, AatCoef a, StripGrid ag, const double* __restrict__ U,
-                                                   const double* __restrict__ Sx, const double* __restrict__ p,
+                                                   const double* __restrict__ X, const double* __restrict__ p,
                                                    double* __restrict__ q, double* partials, DevScalars* sc) {
   dep_sync();
   if (STEP && sc->cg_done) return;
@@ -457,23 +464,21 @@ __global__ void __launch_bounds__(256, kQPerSm) k_aat_q2(Geom g, AatCoef a, Stri
   int j0, i0, i1, k;
   if (strip_item(ag, g, j0, i0, i1, k)) {
     const long long base = (long long)k * g.S;
-    const double* uk = U + base;
+    const double* xk = X + base;
     const int j = j0 + (threadIdx.x & 31);
-    const double* sm = k > 0 ? Sx - g.S : p;  // s^{-1} := p^0
-    const bool last = k == g.nt - 1;
     struct Row {
-      double s0, sm, sp, p;
+      double u, xp, p;
     };
     const int jc = j < g.ny ? j : g.ny - 1;
-    sum_march<ISO, 4>(g, a.rho, i0, i1, j0, [&](int i, int jj) { return uk[i * g.ny + jj]; },
+    sum_march<ISO, 4>(g, a.rho, i0, i1, j0, [&](int i, int jj) { return xk[i * g.ny + jj]; },
                       [&](int i) {
                         const long long e = base + i * g.ny + jc;
-                        return Row{Sx[e], sm[e], last ? 0.0 : Sx[e + g.S], STEP ? p[e] : 0.0};
+                        return Row{U[e], k > 0 ? X[e - g.S] : 0.0, STEP ? p[e] : 0.0};
                       },
                       [&](int i, double c, double sum, const Row& w) {
                         if (j >= g.ny) return;
-                        const double dd = fma(2.0, w.s0, -(w.sm + w.sp));
-                        const double qv = fma(a.gu, c, fma(a.b, sum, a.idt2 * dd));
+                        const double t = fma(a.ay2, w.u, fma(a.c1, sum, a.idt2 * w.xp));
+                        const double qv = fma(a.c4r, c, -t);
                         q[base + i * g.ny + j] = qv;
                         if constexpr (STEP) acc = fma(qv, w.p, acc);
                       });
@@ -699,8 +704,8 @@ void launch_AAt(const Geom& g, const double* p, double* q, double* scratch, doub
     }
     return;
   }
-  double* X = scratch;  // u, or X = dt xm of a viscosity field
-  double* KP = scratch + g.n;  // s, or K p
+  double* X = scratch;
+  double* KP = scratch + g.n;  // K p of a viscosity field, else u
   if (g.kfy != nullptr) {
     if (g.actx) {
       launch_k(k_aat_x<1>, grid, block, 0, s, g, a, kc, p, X, KP, sc, mode);
@@ -714,11 +719,11 @@ void launch_AAt(const Geom& g, const double* p, double* q, double* scratch, doub
   const StripGrid ug = strip_grid(g, kUPerSm), ag = strip_grid(g, kQPerSm);
   const int nth = 32 * ag.warps;
   const bool iso = g.actx && g.ax == g.ay, step = mode != 0;
-#define MFG_AAT(I, ST) launch_k(k_aat_q2<I, ST>, ag.blocks, nth, 0, s, g, a, ag, X, KP, p, q, partials, sc)
+#define MFG_AAT(I, ST) launch_k(k_aat_q2<I, ST>, ag.blocks, nth, 0, s, g, a, ag, KP, X, p, q, partials, sc)
   if (iso)
-    launch_k(k_aat_u<true>, ug.blocks, 32 * ug.warps, 0, s, g, a, ug, p, X, KP, sc, mode);
+    launch_k(k_aat_u<true>, ug.blocks, 32 * ug.warps, 0, s, g, a, ug, p, KP, X, sc, mode);
   else
-    launch_k(k_aat_u<false>, ug.blocks, 32 * ug.warps, 0, s, g, a, ug, p, X, KP, sc, mode);
+    launch_k(k_aat_u<false>, ug.blocks, 32 * ug.warps, 0, s, g, a, ug, p, KP, X, sc, mode);
   if (iso) { if (step) MFG_AAT(true, true); else MFG_AAT(true, false); }
   else     { if (step) MFG_AAT(false, true); else MFG_AAT(false, false); }
 #undef MFG_AAT
