@@ -20,7 +20,6 @@
 #include "df64.cuh"
 #include "mfg_internal.cuh"
 #include "reduce.cuh"
-#include "strip.cuh"
 
 namespace mfg {
 
@@ -291,25 +290,20 @@ __device__ __forceinline__ ProxK prox_consts(double tau, double half_itau, doubl
 // from an FP32 root two steps reach the double-float resolution.  The polish
 // stops after a step below 1e-9 relative and keeps the bracket, bisecting if
 // a step leaves it.  Inputs outside the FP32 range take an FP64 Newton.
-// act: bit q set where some lane of the warp has a nonzero projection P_q; the
-// others are zero throughout and cost nothing.  (FP64 issue bounds the prox, so the
-// set-up takes as few FP64 instructions as it can: sign and zero tests on bit
-// patterns, the bracket in FP32, all FP32 values from the double-float splits.)
+// (FP64 issue bounds the prox, so the set-up takes as few FP64 instructions as it
+// can: sign and zero tests on bit patterns, the bracket in FP32, all FP32 values
+// from the double-float splits.)
 template <int NW>
 __device__ __forceinline__ void prox_cell(double mbar, const double (&wbar)[NW], const ProxK& K, double a1,
-                                          float a1f, const df& a1d, double c, double& m, double (&w)[NW],
-                                          unsigned act = ~0u) {
+                                          float a1f, const df& a1d, double c, double& m, double (&w)[NW]) {
   // projection onto K by sign tests on the bit patterns (no FP64 min/max)
   double P[NW];
   double P2 = 0.0;
 #pragma unroll
   for (int q = 0; q < NW; ++q) {
-    P[q] = 0.0;
-    if (act & (1u << q)) {
-      const bool neg = __double_as_longlong(wbar[q]) < 0;
-      P[q] = ((q & 1) ? neg : !neg) ? wbar[q] : 0.0;
-      P2 = fma(P[q], P[q], P2);
-    }
+    const bool neg = __double_as_longlong(wbar[q]) < 0;
+    P[q] = ((q & 1) ? neg : !neg) ? wbar[q] : 0.0;
+    P2 = fma(P[q], P[q], P2);
   }
   const double B = fma(-K.tau, c, mbar);
   const double hP = K.half_tau * P2;
@@ -366,10 +360,7 @@ __device__ __forceinline__ void prox_cell(double mbar, const double (&wbar)[NW],
   m = df_to_double(x);
   const double s = df_to_double(df_mul(x, r));
 #pragma unroll
-  for (int q = 0; q < NW; ++q) {
-    w[q] = 0.0;
-    if (act & (1u << q)) w[q] = s * P[q];
-  }
+  for (int q = 0; q < NW; ++q) w[q] = s * P[q];
 }
 
 // End of a CP step: acc = this thread's share of ||m_{l+1} - m_l||^2; the last
@@ -415,7 +406,10 @@ __device__ __forceinline__ void prox_tail(double acc, double tau, double theta, 
 // so the difference across the end (a flux slot of Sec. 4.3 that does not
 // exist) is zero and K takes its one-sided form.  VN (viscosity field): nu K z
 // becomes K_nu z = kf_yp dyp - kf_ym dym (+ x terms), the face coefficients of
-// Geom::kfx / kfy.  Point by point: viscosity fields and rows too short for strips.
+// Geom::kfx / kfy.  Point by point: a walk in warp strips forms each difference of z
+// once, but issues a row's loads only behind the previous row's roots, and was slower
+// at every width and occupation (256^2 x 128 755 us point by point, 934 us in strips;
+// 512 x 20 x 200 202, 373 us; 4000 x 250 in 1-D 77, 136 us).
 template <int ACTX, bool GENQ, bool VN>
 __global__ void __launch_bounds__(kThreads) k_prox_cp(Geom g, Coef cf, const double* __restrict__ z,
                                                       double* __restrict__ y, double* __restrict__ ybar,
@@ -494,108 +488,6 @@ __global__ void __launch_bounds__(kThreads) k_prox_cp(Geom g, Coef cf, const dou
   prox_tail(acc, tau, theta, cf.gamma, partials, sc, h, use_handle);
 }
 
-constexpr int kProxPerSm = 2;  // 256-thread blocks per SM of the strip kernel
-
-// The same step in warp strips (strip.cuh; constant viscosity): each face difference
-// of z formed once, and the flux components that are zero across a whole warp, old
-// value and projection alike (half of them where the flow has one direction over 32 cells),
-// skip theirs.  54 FP64 instructions per cell on noisy data (~66 before, 68 with the
-// out-of-range paths of the double-float conversions inlined): 256^2 x 128 754 -> 627 us a
-// step, the 512^2 x 128 solve 140 -> 136 ms.
-template <int ACTX, bool GENQ>
-__global__ void __launch_bounds__(256, kProxPerSm) k_prox_strip(Geom g, StripGrid sg, Coef cf,
-                                                                const double* __restrict__ z,
-                                                                double* __restrict__ y, double* __restrict__ ybar,
-                                                                const double* __restrict__ V,
-                                                                const double* __restrict__ W, double* partials,
-                                                                DevScalars* sc, cudaGraphConditionalHandle h,
-                                                                int use_handle, double* __restrict__ Az,
-                                                                const double* __restrict__ rfin) {
-  dep_sync();
-  constexpr int NW = ACTX ? 4 : 2;
-  const double tau = sc->tau, theta = sc->theta;
-  double acc = 0.0;
-  int j0, i0, i1, k;
-  if (strip_item(sg, g, j0, i0, i1, k)) {
-    const ProxK K = prox_consts(tau, sc->half_itau, cf.f_b);
-    const bool last = k == g.nt - 1;
-    const double a1 = last ? fma(tau, fma(cf.g_a, g.idt, cf.f_a), 1.0) : fma(tau, cf.f_a, 1.0);
-    const float a1f = (float)a1;
-    const df a1d = df_from_double(a1);
-    const double t_idt = tau * g.idt, t_idx = tau * g.idx, t_idy = tau * g.idy, t_ny = tau * g.nu * g.ay,
-                 t_nx = tau * g.nu * g.ax;
-    const long long n = g.n, base = (long long)k * g.S;
-    const double* zk = z + base;
-    const int j = j0 + (threadIdx.x & 31), jc = j < g.ny ? j : g.ny - 1;
-    struct Row {
-      double zn, m, cc, w[NW];
-    };
-    diff_march<ACTX, false, 1>(
-        g, i0, i1, j0, [&](int i, int jj) { return zk[i * g.ny + jj]; },
-        [&](int i) {
-          const int f = i * g.ny + jc;
-          const long long e = base + f;
-          Row x;
-          x.zn = last ? 0.0 : z[e + g.S];
-          x.m = y[e];
-#pragma unroll
-          for (int q = 0; q < NW; ++q) x.w[q] = y[e + (q + 1) * n];
-          x.cc = last ? fma(W[f], g.idt, V[f]) : V[f];
-          return x;
-        },
-        [&](int i, double zc, double dyp, double dym, double dxp, double dxm, const Row& x) {
-          double d[NW];
-          if (ACTX) { d[0] = dxp; d[1] = dxm; }
-          d[NW - 2] = dyp;
-          d[NW - 1] = dym;
-          const bool own = j < g.ny;
-          unsigned act = 0;
-#pragma unroll
-          for (int q = 0; q < NW; ++q) {
-            // -d has the component's sign, or the old value is not zero
-            const bool neg = __double_as_longlong(d[q]) < 0, old = (__double_as_longlong(x.w[q]) << 1) != 0;
-            if (GENQ || __any_sync(0xffffffffu, (old || ((q & 1) ? !neg : neg)))) act |= 1u << q;
-          }
-          // (lanes past the last column run along on its cell and store nothing, so
-          // that the warp can meet again after the root)
-          const long long e = base + i * g.ny + j;
-          if (own && Az != nullptr) Az[e] -= rfin[e];  // AAt z_{l+1} = b - r_final (stop reference)
-          // primal step y - tau x, x_m = nu K z + (z - z_next)/dt, x_w = d / dx
-          double mbar = fma(-t_ny, dyp - dym, fma(-t_idt, zc - x.zn, x.m));
-          if (ACTX) mbar = fma(-t_nx, dxp - dxm, mbar);
-          double wbar[NW], w_new[NW], m_new;
-#pragma unroll
-          for (int q = 0; q < NW; ++q) {
-            wbar[q] = 0.0;
-            if (act & (1u << q)) wbar[q] = fma(-((ACTX && q < 2) ? t_idx : t_idy), d[q], x.w[q]);
-          }
-          if constexpr (GENQ)
-            prox_cell_q<NW>(mbar, wbar, tau, cf.qprime, a1, K.tb, x.cc, m_new, w_new);
-          else
-            prox_cell<NW>(mbar, wbar, K, a1, a1f, a1d, x.cc, m_new, w_new, act);
-          __syncwarp();
-          const double dm = m_new - x.m, mb = fma(theta, dm, m_new);
-          double b[NW];
-#pragma unroll
-          for (int q = 0; q < NW; ++q) {
-            // a skipped component: old value 0, new value 0, or NaN in a cell whose m is NaN
-            b[q] = w_new[q];
-            if (act & (1u << q)) b[q] = fma(theta, w_new[q] - x.w[q], w_new[q]);
-          }
-          if (!own) return;
-          acc = fma(dm, dm, acc);
-          y[e] = m_new;
-          ybar[e] = mb;
-#pragma unroll
-          for (int q = 0; q < NW; ++q) {
-            y[e + (q + 1) * n] = w_new[q];
-            ybar[e + (q + 1) * n] = b[q];
-          }
-        });
-  }
-  prox_tail(acc, tau, theta, cf.gamma, partials, sc, h, use_handle);
-}
-
 template <int ACTX, bool GENQ>
 __global__ void __launch_bounds__(kThreads) k_prox_plain(Geom g, Coef cf, double tau,
                                                          const double* v, double* y,
@@ -656,17 +548,6 @@ void launch_prox_cp(const Geom& g, const Coef& cf, const double* z, double* y, d
                     const double* V, const double* W, double* partials, DevScalars* sc,
                     cudaGraphConditionalHandle h, int use_handle, cudaStream_t s, double* Az,
                     const double* rfin) {
-  if (strips_fit(g)) {
-    const StripGrid sg = strip_grid(g, kProxPerSm);
-    const bool gq = cf.qprime != 2.0;
-#define MFG_PROX_STRIP(A, Q)                                                                                        \
-  launch_k(k_prox_strip<A, Q>, sg.blocks, 32 * sg.warps, 0, s, g, sg, cf, z, y, ybar, V, W, partials, sc, h, use_handle, \
-           Az, rfin)
-    if (g.actx) { if (gq) MFG_PROX_STRIP(1, true); else MFG_PROX_STRIP(1, false); }
-    else        { if (gq) MFG_PROX_STRIP(0, true); else MFG_PROX_STRIP(0, false); }
-#undef MFG_PROX_STRIP
-    return;
-  }
   const int idx = (g.actx ? 4 : 0) + (cf.qprime != 2.0 ? 2 : 0) + (g.kfy != nullptr ? 1 : 0);
   const int nb = red_blocks(g.n, g_prox_wave[idx]);
   // the general-q' root finder and the viscosity field are their own
