@@ -102,11 +102,11 @@ __global__ void __launch_bounds__(256, kCtHinvPerSm) k_ct_hinv(Geom g, StripGrid
   const double* pk = p + base;
   const int j = j0 + (threadIdx.x & 31), jc = j < g.ny ? j : g.ny - 1;
   const bool last = k + 1 >= g.nt;
-  const double nx = g.nu * g.idx, ny = g.nu * g.idy;  // nu K p from the scaled differences
+  const double nx = g.nu * g.ax, ny = g.nu * g.ay;
   struct Row {
     double pn, m, iap, v[NW], um, uw[NW];
   };
-  diff_march<ACTX, true, 2>(
+  diff_march<ACTX, 2>(
       g, i0, i1, j0, [&](int i, int jj) { return pk[i * g.ny + jj]; },
       [&](int i) {
         const long long e = base + i * g.ny + jc;
@@ -122,15 +122,15 @@ __global__ void __launch_bounds__(256, kCtHinvPerSm) k_ct_hinv(Geom g, StripGrid
         }
         return w;
       },
-      [&](int i, double pc, double dyp, double dym, double dxp, double dxm, const Row& w) {
+      [&](int i, double pc, const Diff& d, const Row& w) {
         if (j >= g.ny) return;
-        double xm = fma(ny, dyp - dym, (pc - w.pn) * g.idt), om, ow[NW];
+        double xm = fma(ny, d.yy, (pc - w.pn) * g.idt), om, ow[NW];
         double xw[NW];
         if (ACTX) {
-          xm = fma(nx, dxp - dxm, xm);
-          xw[0] = dxp; xw[1] = dxm; xw[NW - 2] = dyp; xw[NW - 1] = dym;
+          xm = fma(nx, d.xx, xm);
+          xw[0] = d.xp; xw[1] = d.xm; xw[NW - 2] = d.yp; xw[NW - 1] = d.ym;
         } else {
-          xw[0] = dyp; xw[1] = dym;
+          xw[0] = d.yp; xw[1] = d.ym;
         }
         if (GSUB) {
           xm = w.um - xm;

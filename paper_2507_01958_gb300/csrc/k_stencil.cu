@@ -307,21 +307,21 @@ __global__ void __launch_bounds__(256, kCtPerSm) k_apply_Ct(Geom g, StripGrid sg
   double* xy2 = x + (ACTX ? 4 : 2) * n + base;
   const int j = j0 + (threadIdx.x & 31);
   const bool last = k + 1 >= g.nt;
-  const double nx = g.nu * g.idx, ny = g.nu * g.idy;  // nu K p from the scaled differences
+  const double nx = g.nu * g.ax, ny = g.nu * g.ay;
   const int jc = j < g.ny ? j : g.ny - 1;
-  diff_march<ACTX, true, 4>(
+  diff_march<ACTX, 4>(
       g, i0, i1, j0, [&](int i, int jj) { return pk[i * g.ny + jj]; },
       [&](int i) { return last ? 0.0 : pk[i * g.ny + jc + g.S]; },
-      [&](int i, double pc, double dyp, double dym, double dxp, double dxm, double pn) {
+      [&](int i, double pc, const Diff& d, double pn) {
         if (j >= g.ny) return;
         const int e = i * g.ny + j;
-        double m = fma(ny, dyp - dym, (pc - pn) * g.idt);
-        xy1[e] = dyp;
-        xy2[e] = dym;
+        double m = fma(ny, d.yy, (pc - pn) * g.idt);
+        xy1[e] = d.yp;
+        xy2[e] = d.ym;
         if (ACTX) {
-          m = fma(nx, dxp - dxm, m);
-          xx1[e] = dxp;
-          xx2[e] = dxm;
+          m = fma(nx, d.xx, m);
+          xx1[e] = d.xp;
+          xx2[e] = d.xm;
         }
         xm[e] = m;
       });

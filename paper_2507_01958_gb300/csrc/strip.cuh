@@ -136,18 +136,26 @@ __device__ __forceinline__ void sum_march(const Geom& g, double rho, int i0, int
   }
 }
 
-// The march for neighbour differences: f(row, centre p, dyp, dym, dxp, dxm, loaded) with
-// dyp = p - p_{j+1}, dym = p_{j-1} - p, dxp = p - p_{i+1}, dxm = p_{i-1} - p, each formed
-// once per face (0 across a Neumann end).  SCALE: the differences times 1/dy (y) and
-// 1/dx (x), scaled once per face.
-template <int ACTX, bool SCALE, int ROWS, typename Ld, typename Pre, typename F>
+// The march for neighbour differences: f(row, centre p, Diff, loaded).  Each face's
+// difference is formed once, and scaled once for the gradient components.  The second
+// differences come from the unscaled ones, which are exact where p varies slowly: scaled
+// first, they carry an error of the size of the gradient (512^2 Neumann, nu = 1: the m
+// row of C^T p 15 times as far off).  A lane gets its left face's two values from the
+// neighbour by shuffles, which cost less than a second FP64 multiplication.
+struct Diff {
+  double yp, ym, xp, xm;  // (p - p_{j+1})/dy, (p_{j-1} - p)/dy, the same in x; 0 across a Neumann end
+  double yy, xx;          // 2 p - p_{j-1} - p_{j+1}, the same in x
+};
+
+template <int ACTX, int ROWS, typename Ld, typename Pre, typename F>
 __device__ __forceinline__ void diff_march(const Geom& g, int i0, int i1, int j0, Ld ld, Pre pre, F f) {
   const int lane = threadIdx.x & 31;
   const StripCols c = strip_cols(g, j0);
   const int ir = min(i0 + lane, i1 - 1);
   const double right = ld(ir, c.right);
-  double hd = ld(ir, c.left), hc = ld(ir, j0), vc = ld(i0, c.j), dxm = 0.0;
+  double hd = ld(ir, c.left), hc = ld(ir, j0), hs = 0.0, vc = ld(i0, c.j), dxm = 0.0;
   if (ACTX) dxm = ld(ghost(i0 - 1, g.nx, g.perx), c.j);
+  Diff d{};
   for (int i = i0; i < i1; i += ROWS) {
     double v[ROWS];
     decltype(pre(0)) x[ROWS];
@@ -159,23 +167,29 @@ __device__ __forceinline__ void diff_march(const Geom& g, int i0, int i1, int j0
     }
     if (i == i0) {
       hd -= hc;
-      if (ACTX) dxm -= vc;
-      if (SCALE) {
-        hd *= g.idy;
-        dxm *= g.idx;
+      hs = hd * g.idy;
+      if (ACTX) {
+        dxm -= vc;
+        d.xm = dxm * g.idx;
       }
     }
 #pragma unroll
     for (int t = 0; t < ROWS; ++t) {
       if (i + t >= i1) break;
-      double dyp = vc - from_right(vc, right, i + t - i0);
-      if (SCALE) dyp *= g.idy;
-      const double dym = from_left(dyp, hd, i + t - i0);
-      double dxp = ACTX ? vc - v[t] : 0.0;
-      if (ACTX && SCALE) dxp *= g.idx;
-      f(i + t, vc, dyp, dym, dxp, dxm, x[t]);
+      const double dyp = vc - from_right(vc, right, i + t - i0);
+      d.yp = dyp * g.idy;
+      d.ym = from_left(d.yp, hs, i + t - i0);
+      d.yy = dyp - from_left(dyp, hd, i + t - i0);
+      double dxp = 0.0;
+      if (ACTX) {
+        dxp = vc - v[t];
+        d.xp = dxp * g.idx;
+        d.xx = dxp - dxm;
+      }
+      f(i + t, vc, d, x[t]);
       if (ACTX) {
         dxm = dxp;
+        d.xm = d.xp;
         vc = v[t];
       }
     }

@@ -84,3 +84,21 @@ def test_AAt_slow_in_time(ny, bc, length):
     xa = g.nu * g.Kabs(a) + np.abs(a - g.next(a)) * g.idt
     terms = g.nu * g.Kabs(xa) + (xa + g.prev(xa)) * g.idt + 2 * g.Kabs(a)
     assert (np.abs(host(q).reshape(f.shape) - ref) <= 16 * U * terms).all()
+
+
+@pytest.mark.parametrize("shape,bc", [((33, 64, 3), BCS[0]), ((64, 90, 3), BCS[2]), ((300, 40, 2), BCS[1])])
+def test_Ct_slow_in_space(shape, bc):
+    """The m row of C^T p: nu K p from exact differences of neighbours.  Roundings: a second
+    difference, its scale and sum per axis, the time part, and 3 in each coefficient."""
+    import torch
+    nx, ny, nt = shape
+    p = _problem(nx, ny, nt, bc, (0.7, 0.9), 1.0)
+    f = _field(nx, ny, nt, 3, 1e-3)
+    x = torch.empty(5 * f.size, dtype=torch.float64, device="cuda")
+    lib().mfg_apply_Ct(lib().mfg_plan(p), 0, dev(f), x)
+    g, a = _Nb(p), f.astype(LD)
+    dt = (a - g.next(a)) * g.idt
+    kx, ky = (g.ih[q] ** 2 * (g.bwd(a, q) - g.fwd(a, q)) for q in range(2))
+    ref = g.nu * (kx + ky) + dt
+    bound = 8 * U * (g.nu * (np.abs(kx) + np.abs(ky)) + np.abs(dt))
+    assert (np.abs(host(x)[:f.size].reshape(f.shape) - ref) <= bound).all()
