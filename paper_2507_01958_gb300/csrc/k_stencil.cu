@@ -68,10 +68,12 @@ __device__ __forceinline__ int wrap_or_neg(int i, int N, int per) {
 // mode 3: adjoint right-hand side r = C v; reduces ||r||^2, resets the PCG
 //         state with the fixed tolerance.
 //
-// Terms of a point, in face form (each face formed once, see strip.cuh):
-// F = w1_i + w2_{i+1} per face, div_h w = (F_{i+1/2} - F_{i-1/2}) / dx + the y faces, 0
-// past a Neumann end.  FP64 issue bounds the kernel: 13 instructions per point
-// (15 with oblong cells; 2 more with Az) instead of ~28 point by point.
+// Terms of a point: nu K m by neighbour sums (strip.cuh), and per axis
+// ((w1_i - w1_{i-1}) + (w2_{i+1} - w2_i)) / dx, 0 past a Neumann end.  Each flux by its own
+// difference, exact where it varies slowly: sums w1_i + w2_{i+1} per face, formed once,
+// take two FP64 instructions less but round at the size of the flux (128^2 torus, nu = 0,
+// both fluxes smooth: up to 1e-16 -> 5e-15 off 64 bits).  FP64 issue bounds the kernel: 15
+// instructions per point (17 with oblong cells; 2 more with Az), ~28 point by point.
 __device__ __forceinline__ void rhs_tail(double acc, double accb, bool have_b, double* partials, DevScalars* sc) {
   double part[2] = {acc, accb};
   block_sum<2>(part);
@@ -116,13 +118,16 @@ __global__ void __launch_bounds__(256, kCPerSm) k_apply_C(Geom g, StripGrid sg, 
     const double* wy2 = v + (ACTX ? 4 : 2) * n + base;
     const StripCols c = strip_cols(g, j0);
     const int lane = threadIdx.x & 31, j = j0 + lane;
-    const bool end_y = !g.pery && j == g.ny - 1;  // no face beyond
+    const bool end_y = !g.pery && j == g.ny - 1, first_y = !g.pery && j == 0;  // no face beyond
     auto at = [&](int i, int jj) { return i * g.ny + jj; };  // < S, an int
     const int ir = min(i0 + lane, i1 - 1);
     const double w2r = wy2[at(ir, c.right)];
-    const double hf = (!g.pery && j0 == 0) ? 0.0 : wy1[at(ir, c.left)] + wy2[at(ir, j0)];
-    double fxm = 0.0;
-    if (ACTX && (g.perx || i0 > 0)) fxm = wx1[at(ghost(i0 - 1, g.nx, g.perx), c.j)] + wx2[at(i0, c.j)];
+    const double w1l = (!g.pery && j0 == 0) ? 0.0 : wy1[at(ir, c.left)];
+    double x1m = 0.0, x2c = 0.0;  // w1_{i-1}, w2_i
+    if (ACTX && (g.perx || i0 > 0)) {
+      x1m = wx1[at(ghost(i0 - 1, g.nx, g.perx), c.j)];
+      x2c = wx2[at(i0, c.j)];
+    }
     const double ky = alpha * g.nu * g.ay, rho = ACTX ? g.ax / g.ay : 0.0, kc = 2.0 * (1.0 + rho) * ky;
     const double aix = alpha * g.idx, aiy = alpha * g.idy, aidt = alpha * g.idt;
     const double* mp = k >= 1 ? m - g.S : m0;  // m of the previous level (plane 0: m0, or 0)
@@ -145,14 +150,17 @@ __global__ void __launch_bounds__(256, kCPerSm) k_apply_C(Geom g, StripGrid sg, 
           return w;
         },
         [&](int i, double mc, double sum, const Row& w) {
-          double fy = w.wy1 + from_right(w.wy2, w2r, i - i0);
-          if (end_y) fy = 0.0;
-          const double sy = fy - from_left(fy, hf, i - i0);
+          const double y1 = end_y ? 0.0 : w.wy1, y2 = first_y ? 0.0 : w.wy2;
+          double y2r = from_right(y2, w2r, i - i0);
+          if (end_y) y2r = 0.0;
+          const double sy = (y1 - from_left(y1, w1l, i - i0)) + (y2r - y2);
           double val = fma(kc, mc, -ky * sum);
           if (ACTX) {
-            const double fx = (!g.perx && i == g.nx - 1) ? 0.0 : w.wx1 + w.wx2;
-            const double sx = fx - fxm;
-            fxm = fx;
+            const bool end_x = !g.perx && i == g.nx - 1;
+            const double x1 = end_x ? 0.0 : w.wx1, x2 = end_x ? 0.0 : w.wx2;
+            const double sx = (x1 - x1m) + (x2 - x2c);
+            x1m = x1;
+            x2c = x2;
             val = ISO ? fma(aiy, sx + sy, val) : fma(aix, sx, fma(aiy, sy, val));
           } else {
             val = fma(aiy, sy, val);

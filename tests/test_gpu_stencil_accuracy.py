@@ -102,3 +102,29 @@ def test_Ct_slow_in_space(shape, bc):
     ref = g.nu * (kx + ky) + dt
     bound = 8 * U * (g.nu * (np.abs(kx) + np.abs(ky)) + np.abs(dt))
     assert (np.abs(host(x)[:f.size].reshape(f.shape) - ref) <= bound).all()
+
+
+@pytest.mark.parametrize("shape,bc", [((33, 64, 3), BCS[0]), ((64, 90, 3), BCS[2]), ((70, 40, 2), BCS[1]), ((50, 9, 3), BCS[2])])
+@pytest.mark.parametrize("length", [(1.0, 1.0), (0.7, 0.9)])
+@pytest.mark.parametrize("nu", [0.0, 1e-3])
+def test_C_slow_fluxes(shape, bc, length, nu):
+    """div_h w from exact differences of each flux, both of an axis nonzero.  Roundings on
+    the longest path: 7 in the sums, 5 in the coefficients."""
+    import torch
+    nx, ny, nt = shape
+    p = _problem(nx, ny, nt, bc, length, nu)
+    v = np.stack([_field(nx, ny, nt, 4 + q, 1e-3) * (1.0 if q % 2 or q == 0 else -0.4) for q in range(5)])
+    r = torch.empty(v[0].size, dtype=torch.float64, device="cuda")
+    lib().mfg_apply_C(lib().mfg_plan(p), 0, dev(v), r)
+    g, a = _Nb(p), v.astype(LD)
+    dm = (a[0] - g.prev(a[0])) * g.idt
+    ref, terms = g.nu * g.K(a[0]) + dm, g.nu * g.Kabs(a[0]) + np.abs(dm)
+    for ax in range(2):
+        w1, w2 = a[1 + 2 * ax].copy(), a[2 + 2 * ax].copy()
+        if not g.per[ax]:  # slots past the ends
+            w1[(slice(None),) * (1 + ax) + (-1,)] = 0
+            w2[(slice(None),) * (1 + ax) + (0,)] = 0
+        d1, d2 = w1 - np.roll(w1, 1, 1 + ax), np.roll(w2, -1, 1 + ax) - w2
+        ref = ref + g.ih[ax] * (d1 + d2)
+        terms = terms + g.ih[ax] * (np.abs(d1) + np.abs(d2))
+    assert (np.abs(host(r).reshape(a[0].shape) - ref) <= 12 * U * terms).all()
