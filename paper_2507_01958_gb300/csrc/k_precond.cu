@@ -207,25 +207,32 @@ int build_prec_tables(const mfg_problem& p, const Geom& g, PrecTables* t, std::s
     free_prec_tables(t);
     return MFG_ERR_CUDA;
   }
-  if (p.precision == MFG_FP64 && p.l != 0 && p.nu_field == nullptr) {
-    if (cudaMalloc(&t->tri64, sizeof(double) * (size_t)g.n) != cudaSuccess) {
-      *err = "cudaMalloc failed for the time elimination's factors";
-      free_prec_tables(t);
-      return MFG_ERR_CUDA;
-    }
-    launch_k(k_tri_table, (g.S + 127) / 128, 128, 0, (cudaStream_t) nullptr, t->tri64, t->L1_64, t->L2_64, p.l, g.nt, g.S);
-    if (cudaStreamSynchronize(nullptr) != cudaSuccess) {
-      *err = "building the time elimination's factors failed";
-      free_prec_tables(t);
-      return MFG_ERR_CUDA;
-    }
-  }
   if (p.nu_field != nullptr) {
     const int rc = build_band_tables(p, g, lt.data(), t, err);
     if (rc != MFG_OK) {
       free_prec_tables(t);
       return rc;
     }
+  }
+  return MFG_OK;
+}
+
+// The factors are n doubles that the elimination can do without (it then forms them
+// per apply), so a plan takes them last, and only where `reserve` bytes stay free.
+int build_time_factors(const mfg_problem& p, const Geom& g, size_t reserve, PrecTables* t, std::string* err) {
+  if (p.precision != MFG_FP64 || p.l == 0 || t->band_w > 0) return MFG_OK;
+  const size_t vec = sizeof(double) * (size_t)g.n;
+  size_t avail = 0, total = 0;
+  if (cudaMemGetInfo(&avail, &total) != cudaSuccess || avail < vec + reserve ||
+      cudaMalloc(&t->tri64, vec) != cudaSuccess) {
+    t->tri64 = nullptr;
+    cudaGetLastError();
+    return MFG_OK;
+  }
+  launch_k(k_tri_table, (g.S + 127) / 128, 128, 0, (cudaStream_t) nullptr, t->tri64, t->L1_64, t->L2_64, p.l, g.nt, g.S);
+  if (cudaStreamSynchronize(nullptr) != cudaSuccess) {
+    *err = "building the time elimination's factors failed";
+    return MFG_ERR_CUDA;
   }
   return MFG_OK;
 }

@@ -659,6 +659,14 @@ int mfg_plan(const mfg_problem* probs, int batch, mfg_plan_t* out) {
   if (cudaStreamCreateWithFlags(&pl->cap0, cudaStreamNonBlocking) != cudaSuccess ||
       cudaStreamCreateWithFlags(&pl->cap1, cudaStreamNonBlocking) != cudaSuccess)
     return bail(MFG_ERR_CUDA, "cudaStreamCreate failed");
+  // left free for what the plan's use may allocate: the caller's y, ybar and z, the
+  // host call's staging of the same, the adjoint's workspace
+  const size_t reserve = 3 * sizeof(double) * (2 * pl->primal_total + pl->dual_total);
+  for (auto& in : pl->inst) {
+    std::string err;
+    const int rc = build_time_factors(in.p, in.g, reserve, &in.tabs, &err);
+    if (rc != MFG_OK) return bail(rc, err);
+  }
   *out = pl;
   return MFG_OK;
 }

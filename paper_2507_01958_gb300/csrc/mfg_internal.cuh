@@ -161,7 +161,7 @@ struct PrecTables {
   // the off-diagonal per mode (S); null otherwise.
   double *thc64 = nullptr, *thd64 = nullptr, *tho64 = nullptr;
   float *thc32 = nullptr, *thd32 = nullptr, *tho32 = nullptr;
-  double* tri64 = nullptr;  // FP64 plans, l = 1, 2: factors of the time elimination (n); else null
+  double* tri64 = nullptr;  // FP64 plans, l = 1, 2, where memory allows: factors of the time elimination (n)
   // Viscosity field: face coefficients (Geom::kfx, kfy) and the banded Cholesky
   // factors of the per-frequency systems (k_band.cu); null otherwise.
   double *kfx = nullptr, *kfy = nullptr;
@@ -180,6 +180,7 @@ void launch_time_tc(const float* in, float* out, const float* V, const float* la
                     const float* L2, int nt, int S, const DevScalars* sc, cudaStream_t s);
 int time_tc_configure();
 int build_prec_tables(const mfg_problem& p, const Geom& g, PrecTables* t, std::string* err);
+int build_time_factors(const mfg_problem& p, const Geom& g, size_t reserve, PrecTables* t, std::string* err);
 void free_prec_tables(PrecTables* t);
 // Operands of the PCG dot products that the last preconditioner pass can fuse
 // (r.zp and, for the flexible variant, q.zp, then beta).
