@@ -49,8 +49,23 @@ __device__ __forceinline__ void hinv_cell(double m, const double (&v)[NW], doubl
   for (int q = 0; q < NW; ++q) ow[q] = v[q] != 0.0 ? fma(m, uw[q], v[q] * om) : 0.0;
 }
 
+// v = w/m and 1/a' of a cell, 0 where m <= 0.
+template <int NW>
+__device__ __forceinline__ void cell_data(const Geom& g, const Coef& cf, double m, bool last, const double (&w)[NW],
+                                          double (&v)[NW], double& iap) {
+  const bool on = m > 0.0;
+  const double im = on ? 1.0 / m : 0.0;
+  iap = on ? 1.0 / (cf.f_a + 2.0 * cf.f_b * m + (last ? cf.g_a * g.idt : 0.0)) : 0.0;
+#pragma unroll
+  for (int q = 0; q < NW; ++q) {
+    v[q] = on ? w[q] * im : 0.0;
+    // w != 0 marks an active component: a quotient that underflows keeps the mark
+    if (on && w[q] != 0.0 && v[q] == 0.0) v[q] = __longlong_as_double(1);
+  }
+}
+
 // out = H^{-1} u, and the cell data of y that later applies read: vel (v, then
-// 1/a', NW + 1 planes).
+// 1/a', NW + 1 planes; null where the device had no room for them).
 template <int ACTX>
 __global__ void __launch_bounds__(kThreads) k_hinv(Geom g, Coef cf, const double* __restrict__ y,
                                                    const double* __restrict__ u, double* __restrict__ out,
@@ -62,20 +77,18 @@ __global__ void __launch_bounds__(kThreads) k_hinv(Geom g, Coef cf, const double
        e += (long long)gridDim.x * blockDim.x) {
     const int k = (int)(e / g.S);
     const double m = y[e];
-    double v[NW], uw[NW], ow[NW], om, iap = 0.0;
-    const bool on = m > 0.0;
-    const double im = on ? 1.0 / m : 0.0;
-    if (on) iap = 1.0 / (cf.f_a + 2.0 * cf.f_b * m + (k == g.nt - 1 ? cf.g_a * g.idt : 0.0));
+    double w[NW], v[NW], uw[NW], ow[NW], om, iap;
 #pragma unroll
     for (int q = 0; q < NW; ++q) {
       uw[q] = u[e + (q + 1) * n];
-      const double w = y[e + (q + 1) * n];
-      v[q] = on ? w * im : 0.0;
-      // w != 0 marks an active component: a quotient that underflows keeps the mark
-      if (on && w != 0.0 && v[q] == 0.0) v[q] = __longlong_as_double(1);
-      vel[e + q * n] = v[q];
+      w[q] = y[e + (q + 1) * n];
     }
-    vel[e + NW * n] = iap;
+    cell_data<NW>(g, cf, m, k == g.nt - 1, w, v, iap);
+    if (vel != nullptr) {
+#pragma unroll
+      for (int q = 0; q < NW; ++q) vel[e + q * n] = v[q];
+      vel[e + NW * n] = iap;
+    }
     hinv_cell<NW>(m, v, iap, u[e], uw, om, ow);
     out[e] = om;
 #pragma unroll
@@ -146,9 +159,10 @@ __global__ void __launch_bounds__(256, kCtHinvPerSm) k_ct_hinv(Geom g, StripGrid
 }
 
 // The same point by point, for viscosity fields (VN: L = K_nu + I/dt with the face
-// coefficients of Geom::kfx / kfy) and for rows too short for strips.
-template <int ACTX, bool VN>
-__global__ void __launch_bounds__(kThreads) k_ct_hinv_flat(Geom g, const double* __restrict__ mass,
+// coefficients of Geom::kfx / kfy) and for rows too short for strips.  DATA = false:
+// the cell data formed from y again in every apply, for a device without room for vel.
+template <int ACTX, bool VN, bool DATA>
+__global__ void __launch_bounds__(kThreads) k_ct_hinv_flat(Geom g, Coef cf, const double* __restrict__ y,
                                                            const double* __restrict__ vel,
                                                            const double* __restrict__ p,
                                                            const double* __restrict__ gsub,
@@ -199,10 +213,19 @@ __global__ void __launch_bounds__(kThreads) k_ct_hinv_flat(Geom g, const double*
 #pragma unroll
       for (int q = 0; q < NW; ++q) xw[q] = gsub[e + (q + 1) * n] - xw[q];
     }
-    double v[NW], ow[NW], om;
+    double v[NW], ow[NW], om, iap;
+    const double m = y[e];
+    if constexpr (DATA) {
 #pragma unroll
-    for (int q = 0; q < NW; ++q) v[q] = vel[e + q * n];
-    hinv_cell<NW>(mass[e], v, vel[e + NW * n], xm, xw, om, ow);
+      for (int q = 0; q < NW; ++q) v[q] = vel[e + q * n];
+      iap = vel[e + NW * n];
+    } else {
+      double w[NW];
+#pragma unroll
+      for (int q = 0; q < NW; ++q) w[q] = y[e + (q + 1) * n];
+      cell_data<NW>(g, cf, m, k == g.nt - 1, w, v, iap);
+    }
+    hinv_cell<NW>(m, v, iap, xm, xw, om, ow);
     out[e] = om;
 #pragma unroll
     for (int q = 0; q < NW; ++q) out[e + (q + 1) * n] = ow[q];
@@ -296,13 +319,16 @@ void launch_hinv(const Geom& g, const Coef& cf, const double* y, const double* u
     launch_k(k_hinv<0>, nb, kThreads, 0, s, g, cf, y, u, out, vel);
 }
 
-void launch_ct_hinv(const Geom& g, const double* y, const double* vel, const double* p, const double* gsub,
-                    double* out, cudaStream_t s, const DevScalars* sc) {
-  if (!strips_fit(g)) {
+void launch_ct_hinv(const Geom& g, const Coef& cf, const double* y, const double* vel, const double* p,
+                    const double* gsub, double* out, cudaStream_t s, const DevScalars* sc) {
+  if (vel == nullptr || !strips_fit(g)) {
     const int nb = red_blocks(g.n, kVecBlocksMax);
-#define MFG_CT_HINV(A, N) launch_k(k_ct_hinv_flat<A, N>, nb, kThreads, 0, s, g, y, vel, p, gsub, out, sc)
-    if (g.kfy != nullptr) { if (g.actx) MFG_CT_HINV(1, true); else MFG_CT_HINV(0, true); }
-    else                  { if (g.actx) MFG_CT_HINV(1, false); else MFG_CT_HINV(0, false); }
+#define MFG_CT_HINV(A, N, D) launch_k(k_ct_hinv_flat<A, N, D>, nb, kThreads, 0, s, g, cf, y, vel, p, gsub, out, sc)
+#define MFG_CT_HINV_D(D)                                                                                  \
+  if (g.kfy != nullptr) { if (g.actx) MFG_CT_HINV(1, true, D); else MFG_CT_HINV(0, true, D); }            \
+  else                  { if (g.actx) MFG_CT_HINV(1, false, D); else MFG_CT_HINV(0, false, D); }
+    if (vel != nullptr) { MFG_CT_HINV_D(true) } else { MFG_CT_HINV_D(false) }
+#undef MFG_CT_HINV_D
 #undef MFG_CT_HINV
     return;
   }

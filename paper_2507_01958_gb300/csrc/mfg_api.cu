@@ -829,9 +829,12 @@ int mfg_adjoint(mfg_plan_t pl, int b, const double* y, const double* z, const do
     if (!ev && cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess)
       return fail(MFG_ERR_CUDA, "cudaEventCreate failed for adjoint flags");
   if ((!in.adj_t && cudaMalloc(&in.adj_t, (size_t)g.c * n * 8) != cudaSuccess) ||
-      (!in.adj_eta && cudaMalloc(&in.adj_eta, n * 8) != cudaSuccess) ||
-      (!in.adj_vel && cudaMalloc(&in.adj_vel, (size_t)g.c * n * 8) != cudaSuccess))
+      (!in.adj_eta && cudaMalloc(&in.adj_eta, n * 8) != cudaSuccess))
     return fail(MFG_ERR_CUDA, "cudaMalloc failed for adjoint workspace");
+  if (!in.adj_vel && cudaMalloc(&in.adj_vel, (size_t)g.c * n * 8) != cudaSuccess) {
+    in.adj_vel = nullptr;  // no room for the cell data: every apply forms them again
+    cudaGetLastError();
+  }
   cudaStream_t s = (cudaStream_t)stream;
   DevScalars h{};
   h.status = MFG_OK;
@@ -859,7 +862,7 @@ int mfg_adjoint(mfg_plan_t pl, int b, const double* y, const double* z, const do
   for (int i = 0;; ++i) {
     const PcgDot dot{in.r, in.q, in.partials, in.sc, flex};
     const PcgZr zr{in.adj_eta, in.r, in.pv, in.q, in.partials, in.sc};
-    launch_ct_hinv(g, y, in.adj_vel, in.pv, nullptr, in.adj_t, s, in.sc);
+    launch_ct_hinv(g, in.cf, y, in.adj_vel, in.pv, nullptr, in.adj_t, s, in.sc);
     launch_apply_C(g, in.adj_t, in.q, 1.0, nullptr, in.partials, in.sc, 2, s, in.pv);
     launch_precond(g, in.tabs, in.p.precision, in.r, in.zp, in.work64, in.work32, in.sc, s, &dot, &zr);
     launch_update_p(g.n, in.zp, in.pv, in.sc, 0, 0, s, g.vec_blocks);
@@ -870,7 +873,7 @@ int mfg_adjoint(mfg_plan_t pl, int b, const double* y, const double* z, const do
   }
   DevScalars hs;
   // mu = H^{-1}(g - C^T eta), then the contractions
-  launch_ct_hinv(g, y, in.adj_vel, in.adj_eta, gy, in.adj_t, s, nullptr);
+  launch_ct_hinv(g, in.cf, y, in.adj_vel, in.adj_eta, gy, in.adj_t, s, nullptr);
   launch_adj_grads(g, y, z, in.adj_eta, in.adj_t, dm0, dV, dW, dnu, in.partials, in.sc, s);
   launches += 2;
   pl->launches += launches;

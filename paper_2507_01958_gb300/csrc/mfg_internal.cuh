@@ -238,11 +238,11 @@ void fft_x(int N, int periodic, int inverse, const T* in, T* out, const T* tw, c
            long long inner, long long outer, const DevScalars* sc, cudaStream_t s);
 
 // Adjoint (k_adjoint.cu).  vel: (c planes) velocities w/m of y and 1/f_eff'(m),
-// written by launch_hinv and read by launch_ct_hinv.
+// written by launch_hinv and read by launch_ct_hinv; null: formed from y in each.
 void launch_hinv(const Geom& g, const Coef& cf, const double* y, const double* u, double* out, double* vel,
                  cudaStream_t s);
-void launch_ct_hinv(const Geom& g, const double* y, const double* vel, const double* p, const double* gsub,
-                    double* out, cudaStream_t s, const DevScalars* sc);
+void launch_ct_hinv(const Geom& g, const Coef& cf, const double* y, const double* vel, const double* p,
+                    const double* gsub, double* out, cudaStream_t s, const DevScalars* sc);
 int adj_grads_blocks(const Geom& g);  // partial sums launch_adj_grads writes
 void launch_adj_grads(const Geom& g, const double* y, const double* z, const double* eta,
                       const double* mu, double* dm0, double* dV, double* dW, double* dnu,

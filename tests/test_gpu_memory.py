@@ -2,7 +2,8 @@
 device filled up, plans are built and calls answered as in the memory their
 mandatory workspace takes.  Both sides evaluate the same formulas, so the bars are
 those of the tests against the oracle (1e-12 for P^{-1} in FP64, 1e-7 for gradients)."""
-import numpy as np
+import contextlib
+
 import pytest
 
 import mfg_inputs as mi
@@ -19,9 +20,16 @@ def _free():
     return torch.cuda.mem_get_info()[0]
 
 
-def _fill(leave):
+@contextlib.contextmanager
+def _filled(leave):
+    """The device filled up but for `leave` bytes."""
     import torch
-    return torch.empty(max(0, _free() - int(leave)), dtype=torch.uint8, device="cuda")
+    fill = torch.empty(max(0, _free() - int(leave)), dtype=torch.uint8, device="cuda")
+    try:
+        yield
+    finally:
+        del fill
+        torch.cuda.empty_cache()
 
 
 def _rel(a, b):
@@ -43,10 +51,36 @@ def test_plan_without_room_for_the_time_factors(l):
         L.mfg_apply_precond(plan, 0, r, ref)
         torch.cuda.synchronize()
         L.mfg_destroy(plan)
-    fill = _fill(used - 4 * n)  # the factors are 8 n bytes
-    plan = L.mfg_plan(p, precision="fp64")
-    L.mfg_apply_precond(plan, 0, r, z)
-    torch.cuda.synchronize()
-    L.mfg_destroy(plan)
-    del fill
+    with _filled(used - 4 * n):  # the factors are 8 n bytes
+        plan = L.mfg_plan(p, precision="fp64")
+        L.mfg_apply_precond(plan, 0, r, z)
+        torch.cuda.synchronize()
+        L.mfg_destroy(plan)
     assert _rel(z, ref) <= 1e-12
+
+
+def test_adjoint_without_room_for_the_cell_data():
+    import torch
+    L = lib()
+    # nu keeps cond(AAt) u below 1e-8
+    p = mi.small(seed=2, dim=2, nx=256, ny=256, nt=128, bc=("neumann", "periodic"), nu=1e-2)["problem"]
+    n, c = 256 * 256 * 128, 5
+    gen = torch.Generator("cuda").manual_seed(2)
+    y = 0.5 + torch.rand((c, n), dtype=torch.float64, device="cuda", generator=gen)
+    y[2::2] *= -1.0
+    g = torch.randn((c, n), dtype=torch.float64, device="cuda", generator=gen)
+    z = torch.zeros(n, dtype=torch.float64, device="cuda")
+    outs = []
+    for short in (False, True):
+        plan = L.mfg_plan(p, precision="mixed")
+        out = [torch.empty(256 * 256, dtype=torch.float64, device="cuda") for _ in range(3)]
+        out.append(torch.empty(1, dtype=torch.float64, device="cuda"))
+        # room for the two mandatory vectors (c n and n doubles) and half of the cell data
+        with _filled((c + 1 + c / 2) * 8 * n) if short else contextlib.nullcontext():
+            rc, st = L.mfg_adjoint(plan, 0, y.reshape(-1), z, g.reshape(-1), *out, tol=1e-12)
+            torch.cuda.synchronize()
+        L.mfg_destroy(plan)
+        assert rc == 0 and st.status == 0
+        outs.append(out)
+    for a, b in zip(*outs):
+        assert _rel(a, b) <= 1e-7
