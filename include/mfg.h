@@ -282,7 +282,7 @@ typedef struct {
   int measured;       /* 1: this plan's mfg_autotune timed the candidates itself        */
   int time_pass;      /* MFG_TIME_TENSOR_CORES | MFG_TIME_CUDA_CORES                    */
   int fft[2];         /* per problem axis: 1 = FFT spatial pass, 0 = dense transform   */
-  int aat_blocks;     /* blocks of the AAt stencil launch                               */
+  int aat_blocks;     /* blocks of the AAt stencil launch (the larger of its two)       */
   int vec_blocks;     /* grid cap of the vector and reduction kernels                   */
   double precond_us;  /* measured time of the chosen preconditioner step, 0 if none     */
   double aat_us;      /* measured time of the chosen AAt apply, 0 if none               */

@@ -614,9 +614,18 @@ __global__ void __launch_bounds__(AJ * AI, 3) k_aat_q(Geom g, AatCoef a, int kc,
   aat_tail(acc, partials, sc);
 }
 
-// Blocks of the largest reducing launch over the grid, in strips (for any blocks
-// per SM) or in columns (viscosity fields, the double-float stencil).
-int aat_blocks(const Geom& g) {
+// Blocks of the AAt launch, the larger of its two passes.
+int aat_blocks(const Geom& g, int df64) {
+  if (g.kfy != nullptr || df64) {
+    const dim3 g2 = aat2_grid(g, aat2_chunk(g));
+    return (int)((long long)g2.x * g2.y * g2.z);
+  }
+  return std::max(strip_grid(g, kUPerSm).blocks, strip_grid(g, kQPerSm).blocks);
+}
+
+// At least the blocks of any reducing launch over the grid, in strips (for any
+// blocks per SM) or in columns (viscosity fields, the double-float stencil).
+int stencil_blocks_max(const Geom& g) {
   const dim3 g2 = aat2_grid(g, aat2_chunk(g));
   int most = (int)((long long)g2.x * g2.y * g2.z);
   for (int per_sm = 1; per_sm <= 6; ++per_sm) most = std::max(most, strip_grid(g, per_sm).blocks);

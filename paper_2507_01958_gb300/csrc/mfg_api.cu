@@ -559,7 +559,7 @@ int mfg_get_schedule(mfg_plan_t pl, int b, mfg_schedule* out) {
     out->fft[0] = fx;
     out->fft[1] = fy;
   }
-  out->aat_blocks = aat_blocks(g);
+  out->aat_blocks = aat_blocks(g, in.p.precision == MFG_MIXED_DF);
   out->vec_blocks = g.vec_blocks;
   out->precond_us = in.tune_precond_us;
   out->aat_us = in.tune_aat_us;
@@ -632,7 +632,7 @@ int mfg_plan(const mfg_problem* probs, int batch, mfg_plan_t* out) {
     for (int want : kAatWants) {
       Geom gw = in.g;
       gw.aat_want = want;
-      most = std::max<long long>(most, 2LL * aat_blocks(gw));
+      most = std::max<long long>(most, 2LL * stencil_blocks_max(gw));
     }
     const size_t npart = (size_t)most;
     if (cudaMalloc(&in.r, n * 8) != cudaSuccess || cudaMalloc(&in.pv, n * 8) != cudaSuccess ||

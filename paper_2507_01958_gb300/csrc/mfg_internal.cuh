@@ -131,7 +131,8 @@ void launch_apply_Ct(const Geom& g, const double* p, double* x, cudaStream_t s);
 void launch_AAt(const Geom& g, const double* p, double* q, double* scratch, double* partials,
                 DevScalars* sc, int mode, cudaStream_t s, int df64);
 int aat_kernel_count(int df64);
-int aat_blocks(const Geom& g);
+int aat_blocks(const Geom& g, int df64);
+int stencil_blocks_max(const Geom& g);
 bool strips_fit(const Geom& g);
 
 // Vector kernels (k_cg.cu).
