@@ -356,7 +356,7 @@ int solve_eager(mfg_plan_t pl, const double* m0, const double* V, const double* 
 // Launch choices per instance shape (grid, N_t, boundary conditions,
 // precision, time solve, viscosity field or not), measured once per process: a later plan with the
 // same shape takes the cached choice without timing again.
-using TuneKey = std::array<int, 9>;
+using TuneKey = std::array<int, 10>;
 struct TuneVal {
   int vec_blocks, aat_want, time_simt, fft_x, fft_y;
   double precond_us, aat_us;
@@ -366,7 +366,8 @@ std::map<TuneKey, TuneVal> g_tune_cache;
 
 TuneKey tune_key(const Inst& in) {
   return TuneKey{in.g.nx, in.g.ny, in.g.nt, in.g.perx, in.g.pery, in.p.precision, in.p.l == 0 ? 1 : 0,
-                 in.g.actx, in.g.kfy != nullptr ? 1 : 0};
+                 in.g.actx, in.g.kfy != nullptr ? 1 : 0,
+                 in.g.actx && in.g.ax == in.g.ay ? 1 : 0};  // square cells: stencil kernels of their own
 }
 
 // Fills a device buffer with a positive, finite pattern (bytes 0x3F), so that

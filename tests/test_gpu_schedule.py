@@ -48,3 +48,15 @@ def test_aat_blocks(nx, ny, nt):
     assert blocks(p, "mixed_df") == _columns(nx, ny, nt)
     if nx * ny <= 1600:
         assert blocks(dict(p, nu_field=np.full(n, 0.1)), "mixed") == _columns(nx, ny, nt)
+
+
+def test_square_and_oblong_cells_are_tuned_apart():
+    """They run different stencil kernels, so a choice timed for one is not taken for the other."""
+    L = lib()
+    p = mi.small(seed=1, dim=2, nx=44, ny=44, nt=6, bc=("periodic", "periodic"))["problem"]
+    measured = []
+    for length in ((1.0, 1.0), (1.0, 2.0), (2.0, 2.0), (1.0, 3.0)):
+        plan = L.mfg_plan(dict(p, len=length), precision="mixed")
+        L.mfg_autotune(plan)
+        measured.append(L.mfg_get_schedule(plan, 0)["measured"])
+    assert measured == [1, 1, 0, 0]
