@@ -21,11 +21,19 @@ namespace mfg {
 // 256-thread blocks per SM that the launch bounds of the strip kernels admit
 constexpr int kCPerSm = 2, kCtPerSm = 3, kUPerSm = 4, kQPerSm = 3;
 
-// Whether C and C^T run in strips: not for viscosity fields, and not where the
-// strips would be less than ~60 % full (the point-by-point kernels issue 28 and 23 FP64
-// instructions per point, the strips 15 and 12 per lane; 200 x 33 x 31: 44 us for C, C^T
-// and AAt point by point, 51 us in strips; 33 x 200 x 31: 40 against 37).
-bool strips_fit(const Geom& g) { return g.kfy == nullptr && (g.ny + 31) / 32 * 32 * 3 <= 5 * g.ny; }
+// Share of the strips' lanes that have a column, at least num/den.
+static bool strips_filled(const Geom& g, int num, int den) {
+  return (long long)(g.ny + 31) / 32 * 32 * num <= (long long)g.ny * den;
+}
+// Which operators run in strips and which point by point (viscosity fields: all point
+// by point).  C^T and H^-1 C^T from 2/3 of the lanes filled on: 512 x ny x 100, C^T in
+// strips against point by point 39.3 / 36.2 us at ny = 20, 39.3 / 40.0 at 22, 74.7 / 77.3
+// at 43, 75.7 / 92.2 at 52; 2000 x 250 in 1-D 11.1 / 12.5.
+bool strips_fit(const Geom& g) { return g.kfy == nullptr && strips_filled(g, 2, 3); }
+// C in 2-D from 7/8 on: 512 x ny x 100, 51.4 / 39.6 us at ny = 20, 51.6 / 46.8 at 24, 102.0 / 88.8
+// at 45, 102.5 / 101.3 at 52, 103.1 / 108.8 at 56; 512^2 x 64 489 / 602.  Not in 1-D, where a
+// strip is one row and its borders a load each: 2000 x 250 17.9 / 15.3.
+static bool c_strips_fit(const Geom& g) { return g.actx && g.kfy == nullptr && strips_filled(g, 7, 8); }
 
 struct Nb {
   int im, ip;
@@ -99,7 +107,7 @@ __device__ __forceinline__ void rhs_tail(double acc, double accb, bool have_b, d
   }
 }
 
-template <int ACTX, bool ISO, int MODE>
+template <bool ISO, int MODE>
 __global__ void __launch_bounds__(256, kCPerSm) k_apply_C(Geom g, StripGrid sg, const double* __restrict__ v,
                                                     double* __restrict__ r, double alpha,
                                                     const double* __restrict__ m0, const double* __restrict__ pdot,
@@ -114,8 +122,8 @@ __global__ void __launch_bounds__(256, kCPerSm) k_apply_C(Geom g, StripGrid sg, 
     const double* m = v + base;
     const double* wx1 = v + n + base;
     const double* wx2 = v + 2 * n + base;
-    const double* wy1 = v + (ACTX ? 3 : 1) * n + base;
-    const double* wy2 = v + (ACTX ? 4 : 2) * n + base;
+    const double* wy1 = v + 3 * n + base;
+    const double* wy2 = v + 4 * n + base;
     const StripCols c = strip_cols(g, j0);
     const int lane = threadIdx.x & 31, j = j0 + lane;
     const bool end_y = !g.pery && j == g.ny - 1, first_y = !g.pery && j == 0;  // no face beyond
@@ -124,11 +132,11 @@ __global__ void __launch_bounds__(256, kCPerSm) k_apply_C(Geom g, StripGrid sg, 
     const double w2r = wy2[at(ir, c.right)];
     const double w1l = (!g.pery && j0 == 0) ? 0.0 : wy1[at(ir, c.left)];
     double x1m = 0.0, x2c = 0.0;  // w1_{i-1}, w2_i
-    if (ACTX && (g.perx || i0 > 0)) {
+    if (g.perx || i0 > 0) {
       x1m = wx1[at(ghost(i0 - 1, g.nx, g.perx), c.j)];
       x2c = wx2[at(i0, c.j)];
     }
-    const double ky = alpha * g.nu * g.ay, rho = ACTX ? g.ax / g.ay : 0.0, kc = 2.0 * (1.0 + rho) * ky;
+    const double ky = alpha * g.nu * g.ay, rho = g.ax / g.ay, kc = 2.0 * (1.0 + rho) * ky;
     const double aix = alpha * g.idx, aiy = alpha * g.idy, aidt = alpha * g.idt;
     const double* mp = k >= 1 ? m - g.S : m0;  // m of the previous level (plane 0: m0, or 0)
     struct Row {
@@ -140,10 +148,8 @@ __global__ void __launch_bounds__(256, kCPerSm) k_apply_C(Geom g, StripGrid sg, 
         [&](int i) {
           const int e = at(i, c.j);
           Row w{wy1[e], wy2[e], 0.0, 0.0, 0.0, 0.0};
-          if (ACTX) {
-            w.wx1 = wx1[e];
-            w.wx2 = wx2[at(ghost(i + 1, g.nx, g.perx), c.j)];
-          }
+          w.wx1 = wx1[e];
+          w.wx2 = wx2[at(ghost(i + 1, g.nx, g.perx), c.j)];
           if (have_mp) w.mp = mp[e];
           if (MODE == 2) w.extra = pdot[base + e];
           if (have_az) w.extra = Az[base + e];
@@ -155,16 +161,12 @@ __global__ void __launch_bounds__(256, kCPerSm) k_apply_C(Geom g, StripGrid sg, 
           if (end_y) y2r = 0.0;
           const double sy = (y1 - from_left(y1, w1l, i - i0)) + (y2r - y2);
           double val = fma(kc, mc, -ky * sum);
-          if (ACTX) {
-            const bool end_x = !g.perx && i == g.nx - 1;
-            const double x1 = end_x ? 0.0 : w.wx1, x2 = end_x ? 0.0 : w.wx2;
-            const double sx = (x1 - x1m) + (x2 - x2c);
-            x1m = x1;
-            x2c = x2;
-            val = ISO ? fma(aiy, sx + sy, val) : fma(aix, sx, fma(aiy, sy, val));
-          } else {
-            val = fma(aiy, sy, val);
-          }
+          const bool end_x = !g.perx && i == g.nx - 1;
+          const double x1 = end_x ? 0.0 : w.wx1, x2 = end_x ? 0.0 : w.wx2;
+          const double sx = (x1 - x1m) + (x2 - x2c);
+          x1m = x1;
+          x2c = x2;
+          val = ISO ? fma(aiy, sx + sy, val) : fma(aix, sx, fma(aiy, sy, val));
           if (j >= g.ny) return;
           val = fma(aidt, mc - w.mp, val);
           const int e = at(i, j);
@@ -184,13 +186,15 @@ __global__ void __launch_bounds__(256, kCPerSm) k_apply_C(Geom g, StripGrid sg, 
   if constexpr (MODE == 1 || MODE == 3) rhs_tail(acc, accb, Az != nullptr, partials, sc);
 }
 
-// The same terms point by point, for viscosity fields and for grids whose rows
-// would leave most of a 32-column strip empty (strips_fit).  VN (viscosity field):
+// The same terms point by point, for 1-D grids, viscosity fields and grids whose rows
+// would leave too much of a 32-column strip empty (c_strips_fit).  Two blocks per SM in
+// the launch bounds: with the compiler's own choice of 64 registers a grid of two
+// blocks per SM took 99.4 us for 512 x 45 x 100, with 100 registers 88.8.  VN (viscosity field):
 // nu K m becomes K_nu m = sum over the node's faces of kf (m - m_nb), kf the face
 // coefficient of Geom::kfx / kfy; at a Neumann end the neighbour index is the node
 // itself, so the missing face adds nothing.
 template <int ACTX, bool VN>
-__global__ void __launch_bounds__(kThreads) k_apply_C_flat(Geom g, const double* __restrict__ v,
+__global__ void __launch_bounds__(kThreads, 2) k_apply_C_flat(Geom g, const double* __restrict__ v,
                                                       double* __restrict__ r, double alpha,
                                                       const double* __restrict__ m0,
                                                       const double* __restrict__ pdot,
@@ -267,7 +271,7 @@ __global__ void __launch_bounds__(kThreads) k_apply_C_flat(Geom g, const double*
 void launch_apply_C(const Geom& g, const double* v, double* r, double alpha, const double* m0,
                     double* partials, DevScalars* sc, int mode, cudaStream_t s, const double* pdot,
                     double* Az) {
-  if (!strips_fit(g)) {
+  if (!c_strips_fit(g)) {
     const int nb = red_blocks(g.n, g.vec_blocks);
 #define MFG_C_FLAT(A, N) launch_k(k_apply_C_flat<A, N>, nb, kThreads, 0, s, g, v, r, alpha, m0, pdot, partials, sc, mode, Az)
     if (g.kfy != nullptr) { if (g.actx) MFG_C_FLAT(1, true); else MFG_C_FLAT(0, true); }
@@ -276,21 +280,19 @@ void launch_apply_C(const Geom& g, const double* v, double* r, double alpha, con
     return;
   }
   const StripGrid sg = strip_grid(g, kCPerSm);
-#define MFG_C(A, I, M) \
-  launch_k(k_apply_C<A, I, M>, sg.blocks, 32 * sg.warps, 0, s, g, sg, v, r, alpha, m0, pdot, partials, sc, Az)
-#define MFG_C_MODE(A, I)       \
+#define MFG_C(I, M) \
+  launch_k(k_apply_C<I, M>, sg.blocks, 32 * sg.warps, 0, s, g, sg, v, r, alpha, m0, pdot, partials, sc, Az)
+#define MFG_C_MODE(I)       \
   switch (mode) {              \
-    case 0: MFG_C(A, I, 0); break; \
-    case 1: MFG_C(A, I, 1); break; \
-    case 2: MFG_C(A, I, 2); break; \
-    default: MFG_C(A, I, 3); break; \
+    case 0: MFG_C(I, 0); break; \
+    case 1: MFG_C(I, 1); break; \
+    case 2: MFG_C(I, 2); break; \
+    default: MFG_C(I, 3); break; \
   }
-  if (!g.actx)
-    MFG_C_MODE(0, false)
-  else if (g.ax == g.ay)
-    MFG_C_MODE(1, true)
+  if (g.ax == g.ay)
+    MFG_C_MODE(true)
   else
-    MFG_C_MODE(1, false)
+    MFG_C_MODE(false)
 #undef MFG_C_MODE
 #undef MFG_C
 }

@@ -86,7 +86,8 @@ def test_AAt_slow_in_time(ny, bc, length):
     assert (np.abs(host(q).reshape(f.shape) - ref) <= 16 * U * terms).all()
 
 
-@pytest.mark.parametrize("shape,bc", [((33, 64, 3), BCS[0]), ((64, 90, 3), BCS[2]), ((300, 40, 2), BCS[1])])
+@pytest.mark.parametrize("shape,bc", [((33, 64, 3), BCS[0]), ((64, 90, 3), BCS[2]), ((300, 40, 2), BCS[1]),
+                                      ((60, 22, 2), BCS[2]), ((60, 21, 2), BCS[0]), ((9, 65, 2), BCS[1])])  # in strips from 22 of 32 lanes on
 def test_Ct_slow_in_space(shape, bc):
     """The m row of C^T p: nu K p from exact differences of neighbours.  Roundings: a second
     difference, its scale and sum per axis, the time part, and 3 in each coefficient."""
@@ -104,7 +105,8 @@ def test_Ct_slow_in_space(shape, bc):
     assert (np.abs(host(x)[:f.size].reshape(f.shape) - ref) <= bound).all()
 
 
-@pytest.mark.parametrize("shape,bc", [((33, 64, 3), BCS[0]), ((64, 90, 3), BCS[2]), ((70, 40, 2), BCS[1]), ((50, 9, 3), BCS[2])])
+@pytest.mark.parametrize("shape,bc", [((33, 64, 3), BCS[0]), ((64, 90, 3), BCS[2]), ((70, 40, 2), BCS[1]), ((50, 9, 3), BCS[2]),
+                                       ((60, 28, 2), BCS[0]), ((60, 27, 2), BCS[1])])  # in strips from 28 of 32 lanes on
 @pytest.mark.parametrize("length", [(1.0, 1.0), (0.7, 0.9)])
 @pytest.mark.parametrize("nu", [0.0, 1e-3])
 def test_C_slow_fluxes(shape, bc, length, nu):
