@@ -622,7 +622,7 @@ int aat_blocks(const Geom& g, int df64) {
     const dim3 g2 = aat2_grid(g, aat2_chunk(g));
     return (int)((long long)g2.x * g2.y * g2.z);
   }
-  return std::max(strip_grid(g, kUPerSm).blocks, strip_grid(g, kQPerSm).blocks);
+  return std::max(strip_grid(g, kUPerSm, g.aat_want).blocks, strip_grid(g, kQPerSm, g.aat_want).blocks);
 }
 
 // At least the blocks of any reducing launch over the grid, in strips (for any
@@ -630,7 +630,7 @@ int aat_blocks(const Geom& g, int df64) {
 int stencil_blocks_max(const Geom& g) {
   const dim3 g2 = aat2_grid(g, aat2_chunk(g));
   int most = (int)((long long)g2.x * g2.y * g2.z);
-  for (int per_sm = 1; per_sm <= 6; ++per_sm) most = std::max(most, strip_grid(g, per_sm).blocks);
+  for (int per_sm = 1; per_sm <= 6; ++per_sm) most = std::max({most, strip_grid(g, per_sm).blocks, strip_grid(g, per_sm, g.aat_want).blocks});
   return most;
 }
 
@@ -735,7 +735,7 @@ void launch_AAt(const Geom& g, const double* p, double* q, double* scratch, doub
     }
     return;
   }
-  const StripGrid ug = strip_grid(g, kUPerSm), ag = strip_grid(g, kQPerSm);
+  const StripGrid ug = strip_grid(g, kUPerSm, g.aat_want), ag = strip_grid(g, kQPerSm, g.aat_want);
   const int nth = 32 * ag.warps;
   const bool iso = g.actx && g.ax == g.ay, step = mode != 0;
 #define MFG_AAT(I, ST) launch_k(k_aat_q2<I, ST>, ag.blocks, nth, 0, s, g, a, ag, KP, X, p, q, partials, sc)

@@ -37,8 +37,8 @@ struct Geom {
   // measured ones.  They change launch shapes and pass variants, never the
   // operator a kernel applies.
   int vec_blocks;   // grid cap of the vector and reduction kernels
-  int aat_want;     // twice the blocks of a wave the strip kernels' row chunks are chosen for; target
-                    // block count of the column kernels (viscosity field, double-float)
+  int aat_want;     // AAt: 8 times the SMs its row chunks are chosen for (strips); target block
+                    // count of the column kernels (viscosity field, double-float)
   int time_simt;    // 1: time pass by elimination on the CUDA cores even where the tensor-core pass applies
   int fft_x, fft_y; // 1: FFT spatial pass where the axis length allows it; 0: dense pass
   // Viscosity field (mfg_problem::nu_field): per node, the coefficient of its

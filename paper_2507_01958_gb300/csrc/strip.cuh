@@ -25,19 +25,21 @@ __device__ __forceinline__ int ghost(int i, int N, int per) {
 // Launch: 32-column strips x row chunks x planes, one warp each.  A block holds 8
 // warps, fewer where that leaves fewer than 4 blocks per SM.  The chunk length (2 to 32 rows) is
 // the one with the least waves x (rows + 1.5): whole waves of the per_sm blocks a kernel's
-// registers admit per SM (scaled by aat_want over its default), 1.5 rows' worth of work for a chunk's start.  (256^2 x 128: 29
+// registers admit per SM, 1.5 rows' worth of work for a chunk's start.  (256^2 x 128: 29
 // rows, 1.9 waves, where 26 rows filled 2.1 and left the third wave nearly empty.)
+// want scales the wave over kAatWantDefault: AAt passes its tuned Geom::aat_want, which says
+// nothing about the other operators (C in strips, 512 x 45 x 100: 102 us by the default, 125 by half of it).
 struct StripGrid {
   int strips, chunks, rows, warps, blocks;
 };
 
-inline StripGrid strip_grid(const Geom& g, int per_sm) {
+inline StripGrid strip_grid(const Geom& g, int per_sm, int want = kAatWantDefault) {
   StripGrid a;
   a.strips = (g.ny + 31) / 32;
-  const long long base = (long long)a.strips * g.nt, wave = std::max(1, g.aat_want / 8 * per_sm);
+  const long long base = (long long)a.strips * g.nt, wave = std::max(1, want / 8 * per_sm);
   double best = 1e300;
-  for (int want = 32; want >= 2; --want) {
-    const int chunks = (g.nx + want - 1) / want, rows = (g.nx + chunks - 1) / chunks;
+  for (int most = 32; most >= 2; --most) {
+    const int chunks = (g.nx + most - 1) / most, rows = (g.nx + chunks - 1) / chunks;
     const long long blocks = (base * chunks + 7) / 8;
     const double cost = (double)((blocks + wave - 1) / wave) * (rows + 1.5);
     if (cost < best) {
