@@ -374,16 +374,7 @@ __device__ __forceinline__ float recip(float x) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-// 1/x for x >= 1: the hardware's approximation (relative error below 2^-20)
-// and one third-order (Halley) step, y (1 + e + e^2) with e = 1 - x y.  Past
-// 2^1000 the pivot's reciprocal is taken as 0 (nothing is coupled there).
-__device__ __forceinline__ double recip(double x) {
-  if (!(x < 1.0715086071862673e301)) return x != x ? x : 0.0;
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x, y, 1.0);
-  return fma(y, fma(e, e, e), y);
-}
+__device__ __forceinline__ double recip(double x) { return 1.0 / x; }
 
 // The g_k of every mode, [nt][S]: FP64 plans keep them (8 bytes per element read
 // instead of 6 of the 9 FP64 instructions; in FP32 they cost less than their bytes).
