@@ -319,9 +319,10 @@ __global__ void __launch_bounds__(256, kCtPerSm) k_apply_Ct(Geom g, StripGrid sg
   const bool last = k + 1 >= g.nt;
   const double nx = g.nu * g.ax, ny = g.nu * g.ay;
   const int jc = j < g.ny ? j : g.ny - 1;
+  const double* pn1 = pk + (last ? 0 : g.S);  // not i * ny + jc + S, which passes 2^31 from S = 2^30 on
   diff_march<ACTX, 4>(
       g, i0, i1, j0, [&](int i, int jj) { return pk[i * g.ny + jj]; },
-      [&](int i) { return last ? 0.0 : pk[i * g.ny + jc + g.S]; },
+      [&](int i) { return last ? 0.0 : pn1[i * g.ny + jc]; },
       [&](int i, double pc, const Diff& d, double pn) {
         if (j >= g.ny) return;
         const int e = i * g.ny + j;
