@@ -55,11 +55,10 @@ WORKLOAD = ("2-D Neumann unit square 512x512, N_t=128 (n=33,554,432), nu=1e-2, "
 # Precision of the timed solve and of the extras: FP32 preconditioner, its time
 # pass on the tensor cores (tcgen05, split TF32) or by elimination, FP64 elsewhere.
 PRECISION = "mixed_tc"
-# Algorithmic FP64 flops of one AAt apply per unknown in the factored form
-# q = C (C^T p): K p (4 differences, 2 adds, 2 scalings, 1 add = 9),
-# xm = nu Kp + (p - p')/dt (4), q = nu K xm + (xm - xm')/dt + 2 Kp (10 + 2 + 2)
-# -> 27.  (The kernels issue 12 FP64 instructions per unknown, mostly FMAs.)
-AAT_FLOPS_PER_UNKNOWN = 27
+# FP64 work of one AAt apply per unknown: 11 instructions on square cells (u: 2 adds,
+# 1 FMA; X: 1 add, 1 FMA; q: 2 adds, 1 product, 3 FMAs), each of which takes the issue
+# slot of an FMA, 2 flops of the rate below: 22.
+AAT_FLOPS_PER_UNKNOWN = 22
 # Algorithmic bytes of one AAt apply: read p, write q (2 FP64 words per unknown).
 AAT_BYTES_PER_UNKNOWN = 16
 # GB300 FP64 rate (1.25 TFLOP/s, the profiling recipe's table; not in the
@@ -335,7 +334,7 @@ def kernels_measure(L, dev, stream, peak_gbs):
         L.mfg_prox_step(plan, 0, 0.5, zd, y, ybar, V, W, stream=stream)
     # the in-solve primal step: reads z, y; writes y, ybar (y is overwritten in
     # place each repetition, which keeps the values in the same range)
-    out["prox step (k_prox_strip, in-solve)"] = entry(timed(prox_step), 128 * n, 128 * n, "FP64 issue")
+    out["prox step (k_prox_cp, in-solve)"] = entry(timed(prox_step), 128 * n, 128 * n, "FP64 issue")
     # P^-1 in 3 passes' worth of algorithmic bytes (FP64 in, FP64 out, FP32 in between:
     # 8 + 4 + 4 + 4 + 4 + 8); the five passes move 48 B per unknown
     out["P^-1 apply, FP32, eliminated time pass"] = entry(

@@ -88,7 +88,7 @@ typedef struct {
   double T;          /* horizon T > 0, dt = T/N_t                                      */
   double nu;         /* viscosity nu >= 0 (ignored when nu_field is set)               */
   double qprime;     /* Hamiltonian exponent q' of eq. power_hamiltonian, in [1.05, 20];
-                        2 takes the fast prox, others a general FP64 root finder    */
+                        2 takes the fast prox, others a root finder with FP64 residuals */
   double f_a, f_b;   /* f(x,m) = f_a m + f_b m^2 + V(x); f_a, f_b >= 0 (monotone f)   */
   double g_a;        /* g(x,m) = g_a m + W(x); g_a >= 0                                */
   int l;             /* time preconditioner: 1 = DCT-VIII, 2 = DST-I (Sec. 4.1);
@@ -158,7 +158,9 @@ typedef struct mfg_plan_s* mfg_plan_t;
  * [1.05, 20] (MFG_ERR_UNSUPPORTED), N_t < 2, N < 2, T <= 0, nu < 0,
  * f_a/f_b/g_a < 0, l not in {0,1,2}, N_t > 256 (UNSUPPORTED), a viscosity
  * field with a negative or non-finite value (INVALID_ARG) or outside the
- * limits of "Viscosity fields" (UNSUPPORTED).  *out is NULL on failure. */
+ * limits of "Viscosity fields" (UNSUPPORTED).  *out is NULL on failure.
+ * FP64 plans with l = 1, 2 also hold n doubles of the time elimination's factors,
+ * where the device has room for them beside what the calls below may allocate. */
 int mfg_plan(const mfg_problem* probs, int batch, mfg_plan_t* out);
 
 /* Frees all plan-owned memory.  NULL is accepted. */
@@ -253,7 +255,8 @@ int mfg_apply_Ct(mfg_plan_t plan, int b, const double* p, double* x, void* strea
  * The adjoint system is solved through its Schur complement
  * C_A H^{-1} C_A^T with the plan's preconditioner P (eq. prec) inside PCG,
  * H being the per-cell Hessian of phi.  The first call allocates a 2*c*n + n
- * workspace owned by the plan.  Synchronises `stream`. */
+ * workspace owned by the plan (c*n + n where there is no room for the rest: cell data
+ * that are then formed again in every iteration).  Synchronises `stream`. */
 int mfg_adjoint(mfg_plan_t plan, int b, const double* y, const double* z, const double* gy,
                 double* dm0, double* dV, double* dW, double* dnu, double tol, int max_iter,
                 mfg_stats* st, void* stream);
@@ -293,10 +296,11 @@ typedef struct {
  *   - grid cap of the vector and reduction kernels: 152, 304 or 608 blocks;
  *   - the preconditioner step (Alg. 1/2 with the fused PCG vector work): time
  *     pass on the tensor cores or by elimination (MFG_MIXED_TC with N_t in
- *     {32, 64, 128}), FFT or dense transform pass on each power-of-two axis;
- *   - AAt stencil launch: 152 x 4, 8 or 16 (row chunks of the strips).
+ *     {32, 64, 128}), FFT or dense transform pass on each axis with an FFT (no prime factor
+ *     above 13, up to 2048 points);
+ *   - AAt stencil launch: 152 x 4, 8 or 16 (row chunks of its strips).
  * The choice is cached per process by instance shape (grid, N_t, boundary
- * conditions, precision, l): a later plan with the same shape takes it
+ * conditions, precision, l, square or oblong cells): a later plan with the same shape takes it
  * without timing.  Uses the plan's workspace and a temporary n-double buffer
  * (allocated and freed here), overwrites the plan's device scalars, drops
  * the cached solve graph, and synchronises `stream`.  Call it before a

@@ -22,8 +22,8 @@
 //
 // y is fixed over the whole adjoint solve, so the velocities v = w/m and 1/a' are
 // formed once (k_hinv, which also applies H^{-1} to the right-hand side) and each
-// PCG iteration has no division left: 23 FP64 instructions per point instead of
-// 54, FP64 issue being what bounds it (128^2 x 64, cold: 114 -> 70 us; the whole
+// PCG iteration has no division left: 23 FP64 instructions and 5 comparisons per point
+// instead of 54 in all, FP64 issue being what bounds it (128^2 x 64, cold: 114 -> 70 us; the whole
 // adjoint 7.9 -> 5.6 ms).
 #include "mfg_internal.cuh"
 #include "reduce.cuh"
@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(kThreads) k_hinv(Geom g, Coef cf, const double
 constexpr int kCtHinvPerSm = 2;  // 256-thread blocks per SM
 
 // out = H^{-1} (C^T p)  or, with GSUB, out = H^{-1} (gsub - C^T p), in warp strips
-// (strip.cuh): 13 reads and writes of 8 bytes and 23 FP64 instructions per point.
+// (strip.cuh): 13 reads and writes of 8 bytes, 23 FP64 instructions and 5 comparisons per point.
 template <int ACTX, bool GSUB>
 __global__ void __launch_bounds__(256, kCtHinvPerSm) k_ct_hinv(Geom g, StripGrid sg, const double* __restrict__ m,
                                                               const double* __restrict__ vel,

@@ -55,13 +55,6 @@ __device__ __forceinline__ Nb nbr(int i, int N, int per) {
   return b;
 }
 
-__device__ __forceinline__ int wrap_or_neg(int i, int N, int per) {
-  if (i >= 0 && i < N) return i;
-  if (!per) return -1;
-  i %= N;
-  return i < 0 ? i + N : i;
-}
-
 // ------------------------------------------------------------------- C v --
 // mode 0: r = alpha * (C v - d), d = m0/dt on plane 0 when m0 != nullptr.
 // mode 1: CP right-hand side r = sigma (C v - d) with sigma from the device

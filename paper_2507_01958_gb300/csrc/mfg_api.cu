@@ -414,7 +414,7 @@ double time_us(F&& f, cudaStream_t s, cudaEvent_t a, cudaEvent_t b) {
 //   vector and reduction grid cap    152, 304, 608 blocks
 //   preconditioner passes            time pass on the tensor cores or the CUDA
 //                                    cores (MFG_MIXED_TC); FFT or dense pass per
-//                                    power-of-two axis; timed as the PCG step
+//                                    axis with an FFT; timed as the PCG step
 //                                    (fused z, r update and dot products)
 //   AAt stencil launch (aat_want)    152 x 4, 8, 16
 int tune_instance(Inst& in, double* zbuf, cudaStream_t s, cudaEvent_t a, cudaEvent_t b) {

@@ -11,8 +11,8 @@
 namespace mfg {
 
 constexpr int kThreads = 256;        // threads per block for 1-D launches
-// Fixed grid of the grid-stride reduction kernels.  Kept small: every thread
-// pays a warp-shuffle tree of FP64 adds at the end, and FP64 issue is scarce.
+// Fixed grid of the grid-stride reduction kernels.  Kept small: every block pays
+// FP64 adds for its sum at the end (block_sum), and FP64 issue is scarce.
 constexpr int kRedBlocks = 152 * 2;
 constexpr int kVecBlocksMax = 152 * 4;   // largest vec_blocks the autotuner tries
 constexpr int kAatWantDefault = 152 * 8;

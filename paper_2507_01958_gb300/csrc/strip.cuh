@@ -3,7 +3,7 @@
 // A warp owns 32 neighbouring j and marches along i in one time plane.  Values
 // at j +- 1 come from the neighbouring lanes and values at i +- 1 from registers,
 // so each value is loaded once per warp and whatever two neighbours have in
-// common (a pair sum, a face difference, a face flux) is formed once: FP64
+// common (a pair sum, a face difference) is formed once: FP64
 // instructions are what these kernels have to save.  What lanes 0 and 31 need
 // from beyond the strip is gathered once per chunk of at most 32 rows, with lane r
 // holding row r, and handed out row by row.
