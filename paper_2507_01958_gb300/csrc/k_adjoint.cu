@@ -321,7 +321,10 @@ void launch_hinv(const Geom& g, const Coef& cf, const double* y, const double* u
 
 void launch_ct_hinv(const Geom& g, const Coef& cf, const double* y, const double* vel, const double* p,
                     const double* gsub, double* out, cudaStream_t s, const DevScalars* sc) {
-  if (vel == nullptr || !strips_fit(g)) {
+  // an iteration of the adjoint with H^-1 C^T in strips against point by point: 300 x 45 x 60
+  // 203 / 194 us, 300 x 50 x 60 214 / 206, 512 x 26 x 60 189 / 189, 300 x 56 x 60 216 / 219,
+  // 300 x 64 x 60 204 / 217
+  if (vel == nullptr || !strips_filled(g, 7, 8)) {
     const int nb = red_blocks(g.n, kVecBlocksMax);
 #define MFG_CT_HINV(A, N, D) launch_k(k_ct_hinv_flat<A, N, D>, nb, kThreads, 0, s, g, cf, y, vel, p, gsub, out, sc)
 #define MFG_CT_HINV_D(D)                                                                                  \

@@ -21,19 +21,14 @@ namespace mfg {
 // 256-thread blocks per SM that the launch bounds of the strip kernels admit
 constexpr int kCPerSm = 2, kCtPerSm = 3, kUPerSm = 4, kQPerSm = 3;
 
-// Share of the strips' lanes that have a column, at least num/den.
-static bool strips_filled(const Geom& g, int num, int den) {
-  return (long long)(g.ny + 31) / 32 * 32 * num <= (long long)g.ny * den;
-}
-// Which operators run in strips and which point by point (viscosity fields: all point
-// by point).  C^T and H^-1 C^T from 2/3 of the lanes filled on: 512 x ny x 100, C^T in
-// strips against point by point 39.3 / 36.2 us at ny = 20, 39.3 / 40.0 at 22, 74.7 / 77.3
-// at 43, 75.7 / 92.2 at 52; 2000 x 250 in 1-D 11.1 / 12.5.
-bool strips_fit(const Geom& g) { return g.kfy == nullptr && strips_filled(g, 2, 3); }
+// C^T in strips from 2/3 of the lanes filled on: 512 x ny x 100, in strips against point by
+// point 39.3 / 36.2 us at ny = 20, 39.3 / 40.0 at 22, 74.7 / 77.3 at 43, 75.7 / 92.2 at 52;
+// 2000 x 250 in 1-D 11.1 / 12.5.
+static bool ct_strips_fit(const Geom& g) { return strips_filled(g, 2, 3); }
 // C in 2-D from 7/8 on: 512 x ny x 100, 51.4 / 39.6 us at ny = 20, 51.6 / 46.8 at 24, 102.0 / 88.8
 // at 45, 102.5 / 101.3 at 52, 103.1 / 108.8 at 56; 512^2 x 64 489 / 602.  Not in 1-D, where a
 // strip is one row and its borders a load each: 2000 x 250 17.9 / 15.3.
-static bool c_strips_fit(const Geom& g) { return g.actx && g.kfy == nullptr && strips_filled(g, 7, 8); }
+static bool c_strips_fit(const Geom& g) { return g.actx && strips_filled(g, 7, 8); }
 
 struct Nb {
   int im, ip;
@@ -375,7 +370,7 @@ __global__ void __launch_bounds__(kThreads) k_apply_Ct_flat(Geom g, const double
 }
 
 void launch_apply_Ct(const Geom& g, const double* p, double* x, cudaStream_t s) {
-  if (!strips_fit(g)) {
+  if (!ct_strips_fit(g)) {
     const int nb = red_blocks(g.n, g.vec_blocks);
 #define MFG_CT_FLAT(A, N) launch_k(k_apply_Ct_flat<A, N>, nb, kThreads, 0, s, g, p, x)
     if (g.kfy != nullptr) { if (g.actx) MFG_CT_FLAT(1, true); else MFG_CT_FLAT(0, true); }

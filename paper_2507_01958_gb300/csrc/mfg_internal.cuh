@@ -133,7 +133,6 @@ void launch_AAt(const Geom& g, const double* p, double* q, double* scratch, doub
 int aat_kernel_count(int df64);
 int aat_blocks(const Geom& g, int df64);
 int stencil_blocks_max(const Geom& g);
-bool strips_fit(const Geom& g);
 
 // Vector kernels (k_cg.cu).
 // `cap`: grid cap (Geom::vec_blocks).

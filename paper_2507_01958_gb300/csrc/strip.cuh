@@ -22,6 +22,12 @@ __device__ __forceinline__ int ghost(int i, int N, int per) {
 }
 
 
+// Constant viscosity and at least num/den of the strips' lanes with a column: where an
+// operator walks in strips, each by its own measured line; the rest runs point by point.
+inline bool strips_filled(const Geom& g, int num, int den) {
+  return g.kfy == nullptr && (long long)(g.ny + 31) / 32 * 32 * num <= (long long)g.ny * den;
+}
+
 // Launch: 32-column strips x row chunks x planes, one warp each.  A block holds 8
 // warps, fewer where that leaves fewer than 4 blocks per SM.  The chunk length (2 to 32 rows) is
 // the one with the least waves x (rows + 1.5): whole waves of the per_sm blocks a kernel's

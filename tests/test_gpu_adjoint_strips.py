@@ -11,12 +11,12 @@ from _gpu_helpers import dev, host, lib, rel
 
 pytestmark = pytest.mark.gpu
 
-CASES = [  # nx, ny, bc: H^-1 C^T in strips from 2/3 of the lanes on, C from 7/8 (2-D)
-    (5, 21, ("periodic", "neumann")),    # both point by point
-    (9, 45, ("neumann", "periodic")),    # strips / point by point
+CASES = [  # nx, ny, bc: H^-1 C^T and (2-D) C in strips from 7/8 of the lanes on
+    (5, 21, ("periodic", "neumann")),
+    (9, 45, ("neumann", "periodic")),
     (12, 70, ("periodic", "neumann")),
-    (40, 28, ("periodic", "periodic")),  # both in strips, at the line
-    (6, 60, ("neumann", "neumann")),
+    (40, 28, ("periodic", "periodic")),  # at the line
+    (6, 60, ("neumann", "neumann")),     # two strips, the last ragged
     (70, 1, ("neumann", "periodic")),    # 1-D
 ]
 
